@@ -31,8 +31,25 @@ struct PropTables {
     const real *diff;      // [N][Np][5]... stored as [5][N][Np]: coefficient n of g_jk at (k, j)
 };
 
+// Tables of the tensor-core properties pass (props.cu): the Wilke and binary-resistance coefficients
+// as two FP16 terms (hi = fp16(v), lo = fp16(v - hi)) in the shared-memory layout of its B operand,
+// [term 2][chunk of 8 species j][row][8], rows = NR rows of T1, then NP of T0 and of each of the five
+// resistance coefficients, then NR of T2 (row r of a block = species k; NP = N to 8, NR = N to 16).
+struct PropTcTables {
+    const void *B;         // 2 x (K / 8) x rows x 16 bytes; null: coefficients that FP16 pairs cannot hold
+    // [N][8]: c0 .. c4 of log2 r_k (r = sqrt(mu)) as a polynomial in x, its leading term less the
+    // whole n; the reciprocal of the scaling of species k's resistance rows and of X; 2^n; 0
+    const float *species;
+    int rows, NP, NR;
+};
+constexpr int kTcMaxSpecies = 56;         // 2 NR + 6 NP columns fit TMEM and the operands shared memory
+constexpr float kTcXScale = 16384.0f;     // X, X / r, X / r^2 (each at most 1 in magnitude) before rounding
+constexpr float kTcWilkeScale = 1024.0f;  // Wilke tables (at most a few units)
+inline int tc_k(int N) { return N <= 16 ? 16 : (N <= 32 ? 32 : 64); }   // padded contraction length
+
 struct DevMech {
     int N, R, Np, n_tb;
+    PropTcTables tc;
     double P_std, T_mid;
     PropTables<float> f32;
     PropTables<double> f64;

@@ -1,5 +1,7 @@
 // mech.cu -- mechanism loading (host parse, derived tables, one device blob),
 // error reporting and option defaults of the C ABI.
+#include <cuda_fp16.h>
+
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -122,6 +124,61 @@ PropOffsets<real> add_prop_tables(BlobBuilder &bb, int N, int Np, const std::vec
     return o;
 }
 
+// The B operand of the tensor-core properties pass (PropTcTables) from the FP64 coefficients. Row k of
+// the resistance blocks is scaled by a power of two that brings its largest coefficient to 2^14 .. 2^15.
+// Returns false when a value does not fit an FP16 pair (then the pass is not used for the mechanism).
+bool add_tc_tables(BlobBuilder &bb, int N, const std::vector<double> &W, const std::vector<double> &visc,
+                   const std::vector<double> &diff, PropTcTables &t, size_t &off_B, size_t &off_species) {
+    t = PropTcTables{};
+    if (N > kTcMaxSpecies) return false;
+    const int K = tc_k(N);
+    t.NP = (N + 7) & ~7;
+    t.NR = (N + 15) & ~15;
+    t.rows = 2 * t.NR + 6 * t.NP;
+    std::vector<double> v((size_t)t.rows * K, 0.0);
+    std::vector<float> species((size_t)8 * N, 0.0f);
+    auto at = [&](int row, int j) -> double & { return v[(size_t)row * K + j]; };
+    for (int k = 0; k < N; ++k) {
+        double top = 0.0;
+        for (int j = 0; j < N; ++j)
+            for (int n = 0; n < 5; ++n)
+                if (j != k) top = std::fmax(top, std::fabs(diff[((size_t)j * N + k) * 5 + n]));
+        if (!std::isfinite(top)) return false;
+        const int e = top > 0.0 ? 14 - std::ilogb(top) : 0;
+        if (e < -80 || e > 80) return false;
+        if (!(std::fabs(visc[5 * k]) < 100.0)) return false;
+        const double half_log2e = 0.5 / std::log(2.0);            // log2 r = ln mu / (2 ln 2)
+        const int n = (int)std::lround(visc[5 * k] * half_log2e);
+        float *q = species.data() + (size_t)8 * k;
+        q[0] = (float)(visc[5 * k] * half_log2e - n);
+        for (int i = 1; i < 5; ++i) q[i] = (float)(visc[5 * k + i] * half_log2e);
+        q[5] = (float)std::ldexp((double)kTcXScale, e);
+        q[6] = (float)std::ldexp(1.0, n);
+        for (int j = 0; j < N; ++j) {
+            const double c = 1.0 / std::sqrt(8.0 * (1.0 + W[k] / W[j])), w = std::pow(W[j] / W[k], 0.25);
+            at(k, j) = 2.0 * c * w * kTcWilkeScale;                                   // T1
+            at(t.NR + k, j) = c * kTcWilkeScale;                                      // T0
+            at(t.NR + 6 * t.NP + k, j) = c * w * w * kTcWilkeScale;                   // T2
+            for (int n = 0; n < 5; ++n)
+                at(t.NR + (1 + n) * t.NP + k, j) = j == k ? 0.0 : std::ldexp(diff[((size_t)j * N + k) * 5 + n], e);
+        }
+    }
+    std::vector<__half> B((size_t)2 * t.rows * K);
+    for (int r = 0; r < t.rows; ++r)
+        for (int j = 0; j < K; ++j) {
+            const double x = v[(size_t)r * K + j];
+            if (!(std::fabs(x) < 65504.0)) return false;
+            const __half hi = __double2half(x);
+            const __half lo = __double2half(x - (double)__half2float(hi));
+            const size_t q = ((size_t)(j / 8) * t.rows + r) * 8 + j % 8;
+            B[q] = hi;
+            B[(size_t)t.rows * K + q] = lo;
+        }
+    off_B = bb.add(B);
+    off_species = bb.add(species);
+    return true;
+}
+
 template <typename real>
 PropTables<real> resolve(const PropOffsets<real> &o, uint8_t *base) {
     PropTables<real> t;
@@ -206,6 +263,9 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     BlobBuilder bb;
     auto o32 = add_prop_tables<float>(bb, N, Np, W, lo, hi, visc, diff);
     auto o64 = add_prop_tables<double>(bb, N, Np, W, lo, hi, visc, diff);
+    PropTcTables tct;
+    size_t off_tcB = 0, off_tcs = 0;
+    const bool tc_ok = add_tc_tables(bb, N, W, visc, diff, tct, off_tcB, off_tcs);
     std::vector<double> nasa(2 * N * 7);
     for (int k = 0; k < N; ++k)
         for (int i = 0; i < 7; ++i) { nasa[k * 7 + i] = lo[k * 7 + i]; nasa[(N + k) * 7 + i] = hi[k * 7 + i]; }
@@ -300,6 +360,9 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     d.N = N; d.R = R; d.Np = Np; d.n_tb = n_tb; d.P_std = th[0]; d.T_mid = th[2];
     d.f32 = resolve(o32, base);
     d.f64 = resolve(o64, base);
+    d.tc = tct;
+    d.tc.B = tc_ok ? base + off_tcB : nullptr;
+    d.tc.species = tc_ok ? reinterpret_cast<const float *>(base + off_tcs) : nullptr;
     d.W = reinterpret_cast<const double *>(base + off_W);
     d.nasa = reinterpret_cast<const double *>(base + off_nasa);
     d.rtype = reinterpret_cast<const int *>(base + off_rtype);

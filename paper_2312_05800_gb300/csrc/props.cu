@@ -2,7 +2,11 @@
 // transport for every cell (Sec. 2: thermal and transport properties on the
 // GPU; Sec. 3.1: Hirschfelder-Curtiss mixture-averaged model).
 //
-// One thread per cell, persistent grid-stride loop. Cell data are SoA, so a
+// Three kernels: thermo_kernel (cp and h alone), props_tc_kernel (the full pass
+// in FP32, species-pair sums on the tensor cores), and the pair loop below for
+// FP64 and for what the tensor-core pass does not take (more than 56 species).
+//
+// The pair loop: one thread per cell, persistent grid-stride loop. Cell data are SoA, so a
 // warp's loads of T, p and each Y_k row are 128-byte coalesced. The per-pair
 // tables (Wilke weights, binary-resistance fits) are read with uniform
 // addresses (one broadcast per warp) through the read-only cache. The
@@ -14,6 +18,8 @@
 // T0 = c, T1 = 2 c w, T2 = c w^2 (expanded once at load time): one multiply
 // more per pair than three separate sums, for a third fewer registers (which
 // bound the kernel's occupancy).
+#include <cuda_fp16.h>
+
 #include <cmath>
 
 #include "internal.cuh"
@@ -82,8 +88,17 @@ __device__ __forceinline__ real to_real(in_t x) {
     else return real(x);
 }
 
+// Species k is all there is (1 - X_k < 1e-12): D_k is then the mean binary value. FP32 holds an X_k
+// within 3e-8 of 1 as 1, so there the traces' own sum ds (mean resistance gs / (N - 1)) decides, unless
+// 1 - Y_k is lost as well.
+template <typename real>
+__device__ __forceinline__ bool pure_species(real Xk, real y, real ds, real gs, int N) {
+    if (!(real(1) - Xk < real(1e-12))) return false;
+    return sizeof(real) == 8 || y >= real(1) || ds * real(N - 1) <= real(1e-12) * gs;
+}
+
 template <typename real, typename in_t, int NMAX>
-__global__ void __launch_bounds__(128, sizeof(real) == 4 && NMAX <= 32 ? 4 : 1) props_kernel(int N, int Np, real T_mid, PropTables<real> tb, int64_t ncells,
+__global__ void __launch_bounds__(128) props_kernel(int N, int Np, real T_mid, PropTables<real> tb, int64_t ncells,
                                                     int64_t ld, const in_t *__restrict__ Tg,
                                                     const in_t *__restrict__ pg, const in_t *__restrict__ Yg,
                                                     real *__restrict__ cpg, real *__restrict__ hg,
@@ -266,7 +281,7 @@ __global__ void __launch_bounds__(128, sizeof(real) == 4 && NMAX <= 32 ? 4 : 1) 
             lam = fma(Xk, lamk / den, lam);
             if (Dkg) {
                 real D;
-                if (real(1) - Xk < real(1e-12)) D = T15 / (p * gs / real(N - 1));   // pure species k
+                if (pure_species(Xk, y, ds, gs, N)) D = T15 / (p * gs / real(N - 1));
                 else D = (real(1) - y) * T15 / (p * ds);
                 Dkg[(int64_t)k * ld + i] = D;
             }
@@ -462,6 +477,514 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
     return check_cuda(cudaGetLastError(), "props_eval (thermo) launch");
 }
 
+// ---- the full pass in FP32, with the species-pair sums on the tensor cores ------------------
+//
+// Per cell and species k the transport needs sum_j X_j Phi_kj and sum_j X_j g_kj. With
+// Phi_kj = T0_kj + t (T1_kj + t T2_kj), t = r_k / r_j, and g_kj = sum_n d_n,kj x^n these are
+//   T0 X + r_k (T1 (X / r) + r_k T2 (X / r^2))      and      sum_n x^n (D_n X):
+// eight products of constant N x N tables with three per-cell vectors, a contraction. A tile of
+// 128 cells is the M of tcgen05.mma (kind::f16), the tables' rows are its N (2 NR + 6 NP columns of
+// TMEM: 256 for 30 species, 464 for 53) and the species j its K.
+//
+// Precision: both factors are pairs of FP16 terms, hi = fp16(v) and lo = fp16(v - hi), 22 bits, and
+// three products hi hi + lo hi + hi lo are accumulated in FP32. To stay clear of FP16's small range
+// 1/r is divided by the power of two at the cell's largest 1/r (r_k is multiplied by it), every
+// vector entry is then at most 1 in magnitude and scaled by 2^14, and the tables' rows by powers of
+// two (PropTcTables). What is left of absolute error, 2^-39 of a mole fraction, only shows in D_k of
+// a species that is nearly alone (its sum runs over traces): for X_k > 0.999 that sum is taken in FP32
+// from the FP32 tables (near_pure_D). The tensor core cuts its accumulator instead of rounding it,
+// which takes a mean share of a sum that grows with the instructions of full size (K / 16): measured
+// 0.5e-7, 2.8e-7 and 5.7e-7 for 1, 2 and 4, and given back (`cut`). r_k = 2^(polynomial) is formed with
+// the whole part of its exponent taken out at load time. Relative errors against 64 bits (2-norm, 100,003
+// cells, FP32 state; the former pair loop -> this kernel): 30 species mu 3.6e-7 -> 1.2e-7, lambda 3.2e-7 ->
+// 1.1e-7, D 2.0e-7 -> 1.6e-7; 53 species 3.2e-7 -> 1.4e-7, 3.1e-7 -> 1.3e-7, 2.4e-7 -> 1.8e-7; 9 species
+// 2.4e-7 -> 0.9e-7, 2.7e-7 -> 1.0e-7, 1.1e-7 -> 1.1e-7.
+//
+// What bounds it: instruction issue (51 % of the slots) and its latencies for the per-species FP32
+// work that is left; the tensor cores are busy a few per cent of the time, HBM 10 %. The pair loop (10
+// instructions a pair, tables from shared memory) took 1,580 us on 2,097,152 cells of 30 species from
+// FP64 state and 799 us on 300,001 of 53 from FP32; this kernel takes 625 and 192 us.
+//
+// Layout: a thread per cell and chunk of eight species (2, 4 or 8 threads a cell for up to 16, 32 or
+// 56 species: 256 to 1,024 threads, 64 registers; two threads a cell with twice the species each
+// and 128 registers left half the warps and took 792 us). Each thread turns its species into operand
+// entries (no-swizzle K-major core matrices, [chunk][row][16 bytes]: a warp's 16-byte stores are
+// consecutive) and later finishes the same species from TMEM. cp and h are summed over all species in
+// ascending order by one thread each while the tensor cores work, with thermo_kernel's operations, so
+// they are bitwise its results.
+struct TcArgs {
+    int N;
+    float T_mid;
+    PropTables<float> tb;
+    PropTcTables tc;
+    int64_t ncells, ld;
+    float *cp, *h, *mu, *lam, *Dk;
+    unsigned int *err;
+    uint32_t spin;
+};
+
+template <int NMAX>
+struct TcLayout {
+    static constexpr int kChunks = NMAX / 8;                    // chunks of 8 species
+    static constexpr int kTPR = kChunks;                        // threads per cell, a chunk each
+    static constexpr int kThreads = 128 * kTPR;
+    static constexpr int kCtas = NMAX <= 16 ? 4 : (NMAX <= 32 ? 2 : 1);   // resident per SM
+    static constexpr bool kStageY = NMAX <= 32;                 // mass fractions in FP32 kept in shared memory
+    static constexpr uint32_t kABytes = 6 * kChunks * 2048;     // 3 vectors x 2 terms x [chunk][128][16 B]
+    static constexpr uint32_t kYBytes = kStageY ? NMAX * 128 * 4 : 0;
+    static constexpr int kPad = NMAX < kTcMaxSpecies ? NMAX : kTcMaxSpecies;   // species of the padded tables
+    static constexpr int kRedRows = NMAX <= 32 ? 4 : 2;         // sums between a cell's threads (two pairs, or one reused)
+    static constexpr int kShares = kPad / 8;                    // threads of a cell that hold species
+    static constexpr uint32_t kRed = kRedRows * kShares * 128 * 4;
+    static constexpr bool kEuk = NMAX <= 32;                    // conductivity rows of their own
+    static constexpr uint32_t kTab = (kPad * (6 + 2 + (kEuk ? 4 : 0)) + 2) * 16;   // species tables (float4 each)
+    static size_t bytes(int rows) { return (size_t)kABytes + 2 * kChunks * rows * 16 + kYBytes + kTab + kRed + 32; }
+};
+
+// 2 columns of each of 8 TMEM addresses, 32 lanes; one wait. v[2 a + u] = column u of address a.
+__device__ __forceinline__ void tmem_ld8x2(const uint32_t (&a)[8], float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%2, %3}, [%17];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4, %5}, [%18];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%6, %7}, [%19];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8, %9}, [%20];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%10, %11}, [%21];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%12, %13}, [%22];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%14, %15}, [%23];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7])
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// D_k of a species that is nearly alone (X_k > 0.999), the sums over the traces in FP32
+template <typename in_t>
+__device__ __noinline__ float near_pure_D(const PropTables<float> &tb, int N, int Np, int k, int64_t ld, int64_t i,
+                                          const in_t *__restrict__ Yg, float Wbar, float x, float y, float Xk,
+                                          float T15, float p) {
+    float ds = 0.0f, gs = 0.0f;
+    for (int j = 0; j < N; ++j) {
+        const float Xj = to_real<float>(Yg[(int64_t)j * ld + i]) * __ldg(tb.invW + j) * Wbar;
+        float g = 0.0f;
+        for (int n = 4; n >= 0; --n) g = fmaf(g, x, __ldg(tb.diff + ((size_t)n * N + k) * Np + j));
+        ds = fmaf(g, Xj, ds);
+        gs += g;
+    }
+    if (pure_species(Xk, y, ds, gs, N)) return T15 / (p * gs / float(N - 1));
+    return (1.0f - y) * T15 / (p * ds);
+}
+
+__device__ __forceinline__ float ex2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// eight values as FP16 pairs: the hi and lo terms, 16 bytes each
+__device__ __forceinline__ void split8(const float (&v)[8], uint4 &hi, uint4 &lo) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const __half2 a = __floats2half2_rn(v[2 * u], v[2 * u + 1]);
+        const float2 f = __half22float2(a);
+        const __half2 b = __floats2half2_rn(v[2 * u] - f.x, v[2 * u + 1] - f.y);
+        h[u] = *reinterpret_cast<const uint32_t *>(&a);
+        l[u] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Descriptor of a no-swizzle K-major operand: core matrices of 8 rows x 16 bytes, consecutive
+// along the rows (128 bytes apart), `lbo` bytes from one 16-byte chunk of K to the next.
+__device__ __forceinline__ uint64_t sdesc_kmajor_plain(uint32_t saddr, uint32_t lbo) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128u >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+template <typename in_t, int NMAX>
+__global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCtas)
+    props_tc_kernel(TcArgs g, const in_t *__restrict__ Tg, const in_t *__restrict__ pg, const in_t *__restrict__ Yg) {
+    using L = TcLayout<NMAX>;
+    constexpr int TPR = L::kTPR, SH = L::kShares;
+    extern __shared__ __align__(128) uint8_t tc_smem[];
+    const int N = g.N, rows = g.tc.rows, NP = g.tc.NP, NR = g.tc.NR;
+    uint8_t *sA = tc_smem;
+    uint8_t *sB = sA + L::kABytes;
+    const uint32_t b_lbo = (uint32_t)rows * 16, b_term = L::kChunks * b_lbo;
+    float *sY = reinterpret_cast<float *>(sB + 2 * b_term);            // [NMAX][128] (kStageY)
+    // per species, padded to PAD: thermo_kernel's NASA rows of both ranges (3 float4 each), log2 r
+    // (2 float4: c0 .. c3 | c4, 1/W, 1/dscale, 2^n), R (cp/R + 5/4) / W of both ranges (2 float4 each)
+    float4 *tab = reinterpret_cast<float4 *>(reinterpret_cast<uint8_t *>(sY) + L::kYBytes);
+    constexpr int PAD = L::kPad;
+    constexpr int TAB2 = 3 * PAD + 1, EUK2 = 2 * PAD + 1;              // the high range, in other banks than the low
+    float4 *vis = tab + 2 * TAB2 - 1;
+    float4 *euk = vis + 2 * PAD;
+    float *red = reinterpret_cast<float *>(euk + (L::kEuk ? 4 * PAD + 1 : 1));   // [kRedRows][SH][128]
+    constexpr int RED2 = (L::kRedRows - 2) * SH;                       // first row of mu and lambda
+    uint64_t *bars = reinterpret_cast<uint64_t *>(red + L::kRedRows * SH * 128);
+    uint64_t *bar_b = bars, *bar_m = bars + 1;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2);
+    const int warp = threadIdx.x >> 5;
+    const int grp = warp >> 2;                                         // which share of the species
+    const int row = threadIdx.x & 127;                                 // cell of the tile = TMEM lane
+    const uint32_t ncols = rows <= 128 ? 128u : (rows <= 256 ? 256u : 512u);
+
+    if (threadIdx.x == 0) {
+        tc::mbar_init(bar_b, 1);
+        tc::mbar_init(bar_m, 1);
+        tc::fence_barrier_init();
+        tc::mbar_arrive_expect_tx(bar_b, 2 * b_term);
+        for (uint32_t o = 0; o < 2 * b_term; o += 16384) {
+            const uint32_t n = 2 * b_term - o < 16384 ? 2 * b_term - o : 16384;
+            tc::bulk_load_1d(sB + o, static_cast<const uint8_t *>(g.tc.B) + o, n, bar_b);
+        }
+    }
+    if (warp == 0) {
+        tc::tmem_alloc(tmem_slot, ncols);
+        tc::tmem_relinquish();
+    }
+    const float R = float(kR);
+    // the mean share that the cuts of the hi hi instructions take off a sum (measured, below)
+    const int ks16 = (N + 15) / 16;
+    const float cut = ks16 == 1 ? 4e-8f : (ks16 == 2 ? 2.7e-7f : (ks16 == 3 ? 4.2e-7f : 5.6e-7f));
+    for (int e = threadIdx.x; e < 2 * PAD; e += blockDim.x) {
+        const int rg = e / PAD, k = e % PAD;
+        float a[5] = {0, 0, 0, 0, 0}, b[6] = {0, 0, 0, 0, 0, 0}, iw = 0.0f;
+        if (k < N) {
+            for (int q = 0; q < 5; ++q) a[q] = g.tb.nasa_cp[(rg * N + k) * 5 + q];
+            for (int q = 0; q < 6; ++q) b[q] = g.tb.nasa_h[(rg * N + k) * 6 + q];
+            iw = g.tb.invW[k];
+        }
+        float4 *o = tab + rg * TAB2 + 3 * k;
+        o[0] = make_float4(a[0], a[1], a[2], a[3]);
+        o[1] = make_float4(a[4], b[0], b[1], b[2]);
+        o[2] = make_float4(b[3], b[4], b[5], iw);
+        if (L::kEuk) {
+            const float f = R * iw;
+            euk[rg * EUK2 + 2 * k] = make_float4((a[0] + 1.25f) * f, a[1] * f, a[2] * f, a[3] * f);
+            euk[rg * EUK2 + 2 * k + 1] = make_float4(a[4] * f, 0.0f, 0.0f, 0.0f);
+        }
+    }
+    for (int k = threadIdx.x; k < PAD; k += blockDim.x) {
+        const float *q = g.tc.species + 8 * k;
+        vis[2 * k] = k < N ? make_float4(q[0], q[1], q[2], q[3]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        vis[2 * k + 1] = k < N ? make_float4(q[4], g.tb.invW[k], q[5], q[6]) : make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const int64_t ntiles = (g.ncells + 127) / 128;
+    uint32_t phase = 0;
+    bool b_ready = false;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, phase ^= 1u) {
+        const int64_t cell = tile * 128 + row;
+        const bool valid = cell < g.ncells;
+        const int64_t i = valid ? cell : g.ncells - 1;
+        const in_t *Yi = Yg + i;
+        const float T = to_real<float>(Tg[i]);
+        const float p = to_real<float>(pg[i]);
+        // own species: mass fraction, r = sqrt(mu), and their share of 1 / Wbar and of the smallest r
+        const int k0 = grp * 8;
+        float y[8], rk[8];
+        {
+            const in_t *q = Yi + (int64_t)k0 * g.ld;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = k0 + u < N ? to_real<float>(q[u * g.ld]) : 0.0f;
+        }
+        const float x = logf(T * 1e-3f);                               // ln(T / 1000)
+        float S = 0.0f, rmin = 3.0e38f;
+        if (PAD == NMAX || k0 < PAD) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float4 v0 = vis[2 * (k0 + u)], v1 = vis[2 * (k0 + u) + 1];
+                float lr = v1.x;
+                lr = fmaf(lr, x, v0.w);
+                lr = fmaf(lr, x, v0.z);
+                lr = fmaf(lr, x, v0.y);
+                lr = fmaf(lr, x, v0.x);
+                rk[u] = ex2_approx(lr) * v1.w;
+                S = fmaf(y[u], v1.y, S);
+                rmin = fminf(rmin, rk[u]);
+                if (L::kStageY) sY[(k0 + u) * 128 + row] = y[u];
+            }
+        } else {                                                       // a chunk of zeros (warp-uniform)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) rk[u] = 1.0f;
+        }
+        if (SH == TPR || grp < SH) {
+            red[grp * 128 + row] = S;
+            red[(SH + grp) * 128 + row] = rmin;
+        }
+        // the next tile's rows on their way to L2
+        if (const int64_t next = tile + gridDim.x; threadIdx.x >= 32 && threadIdx.x < 64 && (next + 1) * 128 <= g.ncells)
+            for (int q = threadIdx.x - 32; q < N + 2; q += 32) {
+                const in_t *src = (q == 0 ? Tg : q == 1 ? pg : Yg + (int64_t)(q - 2) * g.ld) + next * 128;
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(128 * sizeof(in_t)))
+                             : "memory");
+            }
+        __syncthreads();
+        S = 0.0f;
+        rmin = 3.0e38f;
+#pragma unroll
+        for (int q = 0; q < SH; ++q) {
+            S += red[q * 128 + row];
+            rmin = fminf(rmin, red[(SH + q) * 128 + row]);
+        }
+        const float Wbar = 1.0f / S;
+        // r is scaled by a power of two that brings the smallest one to 1 .. 2, and 1/r by its reciprocal
+        int e = 127 - (int)(__float_as_uint(rmin) >> 23);
+        e = e < -100 ? -100 : (e > 100 ? 100 : e);
+        const float up = __int_as_float((127 + e) << 23), down = __int_as_float((127 - e) << 23);
+        const float xs = Wbar * kTcXScale;
+        {
+            float v[8], ir[8];
+            uint8_t *dst = sA + grp * 2048 + row * 16;
+            uint4 hi, lo;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                ir[u] = rcp_approx(rk[u]) * down;
+                v[u] = PAD < NMAX && k0 >= PAD ? 0.0f : y[u] * vis[2 * (k0 + u) + 1].y * xs;
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {                              // X, X / r, X / r^2
+                split8(v, hi, lo);
+                *reinterpret_cast<uint4 *>(dst + (2 * q) * L::kChunks * 2048) = hi;
+                *reinterpret_cast<uint4 *>(dst + (2 * q + 1) * L::kChunks * 2048) = lo;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] *= ir[u];
+            }
+        }
+        tc::fence_proxy_async_smem();
+        tc::tc_fence_before();
+        __syncthreads();
+        bool ok = true;
+        if (threadIdx.x == 0) {
+            if (!b_ready) {
+                ok = tc::mbar_wait(bar_b, 0, g.spin);
+                b_ready = ok;
+            }
+            if (ok) {
+                tc::tc_fence_after();
+                // the three column groups: vector 1 on T1, vector 0 on T0 and the resistances (two parts
+                // where it is wider than one instruction), vector 2 on T2
+                const int nx = 6 * NP, ksteps = (N + 15) / 16;
+                const int part_v[4] = {1, 0, 0, 2};
+                const int part_r[4] = {0, NR, NR + (nx < 256 ? nx : 256), NR + nx};
+                const int part_n[4] = {NR, nx < 256 ? nx : 256, nx < 256 ? 0 : nx - 256, NR};
+                const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
+                for (int q = 0; q < 4; ++q) {
+                    if (part_n[q] == 0) continue;
+                    const uint32_t idesc = tc::idesc_e4m3_f32(128, part_n[q]);   // format code 0 is F16 for kind::f16
+                    uint32_t acc = 0;
+                    // hi lo, lo hi, hi hi: the accumulator is cut, not rounded, after every instruction, so
+                    // the small products come first and only the last K / 16 cuts are of full size
+                    for (int t = 0; t < 3; ++t) {
+                        const uint32_t at = a0 + (uint32_t)(2 * part_v[q] + (t == 1)) * (L::kChunks * 2048);
+                        const uint32_t bt = b0 + (t == 0 ? b_term : 0u) + (uint32_t)part_r[q] * 16;
+                        for (int ks = 0; ks < ksteps; ++ks) {
+                            tc::umma_f16(tmem + part_r[q], sdesc_kmajor_plain(at + ks * 4096, 2048),
+                                         sdesc_kmajor_plain(bt + ks * 2 * b_lbo, b_lbo), idesc, acc);
+                            acc = 1;
+                        }
+                    }
+                }
+                tc::umma_commit(bar_m);
+            }
+        }
+        __syncwarp();
+        const int hot = (T >= g.T_mid) ? 1 : 0;
+        // beside the products: cp and h over all species, ascending, one thread each (of the last chunks,
+        // which have the fewest species)
+        if (grp >= TPR - 2) {
+            const float4 *tr = tab + hot * TAB2;
+            auto mass = [&](int k) {
+                if constexpr (L::kStageY) return sY[k * 128 + row];
+                else return to_real<float>(Yi[(int64_t)k * g.ld]);
+            };
+            if (grp == TPR - 1 && g.cp) {
+                float cpm = 0.0f;
+#pragma unroll 4
+                for (int k = 0; k < N; ++k) {
+                    const float yk = mass(k);
+                    const float4 q0 = tr[3 * k];
+                    float cpR = tr[3 * k + 1].x;
+                    cpR = fmaf(cpR, T, q0.w);
+                    cpR = fmaf(cpR, T, q0.z);
+                    cpR = fmaf(cpR, T, q0.y);
+                    cpR = fmaf(cpR, T, q0.x);
+                    const float yw = yk * tr[3 * k + 2].w;
+                    cpm = fmaf(yw, cpR, cpm);
+                }
+                if (valid) g.cp[i] = cpm * R;
+            }
+            if (grp == TPR - 2 && g.h) {
+                const float iT = 1.0f / T;
+                float hm = 0.0f;
+#pragma unroll 4
+                for (int k = 0; k < N; ++k) {
+                    const float yk = mass(k);
+                    const float4 q1 = tr[3 * k + 1], q2 = tr[3 * k + 2];
+                    float hR = q2.y;
+                    hR = fmaf(hR, T, q2.x);
+                    hR = fmaf(hR, T, q1.w);
+                    hR = fmaf(hR, T, q1.z);
+                    hR = fmaf(hR, T, q1.y);
+                    hR = fmaf(q2.z, iT, hR);
+                    const float yw = yk * q2.w;
+                    hm = fmaf(yw, hR, hm);
+                }
+                if (valid) g.h[i] = hm * R * T;
+            }
+        }
+        ok = ok && tc::mbar_wait(bar_m, phase, g.spin);
+        tc::tc_fence_after();
+        const float T15 = T * sqrtf(T), T15p = T15 / p;
+        constexpr int ES = L::kEuk ? 2 : 3;
+        const float4 *er = L::kEuk ? euk + hot * EUK2 : tab + hot * TAB2;
+        const float pure = 0.999f * S;
+        float mu = 0.0f, lam = 0.0f;
+        bool alone = false;
+        float *Dp = g.Dk + (int64_t)k0 * g.ld + i;
+#pragma unroll
+        for (int u0 = 0; u0 < 8; u0 += 2) {
+            if (k0 + u0 >= N) break;                                   // warp-uniform
+            float v[16];
+            uint32_t ad[8];
+            ad[0] = tlane + k0 + u0;                                   // T1
+#pragma unroll
+            for (int q = 0; q < 6; ++q) ad[1 + q] = tlane + NR + q * NP + k0 + u0;   // T0, resistances
+            ad[7] = tlane + NR + 6 * NP + k0 + u0;                     // T2
+            __syncwarp();                                              // converged for the TMEM loads
+            tmem_ld8x2(ad, v);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int k = k0 + u0 + u;
+                const float yk = y[u0 + u], r = rk[u0 + u], rn = r * up;
+                const float4 e0 = er[ES * k], v1 = vis[2 * k + 1];
+                float lk = er[ES * k + 1].x;                           // lambda_k / mu_k (Eucken)
+                lk = fmaf(lk, T, e0.w);
+                lk = fmaf(lk, T, e0.z);
+                lk = fmaf(lk, T, e0.y);
+                lk = fmaf(lk, T, e0.x);
+                if (!L::kEuk) lk = (lk + 1.25f) * (R * v1.y);
+                const float yw = yk * v1.y;
+                const float den = fmaf(rn, fmaf(rn, v[14 + u], v[u]), v[2 + u]);
+                const float wk = (r * r) * (yw * rcp_approx(den));     // X_k mu_k / sum, up to a factor of the cell
+                if (k < N) {                                           // (columns past N hold zeros: 0 / 0)
+                    mu += wk;
+                    lam = fmaf(wk, lk, lam);
+                }
+                if (g.Dk) {
+                    float ds = v[12 + u];
+                    ds = fmaf(ds, x, v[10 + u]);
+                    ds = fmaf(ds, x, v[8 + u]);
+                    ds = fmaf(ds, x, v[6 + u]);
+                    ds = fmaf(ds, x, v[4 + u]);
+                    float ri = rcp_approx(ds);
+                    ri = fmaf(ri, fmaf(-ds, ri, 1.0f) - cut, ri);
+                    alone |= yw > pure;
+                    if (valid && ok && k < N) *Dp = (1.0f - yk) * T15p * (ri * v1.z);
+                    Dp += g.ld;
+                }
+            }
+        }
+        if (g.Dk && alone && valid && ok) {                            // rare: redone in FP32
+            for (int k = k0; k < k0 + 8 && k < N; ++k) {
+                const float yk = to_real<float>(Yi[(int64_t)k * g.ld]);
+                const float yw = yk * vis[2 * k + 1].y;
+                if (yw > pure)
+                    g.Dk[(int64_t)k * g.ld + i] = near_pure_D(g.tb, N, (N + 3) & ~3, k, g.ld, i, Yg, Wbar, x, yk,
+                                                              yw * Wbar, T15, p);
+            }
+        }
+        const float unit = Wbar * (kTcXScale * kTcWilkeScale) * (1.0f - cut);
+        if (SH == TPR || grp < SH) {
+            red[(RED2 + grp) * 128 + row] = mu * unit;
+            red[(RED2 + SH + grp) * 128 + row] = lam * unit;
+        }
+        tc::tc_fence_before();                                         // TMEM reads before the next tile's products
+        const bool all_ok = __syncthreads_and(ok);
+        if (grp == 0) {
+            mu = 0.0f;
+            lam = 0.0f;
+#pragma unroll
+            for (int q = 0; q < SH; ++q) {
+                mu += red[(RED2 + q) * 128 + row];
+                lam += red[(RED2 + SH + q) * 128 + row];
+            }
+            if (!all_ok) mu = lam = __int_as_float(0x7fc00000);
+            if (valid && g.mu) g.mu[i] = mu;
+            if (valid && g.lam) g.lam[i] = lam;
+        }
+        if (!all_ok) {
+            // a wait ran out: NaN for the tile, and the CTA ends once what it issued has finished
+            if (g.Dk && valid)
+                for (int k = grp; k < N; k += TPR) g.Dk[(int64_t)k * g.ld + i] = __int_as_float(0x7fc00000);
+            if (threadIdx.x == 0) atomicExch(g.err, 1u);
+            break;
+        }
+        if (RED2 == 0) __syncthreads();                                // the sums' rows are written again
+    }
+    if (threadIdx.x == 0) {
+        // nothing in flight when the CTA ends (full limit): the table copy, then the products
+        if (!b_ready && !tc::mbar_wait(bar_b, 0)) atomicExch(g.err, 1u);
+        uint64_t *bar_d = bars + 3;
+        tc::mbar_init(bar_d, 1);
+        tc::fence_barrier_init();
+        tc::umma_commit(bar_d);
+        if (!tc::mbar_wait(bar_d, 0)) atomicExch(g.err, 1u);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem, ncols);
+    }
+}
+
+template <typename in_t, int NMAX>
+int launch_props_tc(const chem_mech *m, int64_t ncells, int64_t ld, const void *T, const void *p, const void *Y,
+                    void *cp, void *h, void *mu, void *lam, void *Dk, cudaStream_t st) {
+    using L = TcLayout<NMAX>;
+    const size_t smem = L::bytes(m->dev.tc.rows);
+    static bool configured = false;
+    if (!configured) {
+        int rc = check_cuda(cudaFuncSetAttribute(props_tc_kernel<in_t, NMAX>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 NMAX <= 32 ? 113 * 1024 : 227 * 1024),
+                            "props_eval smem attribute");
+        if (rc) return rc;
+        configured = true;
+    }
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t ntiles = (ncells + 127) / 128;
+    const int64_t most = (int64_t)sms * L::kCtas;                      // the resident CTAs
+    const TcArgs a{m->N, float(m->T_mid), m->dev.f32, m->dev.tc, ncells, ld, static_cast<float *>(cp),
+                   static_cast<float *>(h), static_cast<float *>(mu), static_cast<float *>(lam),
+                   static_cast<float *>(Dk), m->dev.counters + kPropsErrCounter, tc::kSpinLimit};
+    void *pb = prof_begin(st);
+    props_tc_kernel<in_t, NMAX><<<(unsigned)(ntiles < most ? ntiles : most), L::kThreads, smem, st>>>(
+        a, static_cast<const in_t *>(T), static_cast<const in_t *>(p), static_cast<const in_t *>(Y));
+    prof_end(pb, st, "props_kernel<f32>", (double)ncells * (16.0 * m->N * m->N + 30.0 * m->N),
+             (double)ncells * ((m->N + 2) * sizeof(in_t) + (4 + m->N) * sizeof(float)));
+    return check_cuda(cudaGetLastError(), "props_eval launch");
+}
+
 template <typename real, typename in_t, int NMAX>
 int launch_props(const chem_mech *m, int64_t ncells, int64_t ld, const void *T, const void *p, const void *Y,
                  void *cp, void *h, void *mu, void *lam, void *Dk, cudaStream_t st) {
@@ -502,9 +1025,17 @@ int dispatch_props(const chem_mech *m, int64_t ncells, int64_t ld, const void *T
                    void *cp, void *h, void *mu, void *lam, void *Dk, cudaStream_t st) {
     if constexpr (sizeof(real) == 4) {
         if (!mu && !lam && !Dk) return launch_thermo<in_t>(m, ncells, ld, T, Y, cp, h, st);
+        // the tensor-core pass wherever its operands fit (up to 56 species with coefficients that FP16
+        // pairs hold); the pair loop for the rest
+        if (m->dev.tc.B) {
+            if (m->N <= 16) return launch_props_tc<in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+            if (m->N <= 32) return launch_props_tc<in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+            return launch_props_tc<in_t, 64>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+        }
+    } else {
+        if (m->N <= 16) return launch_props<real, in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+        if (m->N <= 32) return launch_props<real, in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
     }
-    if (m->N <= 16) return launch_props<real, in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
-    if (m->N <= 32) return launch_props<real, in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
     return launch_props<real, in_t, 64>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
 }
 
