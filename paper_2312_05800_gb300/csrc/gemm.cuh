@@ -17,6 +17,8 @@
 //               chunks between them; tcgen05.ld, then the functor. BF16 or
 //               E4M3 GELU outputs are staged per warp in shared memory (double
 //               buffered) and written by TMA tensor stores.
+// B may also be stored [K][N] (the layer's own weights for the backward product dZ W): its k-blocks are
+// then boxes of 64 columns x 64 rows and the instruction takes it N-major.
 // Ragged M, N and K: TMA fills out-of-range operand elements with zeros, TMA
 // stores clip at the tensor bounds, and direct stores mask rows >= M and
 // columns >= N.
@@ -148,10 +150,13 @@ __device__ __forceinline__ float gelu_grad(float z) {
 }
 
 // ---- epilogue functors: (row, first column, 16 accumulator values) --------
+// kBNMajor: the B operand is [K][N] row-major (see above); BN is then a multiple of 64.
 
-// Y = bf16(GELU(acc + b)); optionally also the FP32 pre-activation acc + b.
-// Without a pre-activation the kernel stages the BF16 chunk and stores it by TMA.
+// Y = bf16(GELU(acc + b)); optionally also the FP32 pre-activation acc + b (stored straight from
+// the lanes, 64 bytes of a row each, where its rows are 16-byte aligned). The kernel stages the BF16
+// chunk and stores it by TMA.
 struct EpiGelu {
+    static constexpr bool kBNMajor = false;
     static constexpr bool kF8 = false;       // operand type: BF16
     static constexpr int kOutBytes = 32;     // bytes of a 16-column output chunk row (TMA store)
     int M, N;
@@ -172,18 +177,26 @@ struct EpiGelu {
     // when rows end on whole 16-column chunks (N % 16 == 0) with a 16-byte
     // aligned bias (read as float4)
     __host__ __device__ __forceinline__ bool tma_store() const {
-        return pre == nullptr && (N & 15) == 0 && bias != nullptr && (reinterpret_cast<uintptr_t>(bias) & 15) == 0;
+        return (pre == nullptr || ((ldp & 3) == 0 && (g_pre & 3) == 0 && (reinterpret_cast<uintptr_t>(pre) & 15) == 0)) &&
+               (N & 15) == 0 && bias != nullptr && (reinterpret_cast<uintptr_t>(bias) & 15) == 0;
     }
     const void *tma_ptr() const { return tma_store() ? out : nullptr; }
     // the 16 BF16 values of (row, col0..col0+15), two per 32-bit word (N % 8 == 0 on this path,
     // and the bias is padded to whole 16-float groups)
-    __device__ __forceinline__ void compute(int col0, const float (&v)[16], uint32_t (&w)[8]) const {
+    __device__ __forceinline__ void compute(int row, int col0, const float (&v)[16], uint32_t (&w)[8]) const {
         float b[16];
         const float4 *bp = reinterpret_cast<const float4 *>(bias + col0);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float4 q = __ldg(bp + i);
             b[4 * i] = q.x; b[4 * i + 1] = q.y; b[4 * i + 2] = q.z; b[4 * i + 3] = q.w;
+        }
+        if (pre && row < M) {
+            float4 *q = reinterpret_cast<float4 *>(pre + (int64_t)row * ldp + col0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                q[i] = make_float4(v[4 * i] + b[4 * i], v[4 * i + 1] + b[4 * i + 1], v[4 * i + 2] + b[4 * i + 2],
+                                   v[4 * i + 3] + b[4 * i + 3]);
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -227,6 +240,7 @@ struct EpiGelu {
 
 // Y = acc + b in FP32 (b may be null).
 struct EpiLinear {
+    static constexpr bool kBNMajor = false;
     static constexpr bool kF8 = false;
     static constexpr int kOutBytes = 32;
     int M, N;
@@ -242,7 +256,7 @@ struct EpiLinear {
     }
     __host__ __device__ __forceinline__ bool tma_store() const { return false; }
     const void *tma_ptr() const { return nullptr; }
-    __device__ __forceinline__ void compute(int, const float (&)[16], uint32_t (&)[8]) const {}
+    __device__ __forceinline__ void compute(int, int, const float (&)[16], uint32_t (&)[8]) const {}
     __device__ __forceinline__ void operator()(int row, int col0, const float (&v)[16]) const {
         if (row >= M) return;
         float *o = out + (int64_t)row * ldo + col0;
@@ -264,8 +278,11 @@ struct EpiLinear {
     }
 };
 
-// Y = bf16(acc * GELU'(Z)), Z the FP32 pre-activation of the layer below (backward pass).
+// Y = bf16(acc * GELU'(Z)), Z the FP32 pre-activation of the layer below (backward pass). With aligned
+// rows Z is read 16 bytes at a time and Y stored by TMA: the product of 4096 x 1600 x 800 took 138 us
+// with element loads and stores (32 rows' sectors per instruction) and GRADUS that way.
 struct EpiGeluGrad {
+    static constexpr bool kBNMajor = true;
     static constexpr bool kF8 = false;
     static constexpr int kOutBytes = 32;
     int M, N;
@@ -280,9 +297,23 @@ struct EpiGeluGrad {
         e.out += g * g_out;
         return e;
     }
-    __host__ __device__ __forceinline__ bool tma_store() const { return false; }
-    const void *tma_ptr() const { return nullptr; }
-    __device__ __forceinline__ void compute(int, const float (&)[16], uint32_t (&)[8]) const {}
+    __host__ __device__ __forceinline__ bool tma_store() const {
+        return (N & 15) == 0 && (ldz & 3) == 0 && (g_z & 3) == 0 && (reinterpret_cast<uintptr_t>(z) & 15) == 0;
+    }
+    const void *tma_ptr() const { return tma_store() ? out : nullptr; }
+    __device__ __forceinline__ void compute(int row, int col0, const float (&v)[16], uint32_t (&w)[8]) const {
+        const float4 *zr = reinterpret_cast<const float4 *>(z + (int64_t)(row < M ? row : M - 1) * ldz + col0);
+        float4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = __ldg(zr + i);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            __nv_bfloat162 a = __floats2bfloat162_rn(v[4 * i] * gelu_grad(q[i].x), v[4 * i + 1] * gelu_grad(q[i].y));
+            __nv_bfloat162 b = __floats2bfloat162_rn(v[4 * i + 2] * gelu_grad(q[i].z), v[4 * i + 3] * gelu_grad(q[i].w));
+            w[2 * i] = *reinterpret_cast<uint32_t *>(&a);
+            w[2 * i + 1] = *reinterpret_cast<uint32_t *>(&b);
+        }
+    }
     __device__ __forceinline__ void operator()(int row, int col0, const float (&v)[16]) const {
         if (row >= M) return;
         const float *zr = z + (int64_t)row * ldz + col0;
@@ -299,6 +330,7 @@ struct EpiGeluGrad {
 // with round-to-nearest-even and saturation at +-448 (F8OUT) or as BF16(h).
 template <bool F8IN, bool F8OUT>
 struct EpiGeluQ {
+    static constexpr bool kBNMajor = false;
     static constexpr bool kF8 = F8IN;
     static constexpr int kOutBytes = F8OUT ? 16 : 32;
     int M, N;
@@ -316,7 +348,7 @@ struct EpiGeluQ {
     __device__ __forceinline__ float act(float v, float c, float b) const {
         return gelu_exact(F8IN ? fmaf(v, c, b) : v + b);
     }
-    __device__ __forceinline__ void compute(int col0, const float (&v)[16], uint32_t (&w)[8]) const {
+    __device__ __forceinline__ void compute(int, int col0, const float (&v)[16], uint32_t (&w)[8]) const {
         float b[16], c[16];
         const float4 *bp = reinterpret_cast<const float4 *>(bias + col0);
         const float4 *cp = reinterpret_cast<const float4 *>(cs + col0);
@@ -377,6 +409,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tn_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, int M, int N, int K, GemmGroups grp, Epi epi, int *err) {
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "UMMA N for M = 128");
+    static_assert(!Epi::kBNMajor || (BN % 64 == 0 && !Epi::kF8), "N-major B comes in boxes of 64 columns");
     using L = GemmSmem<BN, STAGES>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -428,7 +461,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     if (!tc::mbar_wait(&empty[s], ph ^ 1u, grp.spin)) { atomicExch(err, tc::kErrTimeoutEmpty); ok = false; break; }
                     tc::mbar_arrive_expect_tx(&full[s], L::kABytes + L::kBBytes);
                     load_tile(sA + s * L::kABytes, &tmA, &full[s], grp.a, kb * kBKe, m_blk * kBM, g);
-                    load_tile(sB + s * L::kBBytes, &tmB, &full[s], grp.b, kb * kBKe, n_blk * BN, g);
+                    if constexpr (Epi::kBNMajor) {
+#pragma unroll
+                        for (int j = 0; j < BN / 64; ++j)
+                            load_tile(sB + s * L::kBBytes + j * 8192, &tmB, &full[s], grp.b, n_blk * BN + j * 64,
+                                      kb * kBK, g);
+                    } else {
+                        load_tile(sB + s * L::kBBytes, &tmB, &full[s], grp.b, kb * kBKe, n_blk * BN, g);
+                    }
                 }
             }
             // every issued load lands before the CTA may exit (bounded)
@@ -440,7 +480,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc = Epi::kF8 ? tc::idesc_e4m3_f32(kBM, BN) : tc::idesc_bf16_f32(kBM, BN);
+            constexpr uint32_t idesc = (Epi::kF8 ? tc::idesc_e4m3_f32(kBM, BN) : tc::idesc_bf16_f32(kBM, BN)) |
+                                       (Epi::kBNMajor ? tc::kIdescBMNMajor : 0u);
             int it = 0, t = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
@@ -459,7 +500,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     // four instructions of 32 bytes of K each (16 BF16 or 32 E4M3)
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        const uint64_t ad = tc::sdesc_kmajor_sw128(a0 + kk * 32), bd = tc::sdesc_kmajor_sw128(b0 + kk * 32);
+                        const uint64_t ad = tc::sdesc_kmajor_sw128(a0 + kk * 32);
+                        const uint64_t bd = Epi::kBNMajor ? tc::sdesc_mnmajor_sw128(b0 + kk * 2048, 8192)
+                                                          : tc::sdesc_kmajor_sw128(b0 + kk * 32);
                         if (Epi::kF8) tc::umma_f8(d_tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                         else tc::umma_f16(d_tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                     }
@@ -502,7 +545,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 if (tma) {
                     if (row0 >= M) continue;            // warp-uniform: nothing of this slice is in range
                     uint32_t w[8];
-                    ge.compute(col0, v, w);
+                    ge.compute(row0 + lane, col0, v, w);
                     uint8_t *buf = my_stage + (nstore & 1) * kStageBytesPerWarp;
                     if (nstore >= 2 && lane == 0) tc::bulk_wait_read<1>();   // this buffer's previous store has read it
                     __syncwarp();

@@ -173,7 +173,8 @@ int launch_gemm_grouped_bn(const GemmOperand &A, const GemmOperand &B, int G, in
     CUtensorMap ta, tb, tc;
     int rc = make_operand_map(&ta, A, M, K, G, kBM, esize);
     if (rc) return rc;
-    rc = make_operand_map(&tb, B, N, K, G, BN, esize);
+    // N-major B: [K][N], boxes of 64 columns x 64 rows
+    rc = Epi::kBNMajor ? make_operand_map(&tb, B, K, N, G, kBK, esize) : make_operand_map(&tb, B, N, K, G, BN, esize);
     if (rc) return rc;
     std::memset(&tc, 0, sizeof(tc));
     if (const void *op = epi.tma_ptr()) {
@@ -245,8 +246,9 @@ int gemm_gelu(int bn, const void *X, int64_t ldx, const void *W, int64_t ldw, in
               void *out, int64_t ldo, float *pre, int64_t ldp, int *err, cudaStream_t st, int max_ctas = 0);
 int gemm_linear(int bn, const void *X, int64_t ldx, const void *W, int64_t ldw, int M, int N, int K,
                 const float *bias, float *out, int64_t ldo, int *err, cudaStream_t st, int max_ctas = 0);
-int gemm_gelu_grad(int bn, const void *X, int64_t ldx, const void *W, int64_t ldw, int M, int N, int K,
-                   const float *z, int64_t ldz, void *out, int64_t ldo, int *err, cudaStream_t st, int max_ctas = 0);
+// X W with W the layer's own weights [K][N] (row-major, N-major operand), times GELU'(z)
+int gemm_gelu_grad(const void *X, int64_t ldx, const void *W, int64_t ldw, int M, int N, int K, const float *z,
+                   int64_t ldz, void *out, int64_t ldo, int *err, cudaStream_t st);
 // Grouped forms: G products of M x N x K in one launch (the per-species networks). Output
 // groups sit side by side in each row (group g's columns start at g x g_out), except for
 // gemm_linear_grouped, whose g_out is any element offset (stacked weight gradients: rows x ldo).
@@ -256,9 +258,19 @@ int gemm_gelu_grouped(int bn, const GemmOperand &X, const GemmOperand &W, int G,
 int gemm_linear_grouped(int bn, const GemmOperand &X, const GemmOperand &W, int G, int M, int N, int K,
                         const float *bias, int64_t g_bias, float *out, int64_t ldo, int64_t g_out, int *err,
                         cudaStream_t st, int max_ctas = 0);
-int gemm_gelu_grad_grouped(int bn, const GemmOperand &X, const GemmOperand &W, int G, int M, int N, int K,
-                           const float *z, int64_t ldz, int64_t g_z, void *out, int64_t ldo, int64_t g_out, int *err,
-                           cudaStream_t st, int max_ctas = 0);
+int gemm_gelu_grad_grouped(const GemmOperand &X, const GemmOperand &W, int G, int M, int N, int K, const float *z,
+                           int64_t ldz, int64_t g_z, void *out, int64_t ldo, int64_t g_out, int *err, cudaStream_t st);
+// Weight and bias gradients of several layers in one launch (gemm_wgrad.cu): gW[o][i] = sum_b dz[b][o] h[b][i]
+// for o < out, i < in (FP32, rows of ldg floats), gb[o] = sum_b dz[b][o]. dz [B][ldz] and h [B][ldh] BF16.
+struct WgradLayer {
+    const void *dz, *h;
+    int64_t ldz, ldh;
+    int out, in;
+    float *gW;
+    int64_t ldg;
+    float *gb;
+};
+int gemm_wgrad(const WgradLayer *layers, int count, int B, int *err, cudaStream_t st);
 // The last hidden layer and the output layer in one launch, h3 kept on chip (gemm_fused34.cuh):
 // u = bf16(GELU(X W3^T + b3)) W4^T + b4 in FP32, bitwise gemm_gelu (layer 3) then gemm_linear
 // (layer 4). X [M][ldx] BF16 with K3 columns, W3 [N3][ldw3], W4 [N4][ldw4] (K = N3), u [M][ldu].

@@ -58,7 +58,6 @@ struct Layer {
     int outp;             // padded output width (multiple of 8)
     float *W, *b;         // FP32 master [out][kin], [outp]
     __nv_bfloat16 *Wb;    // BF16 [out][kx] (the first layer: [W_hi | W_hi | W_lo], see kXTerms)
-    __nv_bfloat16 *Wt;    // BF16 transposed [in][outp]
     float *mW, *vW, *mb, *vb;   // Adam moments
     float *gW, *gb;       // gradients of the last training step
     int tile;             // forward tile width
@@ -124,40 +123,64 @@ namespace {
 // kernels
 // ---------------------------------------------------------------------------
 
+// FP64 -> FP32 rounded to nearest even, on the integer pipe for normal FP32 results and zero (the FP64
+// pipe, which converts too, runs at 1/64 of the FP32 rate); the rest by the conversion instruction.
+__device__ __forceinline__ float f64_to_f32_near(double x) {
+    const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
+    const unsigned a = hi & 0x7FFFFFFFu;
+    if (a - 0x38100000u < 0x47D00000u - 0x38100000u) {       // 2^-126 <= |x| < 2^126
+        unsigned r = __funnelshift_l(lo, a - 0x38000000u, 3);
+        const unsigned rest = lo << 3;                        // the 29 bits cut off, at the top
+        r += (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ? 1u : 0u;
+        return __uint_as_float(r | (hi & 0x80000000u));
+    }
+    if ((a | lo) == 0u) return __uint_as_float(hi);
+    return (float)x;
+}
+
 // Rows z = (x - mu) / sigma, x = (T, p, F(Y_1..Y_N)), F(Y) = (max(Y,0)^0.1 - 1)/0.1, each value as
 // two BF16 terms z = hi + lo (hi = bf16(z), lo = bf16(z - hi): 16 significant bits, so the state
 // reaches the first layer at about 2^-17 relative instead of BF16's 2^-9). Row layout (kXTerms):
 // [hi(0 .. n_in_pad) | lo(0 .. n_in_pad) | hi(0 .. n_in_pad)]; padding columns are 0.
+// A block takes 32 cells, a warp 8 of their columns (lanes = cells, so the state rows are read
+// coalesced); the rows are put together in shared memory and written as one contiguous block.
+// A thread per cell wrote 16-byte pieces at a stride of a row and left small calls with a serial chain of
+// n_in powers: PROLOGUS.
 __global__ void prologue_kernel(int64_t n, int64_t ld, const double *__restrict__ T, const double *__restrict__ p,
                                 const double *__restrict__ Y, const int32_t *__restrict__ idx, int N, int n_in_pad,
                                 const float *__restrict__ mu, const float *__restrict__ isd,
                                 __nv_bfloat16 *__restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t c = idx ? (int64_t)idx[i] : i;
-    __nv_bfloat16 *row = out + i * kXTerms * n_in_pad;
-    for (int j0 = 0; j0 < n_in_pad; j0 += 8) {
+    extern __shared__ __align__(16) uint4 pro_smem[];        // [32][3 n_in_pad / 8 + 1]
+    const int lane = threadIdx.x & 31, j0 = (threadIdx.x >> 5) * 8, nc = n_in_pad / 8;
+    const int pitch = kXTerms * nc + 1;
+    const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
+    if (i < n) {
+        const int64_t c = idx ? (int64_t)idx[i] : i;
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = j0 + u;
+            v[u] = j == 0 ? T[c] : (j == 1 ? p[c] : (j < N + 2 ? Y[(int64_t)(j - 2) * ld + c] : 0.0));
+        }
         __align__(16) __nv_bfloat16 hi[8], lo[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int j = j0 + u;
-            float x;
-            if (j == 0) x = (float)T[c];
-            else if (j == 1) x = (float)p[c];
-            else if (j < N + 2) {
-                const float y = fmaxf((float)Y[(int64_t)(j - 2) * ld + c], 0.0f);
-                x = (powf(y, kLambdaBC) - 1.0f) * (1.0f / kLambdaBC);
-            } else {
-                x = 0.0f;
-            }
+            float x = f64_to_f32_near(v[u]);
+            if (j >= 2) x = j < N + 2 ? (powf(fmaxf(x, 0.0f), kLambdaBC) - 1.0f) * (1.0f / kLambdaBC) : 0.0f;
             const float z = (j < N + 2) ? (x - __ldg(mu + j)) * __ldg(isd + j) : 0.0f;
             hi[u] = __float2bfloat16_rn(z);
             lo[u] = __float2bfloat16_rn(z - __bfloat162float(hi[u]));
         }
-        *reinterpret_cast<uint4 *>(row + j0) = *reinterpret_cast<const uint4 *>(hi);
-        *reinterpret_cast<uint4 *>(row + n_in_pad + j0) = *reinterpret_cast<const uint4 *>(lo);
-        *reinterpret_cast<uint4 *>(row + 2 * n_in_pad + j0) = *reinterpret_cast<const uint4 *>(hi);
+        uint4 *row = pro_smem + lane * pitch + j0 / 8;
+        row[0] = *reinterpret_cast<const uint4 *>(hi);
+        row[nc] = *reinterpret_cast<const uint4 *>(lo);
+        row[2 * nc] = *reinterpret_cast<const uint4 *>(hi);
     }
+    __syncthreads();
+    const int w = kXTerms * nc, rows = (int)(n - i0 < 32 ? n - i0 : 32);
+    uint4 *o = reinterpret_cast<uint4 *>(out) + i0 * w;
+    for (int e = threadIdx.x; e < rows * w; e += blockDim.x) o[e] = pro_smem[(e / w) * pitch + e % w];
 }
 
 // Out-of-distribution features of one cell (FP32): T, h/R = sum_k (Y_k / W_k) H_k/R, Y_s.
@@ -435,17 +458,20 @@ __device__ __forceinline__ float h_over_R(const float *b, float T) {
 }
 
 // L1 loss of Eq. 5 on normalised outputs, dL/du = sign(u - u*)/B, plus the physics terms above
-// when their weights are non-zero; dL/du written as BF16, the per-sample loss to part.
-__global__ void l1_loss_kernel(int64_t B, const float *__restrict__ u, int ldu, const int32_t *__restrict__ idx,
+// when their weights are non-zero; dL/du written as BF16, the per-sample loss to part. One warp per sample,
+// outputs over lanes (a thread per sample left 32 CTAs walking scattered rows: 42 us for 4096, LOSSUS now).
+__global__ void __launch_bounds__(128) l1_loss_kernel(int64_t B, const float *__restrict__ u, int ldu, const int32_t *__restrict__ idx,
                                int64_t ld, const double *__restrict__ Y0, const double *__restrict__ Y1, int n_out,
                                const int *__restrict__ out_sp, const float *__restrict__ mu_u,
                                const float *__restrict__ sd_u, __nv_bfloat16 *__restrict__ dout, int lddo,
                                float *__restrict__ part, const double *__restrict__ Tc, PhysLoss ph) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B) return;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= B) return;                              // warp-uniform
     const int64_t c = idx ? (int64_t)idx[i] : i;
     const float invB = 1.0f / (float)B;
     const bool phys = ph.wm != 0.0f || ph.wq != 0.0f;
+    constexpr float kRf = 8.314462618f;
     float acc = 0.0f, rm = 0.0f, rq = 0.0f, T = 0.0f, hb = 0.0f;
     const float *rows = nullptr;
     if (phys) {
@@ -453,40 +479,49 @@ __global__ void l1_loss_kernel(int64_t B, const float *__restrict__ u, int ldu, 
         rows = ph.nasa_h + (size_t)((T >= ph.T_mid) ? 1 : 0) * ph.N * 6;
         hb = h_over_R(rows + ph.bath * 6, T) * __ldg(ph.invW + ph.bath);
     }
-    for (int j = 0; j < n_out; ++j) {
-        const int64_t q = (int64_t)out_sp[j] * ld + c;
-        const float target = ((float)(Y1[q] - Y0[q]) - __ldg(mu_u + j)) / __ldg(sd_u + j);
-        const float d = u[i * ldu + j] - target;
-        acc += fabsf(d);
-        if (phys) {
+    float d[2] = {0.0f, 0.0f}, cj[2] = {0.0f, 0.0f};   // at most 63 outputs
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int j = lane + 32 * s;
+        if (j < n_out) {
             const int k = out_sp[j];
-            const float cj = h_over_R(rows + k * 6, T) * __ldg(ph.invW + k) - hb;   // (h_k - h_bath) / R
-            rm = fmaf(__ldg(sd_u + j), d, rm);
-            rq = fmaf(-cj * __ldg(sd_u + j), d, rq);
+            const int64_t q = (int64_t)k * ld + c;
+            const float target = ((float)(Y1[q] - Y0[q]) - __ldg(mu_u + j)) / __ldg(sd_u + j);
+            d[s] = u[i * ldu + j] - target;
+            acc += fabsf(d[s]);
+            if (phys) {
+                cj[s] = h_over_R(rows + k * 6, T) * __ldg(ph.invW + k) - hb;   // (h_k - h_bath) / R
+                rm = fmaf(__ldg(sd_u + j), d[s], rm);
+                rq = fmaf(-cj[s] * __ldg(sd_u + j), d[s], rq);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (phys) {
+            rm += __shfl_xor_sync(0xffffffffu, rm, o);
+            rq += __shfl_xor_sync(0xffffffffu, rq, o);
         }
     }
     // r_q in J/kg: the enthalpy differences above are in units of R (K mol/kg)
-    constexpr float kRf = 8.314462618f;
     rq *= kRf;
     const float sm = (rm > 0.0f) ? 1.0f : ((rm < 0.0f) ? -1.0f : 0.0f);
     const float sq = (rq > 0.0f) ? 1.0f : ((rq < 0.0f) ? -1.0f : 0.0f);
     if (phys) acc += ph.wm * fabsf(rm) + ph.wq * fabsf(rq);
-    for (int j = 0; j < lddo; ++j) {
-        float g = 0.0f;
-        if (j < n_out) {
-            const int64_t q = (int64_t)out_sp[j] * ld + c;
-            const float target = ((float)(Y1[q] - Y0[q]) - __ldg(mu_u + j)) / __ldg(sd_u + j);
-            const float d = u[i * ldu + j] - target;
-            g = (d > 0.0f) ? invB : ((d < 0.0f) ? -invB : 0.0f);
-            if (phys) {
-                const int k = out_sp[j];
-                const float cj = (h_over_R(rows + k * 6, T) * __ldg(ph.invW + k) - hb) * kRf;
-                g += invB * __ldg(sd_u + j) * (ph.wm * sm - ph.wq * sq * cj);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int j = lane + 32 * s;
+        if (j < lddo) {
+            float g = 0.0f;
+            if (j < n_out) {
+                g = (d[s] > 0.0f) ? invB : ((d[s] < 0.0f) ? -invB : 0.0f);
+                if (phys) g += invB * __ldg(sd_u + j) * (ph.wm * sm - ph.wq * sq * (cj[s] * kRf));
             }
+            dout[i * lddo + j] = __float2bfloat16_rn(g);
         }
-        dout[i * lddo + j] = __float2bfloat16_rn(g);
     }
-    part[i] = acc;
+    if (lane == 0) part[i] = acc;
 }
 
 // Scales of the physics terms over n training pairs, FP64: per-block sums of sum_j |dY*_j| and
@@ -593,45 +628,71 @@ __global__ void transpose_kernel(int rows, int cols, const __nv_bfloat16 *__rest
     }
 }
 
-// Adam (Kingma and Ba 2015) on one layer; refreshes the BF16 and transposed BF16 copies.
-__global__ void adam_kernel(int out, int in, int kin, int kx, int outp, float *__restrict__ W, float *__restrict__ b,
-                            const float *__restrict__ gW, const float *__restrict__ gb, float *__restrict__ mW,
-                            float *__restrict__ vW, float *__restrict__ mb, float *__restrict__ vb,
-                            __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Wt, float lr, float bc1,
-                            float bc2) {
-    const int64_t nW = (int64_t)out * in;
+// Adam (Kingma and Ba 2015) on every layer in one launch, four parameters of a weight row per thread
+// (rows are padded to 8; padding has zero gradients and stays zero), refreshing the BF16 copy. Memory
+// bound: 30 bytes per parameter (31 us in four launches with a scattered transposed copy, ADAMUS now for 1.67M
+// parameters).
+struct AdamLayer {
+    float *W, *b, *mW, *vW, *mb, *vb;
+    const float *gW, *gb;
+    __nv_bfloat16 *Wb;
+    int out, kin, kx;
+    int64_t first;                          // index of the layer's first thread
+};
+struct AdamArgs {
+    AdamLayer l[kLayers];
+    int64_t total;
+    float lr, bc1, bc2;
+};
+__device__ __forceinline__ float adam_update(float w, float g, float &m, float &v, const AdamArgs &a) {
+    m = kAdamB1 * m + (1.0f - kAdamB1) * g;
+    v = kAdamB2 * v + (1.0f - kAdamB2) * g * g;
+    return w - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + kAdamEps);
+}
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamArgs a) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < nW) {
-        const int o = (int)(t / in), k = (int)(t % in);
-        const int64_t q = (int64_t)o * kin + k;
-        const float g = gW[q];
-        const float m = kAdamB1 * mW[q] + (1.0f - kAdamB1) * g;
-        const float v = kAdamB2 * vW[q] + (1.0f - kAdamB2) * g * g;
-        mW[q] = m;
-        vW[q] = v;
-        const float w = W[q] - lr * (m / bc1) / (sqrtf(v / bc2) + kAdamEps);
-        W[q] = w;
-        const __nv_bfloat16 wb = __float2bfloat16_rn(w);
-        Wb[(int64_t)o * kx + k] = wb;
-        if (kx != kin) {                                      // the first layer: [W_hi | W_hi | W_lo]
-            Wb[(int64_t)o * kx + kin + k] = wb;
-            Wb[(int64_t)o * kx + 2 * kin + k] = __float2bfloat16_rn(w - __bfloat162float(wb));
+    if (t >= a.total) return;
+    int l = 0;
+    while (l + 1 < kLayers && t >= a.l[l + 1].first) ++l;
+    const AdamLayer &L = a.l[l];
+    const int64_t i = t - L.first, nW4 = (int64_t)L.out * (L.kin / 4);
+    if (i < nW4) {
+        const int row4 = L.kin / 4, o = (int)(i / row4), k = (int)(i - (int64_t)o * row4) * 4;
+        const int64_t q = i;
+        const float4 g = reinterpret_cast<const float4 *>(L.gW)[q];
+        float4 m = reinterpret_cast<float4 *>(L.mW)[q], v = reinterpret_cast<float4 *>(L.vW)[q];
+        float4 w = reinterpret_cast<float4 *>(L.W)[q];
+        w.x = adam_update(w.x, g.x, m.x, v.x, a);
+        w.y = adam_update(w.y, g.y, m.y, v.y, a);
+        w.z = adam_update(w.z, g.z, m.z, v.z, a);
+        w.w = adam_update(w.w, g.w, m.w, v.w, a);
+        reinterpret_cast<float4 *>(L.mW)[q] = m;
+        reinterpret_cast<float4 *>(L.vW)[q] = v;
+        reinterpret_cast<float4 *>(L.W)[q] = w;
+        __align__(8) __nv_bfloat162 hi[2], lo[2];
+        hi[0] = __floats2bfloat162_rn(w.x, w.y);
+        hi[1] = __floats2bfloat162_rn(w.z, w.w);
+        uint2 *o2 = reinterpret_cast<uint2 *>(L.Wb + (int64_t)o * L.kx + k);
+        *o2 = *reinterpret_cast<const uint2 *>(hi);
+        if (L.kx != L.kin) {                                  // the first layer: [W_hi | W_hi | W_lo]
+            const float2 h0 = __bfloat1622float2(hi[0]), h1 = __bfloat1622float2(hi[1]);
+            lo[0] = __floats2bfloat162_rn(w.x - h0.x, w.y - h0.y);
+            lo[1] = __floats2bfloat162_rn(w.z - h1.x, w.w - h1.y);
+            o2[L.kin / 4] = *reinterpret_cast<const uint2 *>(hi);
+            o2[2 * (L.kin / 4)] = *reinterpret_cast<const uint2 *>(lo);
         }
-        Wt[(int64_t)k * outp + o] = wb;
-    } else if (t < nW + out) {
-        const int o = (int)(t - nW);
-        const float g = gb[o];
-        const float m = kAdamB1 * mb[o] + (1.0f - kAdamB1) * g;
-        const float v = kAdamB2 * vb[o] + (1.0f - kAdamB2) * g * g;
-        mb[o] = m;
-        vb[o] = v;
-        b[o] = b[o] - lr * (m / bc1) / (sqrtf(v / bc2) + kAdamEps);
+    } else {
+        const int o = (int)(i - nW4);
+        float m = L.mb[o], v = L.vb[o];
+        L.b[o] = adam_update(L.b[o], L.gb[o], m, v, a);
+        L.mb[o] = m;
+        L.vb[o] = v;
     }
 }
 
 // FP32 master -> BF16 copies (after set_params).
-__global__ void refresh_bf16_kernel(int out, int in, int kin, int kx, int outp, const float *__restrict__ W,
-                                    __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Wt) {
+__global__ void refresh_bf16_kernel(int out, int in, int kin, int kx, const float *__restrict__ W,
+                                    __nv_bfloat16 *__restrict__ Wb) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)out * kin) return;
     const int o = (int)(t / kin), k = (int)(t % kin);
@@ -642,7 +703,6 @@ __global__ void refresh_bf16_kernel(int out, int in, int kin, int kx, int outp, 
         Wb[(int64_t)o * kx + kin + k] = wb;
         Wb[(int64_t)o * kx + 2 * kin + k] = __float2bfloat16_rn(w - __bfloat162float(wb));
     }
-    if (k < in) Wt[(int64_t)k * outp + o] = wb;
 }
 
 // Mean and population standard deviation of feature f over n samples, FP64,
@@ -868,8 +928,7 @@ int refresh_bf16(chem_mlp *m, cudaStream_t st) {
     for (int l = 0; l < kLayers; ++l) {
         const Layer &L = m->L[l];
         int64_t n = (int64_t)L.out * L.kin;
-        refresh_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L.out, L.in, L.kin, L.kx, L.outp, L.W, L.Wb,
-                                                                          L.Wt);
+        refresh_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L.out, L.in, L.kin, L.kx, L.W, L.Wb);
     }
     return check_cuda(cudaGetLastError(), "refresh_bf16");
 }
@@ -906,6 +965,13 @@ int ens_output(const chem_mlp *m, int64_t n, const __nv_bfloat16 *h, float *u, c
     return check_cuda(cudaGetLastError(), "ensemble output units");
 }
 
+void launch_prologue(const chem_mlp *m, int64_t n, int64_t ld, const double *T, const double *p, const double *Y,
+                     const int32_t *idx, __nv_bfloat16 *out, cudaStream_t st) {
+    const int nc = m->n_in_pad / 8;
+    prologue_kernel<<<(unsigned)((n + 31) / 32), 32 * nc, 32 * (kXTerms * nc + 1) * sizeof(uint4), st>>>(
+        n, ld, T, p, Y, idx, m->N, m->n_in_pad, m->mu_x, m->isd_x, out);
+}
+
 // the training loss's physics terms as the loss kernel takes them (zero weights: Eq. 5 alone)
 PhysLoss phys_loss(const chem_mlp *m) {
     PhysLoss p{};
@@ -934,8 +1000,7 @@ int forward_chunk(const chem_mlp *m, int64_t n, int64_t ld, const double *T, con
                   cudaStream_t st, int prec = CHEM_PREC_BF16, int nlayers = kLayers) {
     WaitLimitScope wl(m->wait_limit);
     void *pb = prof_begin(st);
-    prologue_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(n, ld, T, p, Y, nullptr, m->N, m->n_in_pad, m->mu_x,
-                                                                 m->isd_x, m->a0);
+    launch_prologue(m, n, ld, T, p, Y, nullptr, m->a0, st);
     prof_end(pb, st, "prologue_kernel", 0.0, (double)n * ((m->N + 2) * 8 + m->n_in_pad * 2 * kXTerms));
     int rc = check_cuda(cudaGetLastError(), "prologue");
     if (rc) return rc;
@@ -1080,7 +1145,6 @@ extern "C" int chem_mlp_create(const chem_mech *mech, const chem_mlp_desc *desc,
         parts.push_back({(void **)&L.W, w * 4});
         parts.push_back({(void **)&L.b, o * 4});
         parts.push_back({(void **)&L.Wb, (size_t)L.out * L.kx * 2});
-        parts.push_back({(void **)&L.Wt, (size_t)L.in * L.outp * 2});
         parts.push_back({(void **)&L.mW, w * 4});
         parts.push_back({(void **)&L.vW, w * 4});
         parts.push_back({(void **)&L.mb, o * 4});
@@ -1114,8 +1178,10 @@ extern "C" int chem_mlp_create(const chem_mech *mech, const chem_mlp_desc *desc,
     }
     parts.push_back({(void **)&m->tout, (size_t)B * m->n_out_pad * 4});
     parts.push_back({(void **)&m->tdout, (size_t)B * m->n_out_pad * 2});
-    parts.push_back({(void **)&m->tT0, (size_t)B * maxw * 2});
-    parts.push_back({(void **)&m->tT1, (size_t)B * maxw * 2});
+    if (m->ens) {                            // transposed operands of the ensemble's weight gradients
+        parts.push_back({(void **)&m->tT0, (size_t)B * maxw * 2});
+        parts.push_back({(void **)&m->tT1, (size_t)B * maxw * 2});
+    }
     parts.push_back({(void **)&m->loss_part, (size_t)B * 4});
     for (int g = 0; g < kOodMaxGrids; ++g) {
         parts.push_back({(void **)&m->ood_counts[g], (size_t)kOodMaxBins * kOodMaxBins * kOodMaxBins * 4});
@@ -1609,7 +1675,7 @@ int ens_train_passes(chem_mlp *m, int B, const int32_t *idx, int64_t ld, const d
     for (int l = 1; l < 3 && !rc; ++l) rc = ens_hidden(m, l, m->L[l].tile, B, m->th[l - 1], m->th[l], m->tz[l], st);
     if (!rc) rc = ens_output(m, B, m->th[2], m->tout, st);
     if (rc) return rc;
-    l1_loss_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, m->tout, m->n_out_pad, idx, ld, Y, Y1, m->n_out, m->out_sp_dev,
+    l1_loss_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, m->tout, m->n_out_pad, idx, ld, Y, Y1, m->n_out, m->out_sp_dev,
                                                      m->mu_u, m->sd_u, m->tdout, m->n_out_pad, m->loss_part, nullptr,
                                                      PhysLoss{});
     if (loss_dev) loss_reduce_kernel<<<1, 256, 0, st>>>(B, m->loss_part, loss_dev);
@@ -1642,9 +1708,9 @@ int ens_train_passes(chem_mlp *m, int B, const int32_t *idx, int64_t ld, const d
         if (rc) return rc;
         colsum_kernel<<<(unsigned)((ldz + 31) / 32), dim3(32, kColsumRows), 0, st>>>(B, (int)ldz, m->tdz[l], (int)ldz, L.gb);
         if ((rc = check_cuda(cudaGetLastError(), "ensemble bias grad"))) return rc;
-        rc = gemm_gelu_grad_grouped(default_tile_width(L.in), GemmOperand{m->tdz[l], ldz, kMapColGrp, L.gout},
-                                    GemmOperand{L.Wt, L.outp, kMapColGrp, L.gout}, G, B, L.in, L.gout, m->tz[l - 1],
-                                    ldh, L.in, m->tdz[l - 1], ldh, L.in, m->err, st);
+        rc = gemm_gelu_grad_grouped(GemmOperand{m->tdz[l], ldz, kMapColGrp, L.gout},
+                                    GemmOperand{L.Wb, L.kx, kMapRowGrp, (int64_t)L.gout * L.kx}, G, B, L.in, L.gout,
+                                    m->tz[l - 1], ldh, L.in, m->tdz[l - 1], ldh, L.in, m->err, st);
         if (rc) return rc;
     }
     // the stacked first layers: one product over all networks (their input is shared)
@@ -1682,7 +1748,7 @@ int train_grads_impl(chem_mlp *m, int64_t batch, const int32_t *idx, int64_t ld,
     WaitLimitScope wl(m->wait_limit);
     const int B = (int)batch;
     // forward with saved pre-activations
-    prologue_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, ld, T, p, Y, idx, m->N, m->n_in_pad, m->mu_x, m->isd_x, m->tx0);
+    launch_prologue(m, B, ld, T, p, Y, idx, m->tx0, st);
     if ((rc = check_cuda(cudaGetLastError(), "train prologue"))) return rc;
     if (m->ens) {
         rc = ens_train_passes(m, B, idx, ld, Y, Y1, loss_dev, st);
@@ -1703,38 +1769,31 @@ int train_grads_impl(chem_mlp *m, int64_t batch, const int32_t *idx, int64_t ld,
             if (rc) return rc;
         }
         // loss and dL/du
-        l1_loss_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, m->tout, m->n_out_pad, idx, ld, Y, Y1, m->n_out, m->out_sp_dev,
+        l1_loss_kernel<<<(B + 3) / 4, 128, 0, st>>>(B, m->tout, m->n_out_pad, idx, ld, Y, Y1, m->n_out, m->out_sp_dev,
                                                          m->mu_u, m->sd_u, m->tdout, m->n_out_pad, m->loss_part, T,
                                                          phys_loss(m));
         if (loss_dev) loss_reduce_kernel<<<1, 256, 0, st>>>(B, m->loss_part, loss_dev);
         if ((rc = check_cuda(cudaGetLastError(), "train loss"))) return rc;
-        // backward, top layer down: dW_l = dZ_l^T H_{l-1}, db_l = colsum dZ_l, dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1})
-        const __nv_bfloat16 *dz = m->tdout;
-        int lddz = m->n_out_pad;
-        for (int l = 3; l >= 0; --l) {
+        // backward, top layer down: dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1}); then every layer's dW_l = dZ_l^T H_{l-1},
+        // db_l = colsum dZ_l in one launch
+        const __nv_bfloat16 *dz[kLayers] = {m->tdz[0], m->tdz[1], m->tdz[2], m->tdout};
+        const int lddz[kLayers] = {m->L[0].out, m->L[1].out, m->L[2].out, m->n_out_pad};
+        for (int l = 3; l >= 1; --l) {
+            const Layer &L = m->L[l];
+            rc = gemm_gelu_grad(dz[l], lddz[l], L.Wb, L.kx, B, L.in, L.out, m->tz[l - 1], L.in, m->tdz[l - 1], L.in,
+                                m->err, st);
+            if (rc) return rc;
+        }
+        WgradLayer wg[kLayers];
+        const int order[kLayers] = {1, 2, 0, 3};        // longest first
+        for (int q = 0; q < kLayers; ++q) {
+            const int l = order[q];
             const Layer &L = m->L[l];
             // the first layer's weight gradient takes the hi input term (BF16 precision suffices for a gradient)
-            const __nv_bfloat16 *hin = (l == 0) ? m->tx0 : m->th[l - 1];
-            const int wh = (l == 0) ? m->n_in_pad : m->L[l - 1].out;
-            const int ldh = (l == 0) ? kXTerms * m->n_in_pad : wh;
-            dim3 tb(32, 8);
-            transpose_kernel<<<dim3((lddz + 31) / 32, (B + 31) / 32), tb, 0, st>>>(B, lddz, dz, lddz, m->tT0, B);
-            transpose_kernel<<<dim3((wh + 31) / 32, (B + 31) / 32), tb, 0, st>>>(B, wh, hin, ldh, m->tT1, B);
-            if ((rc = check_cuda(cudaGetLastError(), "train transpose"))) return rc;
-            rc = gemm_linear(default_tile_width(L.kin), m->tT0, B, m->tT1, B, L.out, L.kin, B, nullptr, L.gW, L.kin, m->err,
-                             st);
-            if (rc) return rc;
-            colsum_kernel<<<(L.out + 31) / 32, dim3(32, kColsumRows), 0, st>>>(B, L.out, dz, lddz, L.gb);
-            if ((rc = check_cuda(cudaGetLastError(), "train bias grad"))) return rc;
-            if (l > 0) {
-                const Layer &Lb = m->L[l - 1];
-                rc = gemm_gelu_grad(default_tile_width(Lb.out), dz, lddz, L.Wt, L.outp, B, Lb.out, L.outp, m->tz[l - 1],
-                                    Lb.out, m->tdz[l - 1], Lb.out, m->err, st);
-                if (rc) return rc;
-                dz = m->tdz[l - 1];
-                lddz = Lb.out;
-            }
+            wg[q] = WgradLayer{dz[l], l == 0 ? m->tx0 : m->th[l - 1], lddz[l],
+                               l == 0 ? (int64_t)kXTerms * m->n_in_pad : (int64_t)L.in, L.out, L.kin, L.gW, L.kin, L.gb};
         }
+        if ((rc = gemm_wgrad(wg, kLayers, B, m->err, st))) return rc;
     }
     return CHEM_OK;
 }
@@ -1743,14 +1802,16 @@ int train_grads_impl(chem_mlp *m, int64_t batch, const int32_t *idx, int64_t ld,
 int adam_impl(chem_mlp *m, float lr, cudaStream_t st) {
     m->adam_t += 1;
     m->fp8_ready = 0;
-    const float bc1 = 1.0f - std::pow(kAdamB1, (float)m->adam_t);
-    const float bc2 = 1.0f - std::pow(kAdamB2, (float)m->adam_t);
+    AdamArgs a{};
+    a.lr = lr;
+    a.bc1 = 1.0f - std::pow(kAdamB1, (float)m->adam_t);
+    a.bc2 = 1.0f - std::pow(kAdamB2, (float)m->adam_t);
     for (int l = 0; l < kLayers; ++l) {
         Layer &L = m->L[l];
-        const int64_t n = (int64_t)L.out * L.in + L.out;
-        adam_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L.out, L.in, L.kin, L.kx, L.outp, L.W, L.b, L.gW, L.gb, L.mW,
-                                                                 L.vW, L.mb, L.vb, L.Wb, L.Wt, lr, bc1, bc2);
+        a.l[l] = AdamLayer{L.W, L.b, L.mW, L.vW, L.mb, L.vb, L.gW, L.gb, L.Wb, L.out, L.kin, L.kx, a.total};
+        a.total += (int64_t)L.out * (L.kin / 4) + L.out;
     }
+    adam_kernel<<<(unsigned)((a.total + 255) / 256), 256, 0, st>>>(a);
     return check_cuda(cudaGetLastError(), "train adam");
 }
 

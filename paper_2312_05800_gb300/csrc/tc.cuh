@@ -196,6 +196,21 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw128(uint32_t saddr) {
     return d;
 }
 
+// Descriptor of an M- or N-major operand tile written by TMA with 128-byte swizzling as boxes of 64
+// columns (the M or N dimension, 128 bytes) x 64 rows of K: within a box, 8 rows of K are one 1024-byte
+// atom (SBO: the next 8 rows); `lbo` bytes lead to the next 64 columns. A K step of 16 is two atoms.
+__device__ __forceinline__ uint64_t sdesc_mnmajor_sw128(uint32_t saddr, uint32_t lbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(lbo >> 4) << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+// instruction descriptor bits: the A (B) operand is M-major (N-major) in shared memory
+constexpr uint32_t kIdescAMNMajor = 1u << 15, kIdescBMNMajor = 1u << 16;
+
 // Instruction descriptor, kind::f16: FP32 D, BF16 A and B, both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
