@@ -55,10 +55,8 @@ struct DevMech {
     PropTables<double> f64;
     // FP64 kinetics
     const double *W;        // [N]
-    const double *nasa;     // [2][N][7] raw NASA-7 rows (low, high)
-    const int *rtype;       // [R]
-    const int *reac;        // [R][3]
-    const int *prod;        // [R][3]
+    const int *rtype;       // [R] in device order: Troe fall-off, three-body, elementary, so a reaction with
+                            // a third body is its own row of eff
     const double *lnA;      // [R]
     const double *beta;     // [R]
     const double *EaR;      // [R] Ea / R (K)
@@ -66,17 +64,25 @@ struct DevMech {
     const double *beta0;    // [R]
     const double *Ea0R;     // [R]
     const double *troe;     // [R][4]
-    const int *tb_row;      // [R] row in eff, or -1
     const double *eff;      // [n_tb][N]
-    const int *inc_ptr;     // [N+1] species -> reactions incidence (CSR)
-    const int2 *inc;        // (reaction, signed nu)
-    const int *dnu;         // [R] sum of nu over the reaction
-    // derived FP64 tables of the stiff integrator
-    const double *nasa_s;   // [2][N][6] S/R: a1 (times ln T), a2, a3/2, a4/3, a5/4, a7
+    // derived tables of the stiff integrator. "code" words hold a small integer as the high half of its
+    // floating-point pattern (FP32 or the high word of FP64) in bits 16..31, an index in bits 0..15.
+    const double *nasa_t;   // [2][17][64] per species (coalesced over lanes): cp/R 5, H/RT 6, S/R 6
+    const double *dnu_d;    // [R] dnu as FP64
+    const uint2 *rspec;     // [R] reactant species (bytes, N where absent), flags | product species, flags:
+                            // byte 3 of x is 1 when every species of the reaction occurs once
+    int nslot;              // distinct species of a reaction, at most (row length of d q / d C)
+    int three;              // some reaction has a third reactant or product
+    int gath_len;           // longest species incidence list, rounded up to 4
+    const unsigned *gath;   // [gath_len][64] code: nu (FP64), reaction; 0 pads
+    int ell_groups;         // groups of 32 entries of the sparse part of d wdot / d C, longest first
+    const int *ell_off, *ell_len, *ell_pos;   // [groups] first word, iterations; [groups][32] matrix offset or -1
+    const unsigned *ell_f, *ell_d;            // code: nu (FP32 / FP64), index in d q / d C [R][nslot]; 0 pads
+    const int *tbrow_ptr;   // [N+1] third-body reactions of each species (net nu != 0), ascending
+    const unsigned *tbrow_f, *tbrow_d;        // code: nu, third-body reaction
+    const float *eff_f;     // [n_tb][N] eff cut to FP32
     const double *troe_r;   // [R][4] a, 1/T***, 1/T*, T**
     const int *rsp;         // [R][6] distinct species of reaction j (first-occurrence order), -1 pad
-    const int *rnu;         // [R][6] their net stoichiometric coefficients
-    const int *tb_list;     // [n_tb] reactions with a third body, ascending
     double lnPR;            // ln(P_std / R)
     unsigned int *counters; // [kNumCounters] work-queue counters (scratch) and error words
 };

@@ -2,6 +2,7 @@
 // error reporting and option defaults of the C ABI.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -266,11 +267,8 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     PropTcTables tct;
     size_t off_tcB = 0, off_tcs = 0;
     const bool tc_ok = add_tc_tables(bb, N, W, visc, diff, tct, off_tcB, off_tcs);
-    std::vector<double> nasa(2 * N * 7);
-    for (int k = 0; k < N; ++k)
-        for (int i = 0; i < 7; ++i) { nasa[k * 7 + i] = lo[k * 7 + i]; nasa[(N + k) * 7 + i] = hi[k * 7 + i]; }
     std::vector<double> lnA(R), EaR(R), lnA0(R), Ea0R(R);
-    std::vector<int32_t> tb_row(R, -1), dnu(R, 0);
+    std::vector<double> dnu(R, 0.0);
     std::vector<double> effc;
     int n_tb = 0;
     for (int j = 0; j < R; ++j) {
@@ -280,33 +278,20 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
         Ea0R[j] = Ea0[j] / kR;
         for (int i = 0; i < 3; ++i) dnu[j] += (prod[3 * j + i] >= 0) - (reac[3 * j + i] >= 0);
         if (rtype[j] != 0) {
-            tb_row[j] = n_tb++;
+            ++n_tb;                             // these reactions come first: row j of eff is reaction j's
             for (int k = 0; k < N; ++k) effc.push_back(eff[(size_t)j * N + k]);
         }
     }
     if (effc.empty()) effc.push_back(0.0);
-    // species -> (reaction, signed nu) incidence, reactions in ascending order
-    std::vector<int32_t> inc_ptr(N + 1, 0);
-    std::vector<int2> inc;
-    for (int k = 0; k < N; ++k) {
-        inc_ptr[k] = (int)inc.size();
-        for (int j = 0; j < R; ++j) {
-            int nu = 0;
-            for (int i = 0; i < 3; ++i) nu += (prod[3 * j + i] == k) - (reac[3 * j + i] == k);
-            bool touches = false;
-            for (int i = 0; i < 3; ++i) touches |= (prod[3 * j + i] == k) || (reac[3 * j + i] == k);
-            if (touches && nu != 0) inc.push_back(make_int2(j, nu));
-        }
-    }
-    inc_ptr[N] = (int)inc.size();
-    if (inc.empty()) inc.push_back(make_int2(0, 0));
     std::vector<uint32_t> counters(kNumCounters, 0u);
-    std::vector<double> nasa_s(2 * N * 6), troe_r(4 * R);
+    std::vector<double> nasa_t((size_t)2 * 17 * 64, 0.0), troe_r(4 * R);
     for (int r = 0; r < 2; ++r)
         for (int k = 0; k < N; ++k) {
             const double *a = (r == 0 ? lo.data() : hi.data()) + 7 * k;
-            double *o = nasa_s.data() + (r * N + k) * 6;
-            o[0] = a[0]; o[1] = a[1]; o[2] = a[2] / 2.0; o[3] = a[3] / 3.0; o[4] = a[4] / 4.0; o[5] = a[6];
+            const double v[17] = {a[0], a[1], a[2], a[3], a[4],
+                                  a[0], a[1] / 2.0, a[2] / 3.0, a[3] / 4.0, a[4] / 5.0, a[5],
+                                  a[0], a[1], a[2] / 2.0, a[3] / 3.0, a[4] / 4.0, a[6]};
+            for (int i = 0; i < 17; ++i) nasa_t[((size_t)r * 17 + i) * 64 + k] = v[i];
         }
     for (int j = 0; j < R; ++j) {
         troe_r[4 * j + 0] = troe[4 * j + 0];
@@ -314,12 +299,17 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
         troe_r[4 * j + 2] = (troe[4 * j + 2] != 0.0) ? 1.0 / troe[4 * j + 2] : 0.0;
         troe_r[4 * j + 3] = troe[4 * j + 3];
     }
-    std::vector<int32_t> rsp(6 * R, -1), rnu(6 * R, 0), tb_list;
+    // distinct species of each reaction (first occurrence) with their net coefficients
+    std::vector<int32_t> rsp(6 * R, -1), rnu(6 * R, 0);
+    std::vector<uint2> rspec(R);
+    int nslot = 1, three = 0;
     for (int j = 0; j < R; ++j) {
-        int cnt = 0;
+        int cnt = 0, present = 0;
         for (int slot = 0; slot < 6; ++slot) {
             int sp = slot < 3 ? reac[3 * j + slot] : prod[3 * j + slot - 3];
             if (sp < 0) continue;
+            ++present;
+            if (slot % 3 == 2) three = 1;
             bool seen = false;
             for (int u = 0; u < cnt; ++u) seen |= (rsp[6 * j + u] == sp);
             if (seen) continue;
@@ -329,16 +319,108 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
             rnu[6 * j + cnt] = nu;
             ++cnt;
         }
-        if (rtype[j] != 0) tb_list.push_back(j);
+        nslot = cnt > nslot ? cnt : nslot;
+        unsigned w[2] = {0u, 0u};
+        for (int i = 0; i < 3; ++i) {
+            w[0] |= (unsigned)(reac[3 * j + i] >= 0 ? reac[3 * j + i] : N) << (8 * i);
+            w[1] |= (unsigned)(prod[3 * j + i] >= 0 ? prod[3 * j + i] : N) << (8 * i);
+        }
+        if (present == cnt) w[0] |= 1u << 24;
+        rspec[j] = make_uint2(w[0], w[1]);
     }
-    if (tb_list.empty()) tb_list.push_back(0);
+    // code words of the integrator's index lists
+    auto code_d = [](int nu, int idx) {
+        const double x = (double)nu;
+        uint64_t b;
+        std::memcpy(&b, &x, 8);
+        return (unsigned)((b >> 48) << 16) | (unsigned)idx;
+    };
+    auto code_f = [](int nu, int idx) {
+        const float x = (float)nu;
+        uint32_t b;
+        std::memcpy(&b, &x, 4);
+        return (b & 0xFFFF0000u) | (unsigned)idx;
+    };
+    // species -> (reaction, nu) incidence, reactions ascending, one column of `gath` per species
+    std::vector<std::vector<unsigned>> inc(N);
+    std::vector<int32_t> tbrow_ptr(N + 1, 0);
+    std::vector<unsigned> tbrow_f, tbrow_d;
+    size_t longest = 1;
+    for (int k = 0; k < N; ++k) {
+        tbrow_ptr[k] = (int)tbrow_f.size();
+        for (int j = 0; j < R; ++j)
+            for (int u = 0; u < 6 && rsp[6 * j + u] >= 0; ++u)
+                if (rsp[6 * j + u] == k && rnu[6 * j + u] != 0) {
+                    inc[k].push_back(code_d(rnu[6 * j + u], j));
+                    if (rtype[j] != 0) {
+                        tbrow_f.push_back(code_f(rnu[6 * j + u], j));
+                        tbrow_d.push_back(code_d(rnu[6 * j + u], j));
+                    }
+                }
+        longest = inc[k].size() > longest ? inc[k].size() : longest;
+    }
+    tbrow_ptr[N] = (int)tbrow_f.size();
+    if (tbrow_f.empty()) { tbrow_f.push_back(0u); tbrow_d.push_back(0u); }
+    const int gath_len = (int)((longest + 3) & ~size_t(3));
+    std::vector<unsigned> gath((size_t)gath_len * 64, 0u);
+    for (int k = 0; k < N; ++k)
+        for (size_t t = 0; t < inc[k].size(); ++t) gath[t * 64 + k] = inc[k][t];
+    // entries (row, column) of the sparse part of d wdot / d C: their reactions ascending, entries
+    // sorted by length into groups of 32 (one per lane) so that a group's lanes finish together
+    struct Entry { int pos; std::vector<unsigned> f, d; };
+    std::vector<Entry> ent;
+    {
+        std::vector<int> at((size_t)N * N, -1);
+        for (int j = 0; j < R; ++j)
+            for (int u = 0; u < 6 && rsp[6 * j + u] >= 0; ++u) {
+                if (rnu[6 * j + u] == 0) continue;
+                for (int q = 0; q < 6 && rsp[6 * j + q] >= 0; ++q) {
+                    int &e = at[(size_t)rsp[6 * j + u] * N + rsp[6 * j + q]];
+                    if (e < 0) {
+                        e = (int)ent.size();
+                        ent.push_back({(1 + rsp[6 * j + u]) * (N + 1) + 1 + rsp[6 * j + q], {}, {}});
+                    }
+                    ent[e].f.push_back(code_f(rnu[6 * j + u], j * nslot + q));
+                    ent[e].d.push_back(code_d(rnu[6 * j + u], j * nslot + q));
+                }
+            }
+        std::stable_sort(ent.begin(), ent.end(),
+                         [](const Entry &a, const Entry &b) { return a.f.size() > b.f.size(); });
+    }
+    const int ell_groups = (int)((ent.size() + 31) / 32);
+    std::vector<int32_t> ell_off(ell_groups + 1, 0), ell_len(ell_groups + 1, 0), ell_pos((size_t)32 * ell_groups + 1, -1);
+    std::vector<unsigned> ell_f, ell_d;
+    for (int q = 0; q < ell_groups; ++q) {
+        const int len = (int)ent[(size_t)32 * q].f.size();
+        ell_off[q] = (int)ell_f.size();
+        ell_len[q] = len;
+        ell_f.resize(ell_f.size() + (size_t)32 * len, 0u);
+        ell_d.resize(ell_d.size() + (size_t)32 * len, 0u);
+        for (int l = 0; l < 32; ++l) {
+            const size_t e = (size_t)32 * q + l;
+            if (e >= ent.size()) break;
+            ell_pos[e] = ent[e].pos;
+            for (size_t t = 0; t < ent[e].f.size(); ++t) {
+                ell_f[ell_off[q] + 32 * t + l] = ent[e].f[t];
+                ell_d[ell_off[q] + 32 * t + l] = ent[e].d[t];
+            }
+        }
+    }
+    if (ell_f.empty()) { ell_f.push_back(0u); ell_d.push_back(0u); }
+    std::vector<float> eff_f(effc.size());
+    for (size_t i = 0; i < effc.size(); ++i) {                // toward zero, as f64_to_f32_trunc
+        float v = (float)effc[i];
+        if (std::fabs((double)v) > std::fabs(effc[i])) v = std::nextafterf(v, 0.0f);
+        eff_f[i] = v;
+    }
 
-    size_t off_W = bb.add(W), off_nasa = bb.add(nasa), off_rtype = bb.add(rtype), off_reac = bb.add(reac),
-           off_prod = bb.add(prod), off_lnA = bb.add(lnA), off_beta = bb.add(beta), off_EaR = bb.add(EaR),
-           off_lnA0 = bb.add(lnA0), off_beta0 = bb.add(beta0), off_Ea0R = bb.add(Ea0R), off_troe = bb.add(troe),
-           off_tb = bb.add(tb_row), off_eff = bb.add(effc), off_incp = bb.add(inc_ptr), off_inc = bb.add(inc),
-           off_dnu = bb.add(dnu), off_cnt = bb.add(counters), off_nasa_s = bb.add(nasa_s),
-           off_troe_r = bb.add(troe_r), off_rsp = bb.add(rsp), off_rnu = bb.add(rnu), off_tbl = bb.add(tb_list);
+    size_t off_W = bb.add(W), off_rtype = bb.add(rtype), off_lnA = bb.add(lnA), off_beta = bb.add(beta),
+           off_EaR = bb.add(EaR), off_lnA0 = bb.add(lnA0), off_beta0 = bb.add(beta0), off_Ea0R = bb.add(Ea0R),
+           off_troe = bb.add(troe), off_eff = bb.add(effc), off_cnt = bb.add(counters), off_troe_r = bb.add(troe_r),
+           off_rsp = bb.add(rsp), off_nasa_t = bb.add(nasa_t), off_dnu = bb.add(dnu), off_rspec = bb.add(rspec),
+           off_gath = bb.add(gath), off_eo = bb.add(ell_off), off_el = bb.add(ell_len), off_ep = bb.add(ell_pos),
+           off_ef = bb.add(ell_f), off_ed = bb.add(ell_d), off_tp = bb.add(tbrow_ptr), off_tf = bb.add(tbrow_f),
+           off_td = bb.add(tbrow_d), off_eff_f = bb.add(eff_f);
 
     std::string why;
     if (!device_ok(&why)) return set_error(CHEM_EUNSUPPORTED, "chem_mech_load: " + why);
@@ -364,10 +446,7 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     d.tc.B = tc_ok ? base + off_tcB : nullptr;
     d.tc.species = tc_ok ? reinterpret_cast<const float *>(base + off_tcs) : nullptr;
     d.W = reinterpret_cast<const double *>(base + off_W);
-    d.nasa = reinterpret_cast<const double *>(base + off_nasa);
     d.rtype = reinterpret_cast<const int *>(base + off_rtype);
-    d.reac = reinterpret_cast<const int *>(base + off_reac);
-    d.prod = reinterpret_cast<const int *>(base + off_prod);
     d.lnA = reinterpret_cast<const double *>(base + off_lnA);
     d.beta = reinterpret_cast<const double *>(base + off_beta);
     d.EaR = reinterpret_cast<const double *>(base + off_EaR);
@@ -375,17 +454,27 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     d.beta0 = reinterpret_cast<const double *>(base + off_beta0);
     d.Ea0R = reinterpret_cast<const double *>(base + off_Ea0R);
     d.troe = reinterpret_cast<const double *>(base + off_troe);
-    d.tb_row = reinterpret_cast<const int *>(base + off_tb);
     d.eff = reinterpret_cast<const double *>(base + off_eff);
-    d.inc_ptr = reinterpret_cast<const int *>(base + off_incp);
-    d.inc = reinterpret_cast<const int2 *>(base + off_inc);
-    d.dnu = reinterpret_cast<const int *>(base + off_dnu);
     d.counters = reinterpret_cast<unsigned int *>(base + off_cnt);
-    d.nasa_s = reinterpret_cast<const double *>(base + off_nasa_s);
     d.troe_r = reinterpret_cast<const double *>(base + off_troe_r);
     d.rsp = reinterpret_cast<const int *>(base + off_rsp);
-    d.rnu = reinterpret_cast<const int *>(base + off_rnu);
-    d.tb_list = reinterpret_cast<const int *>(base + off_tbl);
+    d.nasa_t = reinterpret_cast<const double *>(base + off_nasa_t);
+    d.dnu_d = reinterpret_cast<const double *>(base + off_dnu);
+    d.rspec = reinterpret_cast<const uint2 *>(base + off_rspec);
+    d.nslot = nslot;
+    d.three = three;
+    d.gath_len = gath_len;
+    d.gath = reinterpret_cast<const unsigned *>(base + off_gath);
+    d.ell_groups = ell_groups;
+    d.ell_off = reinterpret_cast<const int *>(base + off_eo);
+    d.ell_len = reinterpret_cast<const int *>(base + off_el);
+    d.ell_pos = reinterpret_cast<const int *>(base + off_ep);
+    d.ell_f = reinterpret_cast<const unsigned *>(base + off_ef);
+    d.ell_d = reinterpret_cast<const unsigned *>(base + off_ed);
+    d.tbrow_ptr = reinterpret_cast<const int *>(base + off_tp);
+    d.tbrow_f = reinterpret_cast<const unsigned *>(base + off_tf);
+    d.tbrow_d = reinterpret_cast<const unsigned *>(base + off_td);
+    d.eff_f = reinterpret_cast<const float *>(base + off_eff_f);
     d.lnPR = std::log(th[0] / kR);
     *out = m;
     return CHEM_OK;

@@ -6,21 +6,36 @@
 // Design for sm_103a:
 //  - One warp per cell. Cells are popped from a device work queue (one atomic
 //    per cell), so cells with very different step counts balance across the
-//    persistent grid (one block of kWarps warps per resident slot).
-//  - Few cells (at most one per SM, e.g. the learned step's out-of-distribution
-//    cells): a team of the block's kWarps warps integrates each cell. The FP64
-//    pipe is per SM sub-partition, so a lone warp leaves three of them idle.
-//    The team splits the reaction pass (reactions over all 128 lanes) and the
-//    LU trailing updates (rows over warps); the rest runs redundantly in every
-//    warp on identical data, and one warp writes the shared results. Every
-//    value is computed by the same operations in the same order as by a lone
-//    warp, so the results are bitwise those of one warp per cell.
+//    persistent grid.
 //  - The state vector y = (T, Y_1..Y_N) is distributed over the lanes:
-//    component c lives in lane c % 32, register slot c / 32 (N <= 63).
-//  - Species work runs lane-per-species, reaction work lane-per-reaction; the
-//    dense Jacobian and its LU factors (n x n FP64, n = N + 1) live in the
-//    warp's shared-memory slice. The LU is right-looking with partial pivoting;
-//    its rank-1 updates are column-parallel (each lane owns columns c % 32).
+//    component c lives in lane c % 32, register slot c / 32 (n = N + 1 <= 64;
+//    one slot up to n = 32).
+//  - Species work runs lane-per-species, reaction work lane-per-reaction.
+//    Up to n = 32 the LU factors live in registers, lane i holding row i: the
+//    pivot search is a warp reduction, rows are not moved (each lane tracks its
+//    row's position), the pivot row is broadcast by shuffles, and the triangular
+//    solves are one shuffle and one multiply-add per column. Above, the matrix
+//    is factored in the warp's shared-memory slice, columns over lanes.
+//  - What bounds it: FP64 issues one warp instruction per 16 clocks and SM (64
+//    per sub-partition), so the reaction and species passes count FP64
+//    instructions: no integer-to-FP64 conversions (stoichiometric coefficients are
+//    kept as the high half of their FP64 pattern), d q / d C_l from the mass-action
+//    factors directly, several warp sums in one butterfly, T-dependent data in
+//    tables that a warp reads coalesced. The Jacobian's sparse part is summed entry
+//    by entry from lists sorted by length (ELLPACK). The former kernel (row-owner
+//    sums over each species' reactions, the factors in shared memory, 23 KB per warp and
+//    8 warps per SM) took 54,000 warp instructions and 1,600 FP64 ones a step of the
+//    30-species mixed mode, with the FP64 pipe 44 % busy; this one 30,000 and 1,350 at 16
+//    warps per SM (12 KB each), 60 %. 65,536 cells at rtol 1e-2: 148 -> 87 ms; 4,096
+//    cells of the 9-species mechanism in FP64 at rtol 1e-6: 111 -> 76 ms; the 2 % fallback
+//    of 262,144 learned cells: 14.5 -> 9.1 ms.
+//  - Few cells (at most one per SM, e.g. the learned step's out-of-distribution
+//    cells): a team of kWarps warps integrates each cell, one per SM
+//    sub-partition. The reaction pass, the Jacobian's lists and the species' sums
+//    are split over the team, the rest runs redundantly in every warp on identical
+//    data, and one warp writes the shared results. Every value is computed by the
+//    same operations in the same order as by a lone warp, so the results are
+//    bitwise those of one warp per cell.
 //  - Integrator: Rodas3 (Sandu et al. 1997), an embedded L-stable Rosenbrock
 //    method of order 3(2), in the transformed form
 //      (I/(h g) - J) K_i = f(y + sum_j a_ij K_j) + sum_j (c_ij / h) K_j,
@@ -30,6 +45,7 @@
 
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -43,15 +59,35 @@ constexpr double kMixedMinRtol = 1e-5;   // tightest rtol the mixed mode integra
 
 // Rodas3 coefficients (g = 1/2 on the diagonal)
 constexpr double kGam = 0.5;
-constexpr double kA31 = 2.0, kA41 = 2.0, kA43 = 1.0;      // a21 = a32 = a42 = 0
+// a31 = a41 = 2, a43 = 1, the others 0; m = (2, 0, 1, 1), e = (0, 0, 0, 1)
 constexpr double kC21 = 4.0, kC31 = 1.0, kC32 = -1.0, kC41 = 1.0, kC42 = -1.0, kC43 = -8.0 / 3.0;
-// m = (2, 0, 1, 1), e = (0, 0, 0, 1)
 
 __device__ __forceinline__ double warp_sum(double v) {
     // butterfly: every lane ends with the same bits (addition is commutative)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
+}
+// Two (four) sums in one butterfly: the halves (quarters) of the warp carry one sum each, so the FP64
+// pipe sees 5 (6) additions instead of 10 (20). Every lane ends with all of them.
+__device__ __forceinline__ void warp_sum2(double &a, double &b, int lane) {
+    const bool up = lane & 16;
+    double v = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0);
+    b = __shfl_sync(kFull, v, 16);
+}
+__device__ __forceinline__ void warp_sum3(double &a, double &b, double &c, int lane) {
+    const bool up = lane & 16, mid = lane & 8;
+    const double ab = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, 16);
+    const double cc = c + __shfl_xor_sync(kFull, c, 16);
+    double v = (mid ? cc : ab) + __shfl_xor_sync(kFull, mid ? ab : cc, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0);
+    b = __shfl_sync(kFull, v, 16);
+    c = __shfl_sync(kFull, v, 8);
 }
 
 // The warps integrating one cell: W = 1 (a lone warp) or W = kWarps (the block).
@@ -65,46 +101,87 @@ struct Team {
     __device__ __forceinline__ bool lead() const { return W == 1 || wt == 0; }
 };
 
-struct Slice {                 // one warp's shared-memory slice
-    double *G;                 // [n][n] Jacobian, then its LU factors
-    double *bsw;               // [n] permutation buffer
-    double *invd;              // [n] reciprocal diagonal of U
-    double *C, *HRT, *SR, *cpR, *wdot, *wT, *JCC, *U, *V;   // [N]
-    double *rq, *rdqT, *rc3;   // [R] rate of progress, d q / dT, third-body coefficient
-    double *rdq;               // [R][6] d q / d C_l for the reaction's distinct species
-    int *piv;                  // [n]
+// One warp's shared-memory slice. mreal is the type of the matrix and of what only the matrix reads:
+// FP32 in the mixed mode (values cut from FP64 once, when they are stored). BIG (n > 32): the LU
+// factors live in shared memory too. Absent species have index N: C = 1, g = H = 0.
+template <bool MX>
+struct Slice {
+    using mreal = typename std::conditional<MX, float, double>::type;
+    double *C, *g, *H;             // [N+1] concentration, S/R - H/RT, H/RT
+    double *rq, *rdqT;             // [R] rate of progress, its derivative to T
+    double *xs;                    // [n] this warp's own vector buffer
+    mreal *G;                      // [n][n] I/(h g) - J
+    mreal *F, *invd;               // [n][n], [n] LU factors, reciprocal pivots (BIG)
+    mreal *cpR, *wdot, *wT, *JCC, *U, *V, *HR;   // [N]
+    mreal *rc3, *rdq;              // [n_tb] third-body coefficient, [R][nslot] d q / d C of its species
+    float *Cf;                     // [N] concentrations in FP32 (mixed mode)
+    int *piv;                      // [n] (BIG)
 };
 
-__host__ __device__ inline size_t slice_doubles(int N, int R) {
-    int n = N + 1;
-    return (size_t)n * n + 2 * (size_t)n + 9 * (size_t)N + 9 * (size_t)R;
-}
-__host__ __device__ inline size_t slice_bytes(int N, int R) {
-    size_t b = slice_doubles(N, R) * sizeof(double) + (size_t)(N + 1) * sizeof(int);
-    return (b + 15) & ~size_t(15);
-}
-
-__device__ Slice make_slice(char *base, int N, int R) {
-    Slice s;
-    int n = N + 1;
-    double *d = reinterpret_cast<double *>(base);
-    s.G = d; d += (size_t)n * n;
-    s.bsw = d; d += n;
-    s.invd = d; d += n;
-    s.C = d; d += N; s.HRT = d; d += N; s.SR = d; d += N; s.cpR = d; d += N; s.wdot = d; d += N;
-    s.wT = d; d += N; s.JCC = d; d += N; s.U = d; d += N; s.V = d; d += N;
-    s.rq = d; d += R; s.rdqT = d; d += R; s.rc3 = d; d += R;
-    s.rdq = d; d += 6 * (size_t)R;
-    s.piv = reinterpret_cast<int *>(d);
-    return s;
+// Lays the slice out from `base` (null: only counts) and returns its bytes. Overlaps: in FP64 up to n = 32
+// the matrix (dead once its rows are in registers) shares its space with rq and rdqT (dead when it
+// is built); BIG mixed factors share theirs with rdq (dead when the matrix is built).
+template <bool MX, bool BIG>
+__host__ __device__ inline size_t make_slice(char *base, int N, int R, int n_tb, int nslot, Slice<MX> *s) {
+    using mreal = typename Slice<MX>::mreal;
+    const int n = N + 1;
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        char *p = base + o;
+        o += (bytes + 7) & ~size_t(7);
+        return p;
+    };
+    Slice<MX> t;
+    t.C = reinterpret_cast<double *>(take((size_t)(N + 1) * 8));
+    t.g = reinterpret_cast<double *>(take((size_t)(N + 1) * 8));
+    t.H = reinterpret_cast<double *>(take((size_t)(N + 1) * 8));
+    t.xs = reinterpret_cast<double *>(take((size_t)n * 8));
+    const size_t g_bytes = (size_t)n * n * sizeof(mreal), q_bytes = (size_t)R * 8;
+    if (!MX && !BIG) {
+        char *p = take(g_bytes > 2 * q_bytes ? g_bytes : 2 * q_bytes);
+        t.G = reinterpret_cast<mreal *>(p);
+        t.rq = reinterpret_cast<double *>(p);
+        t.rdqT = t.rq + R;
+    } else {
+        t.rq = reinterpret_cast<double *>(take(q_bytes));
+        t.rdqT = reinterpret_cast<double *>(take(q_bytes));
+        t.G = reinterpret_cast<mreal *>(take(g_bytes));
+    }
+    const size_t d_bytes = (size_t)R * nslot * sizeof(mreal);
+    if (MX && BIG) {
+        char *p = take(g_bytes > d_bytes ? g_bytes : d_bytes);
+        t.F = t.rdq = reinterpret_cast<mreal *>(p);
+    } else {
+        t.rdq = reinterpret_cast<mreal *>(take(d_bytes));
+        t.F = t.G;
+    }
+    t.invd = BIG ? reinterpret_cast<mreal *>(take((size_t)n * sizeof(mreal))) : nullptr;
+    mreal **small[] = {&t.cpR, &t.wdot, &t.wT, &t.JCC, &t.U, &t.V, &t.HR};
+    for (mreal **q : small) *q = reinterpret_cast<mreal *>(take((size_t)N * sizeof(mreal)));
+    t.rc3 = reinterpret_cast<mreal *>(take((size_t)n_tb * sizeof(mreal)));
+    t.Cf = MX ? reinterpret_cast<float *>(take((size_t)N * 4)) : nullptr;
+    t.piv = BIG ? reinterpret_cast<int *>(take((size_t)n * 4)) : nullptr;
+    if (s) *s = t;
+    return (o + 15) & ~size_t(15);
 }
 
 // values of the last right-hand-side evaluation needed by the Jacobian
 struct EvalInfo {
-    double T, invT, rho, invrho, cp, dcpdT, Wbar, Q;
+    double T, invT, rho, cp, dcpdT, Wbar, Q;
 };
 
-__device__ __forceinline__ double sel(const double v[2], int slot) { return slot ? v[1] : v[0]; }
+// the FP64 (FP32) value whose high 16 bits a code word carries
+template <typename real>
+__device__ __forceinline__ real code_value(unsigned w) {
+    if constexpr (sizeof(real) == 4) return __uint_as_float(w & 0xFFFF0000u);
+    else return __hiloint2double((int)(w & 0xFFFF0000u), 0);
+}
+// an FP64 value in the matrix type (FP32: cut on the integer pipe)
+template <typename real>
+__device__ __forceinline__ real rd(double x) {
+    if constexpr (sizeof(real) == 4) return f64_to_f32_trunc(x);
+    else return x;
+}
 
 // Troe blending function F(T, Pr) (Gilbert, Luther and Troe 1983), with
 // glg = d log10 F / d log10 Pr and dF/dT at fixed Pr. tp = (a, 1/T***, 1/T*, T**).
@@ -155,113 +232,123 @@ __device__ void troe_F_f32(const double *tp, float T, float invT, float Prd, flo
 // integer pipe (truncation: relative error below 2^-23 of the argument), exp in FP32
 __device__ __forceinline__ double exp_mx(double x) { return f32_to_f64_int(expf(f64_to_f32_trunc(x))); }
 
-// f = f(y) for the warp's cell. With jac, also stores what build_matrix needs. MX (the mixed
-// mode): the rate constants' exponentials and the fall-off blending in FP32, the rest FP64.
-template <int W, bool MX>
-__device__ EvalInfo eval_rhs(const DevMech &m, const Slice &sh, Team<W> tm, int lane, double p, const double y[2],
-                             double f[2], bool jac) {
+// f = f(y) for the warp's cell. JAC: also what build_matrix needs. MX (the mixed mode): the rate
+// constants' exponentials and the fall-off blending in FP32, the rest FP64.
+template <int W, int NS, bool MX, bool JAC>
+__device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &sh, Team<W> tm, int lane, double p,
+                                             double Rinvp, const double (&y)[NS], double (&f)[NS]) {
+    using mreal = typename Slice<MX>::mreal;
     const int N = m.N, R = m.R, n = N + 1;
     EvalInfo info;
-    f[0] = 0.0;
-    f[1] = 0.0;
     const double T = __shfl_sync(kFull, y[0], 0);
     const double invT = 1.0 / T;
     const double lnT = log(T);
     info.T = T;
     info.invT = invT;
-    const int rng = (T >= m.T_mid) ? 1 : 0;
+    const double *tab = m.nasa_t + (T >= m.T_mid ? 17 * 64 : 0);
     tm.sync();                 // every warp of the team is done reading the previous evaluation
     // species pass: thermo and mixture sums (lane per species; in a team every warp
     // computes them and the first writes the shared copies)
     const bool wr = tm.lead();
     double S = 0.0, cp = 0.0, dcp = 0.0;
-    double yw_s[2] = {0.0, 0.0};
-    for (int s = 0; s < 2; ++s) {
+    double yw_s[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
         const int c = lane + 32 * s;
+        f[s] = 0.0;
+        yw_s[s] = 0.0;
         if (c >= 1 && c < n) {
             const int k = c - 1;
-            const double *a = m.f64.nasa_cp + (size_t)(rng * N + k) * 5;
-            const double *b = m.f64.nasa_h + (size_t)(rng * N + k) * 6;
-            const double *e = m.nasa_s + (size_t)(rng * N + k) * 6;
-            const double a0 = __ldg(a), a1 = __ldg(a + 1), a2 = __ldg(a + 2), a3 = __ldg(a + 3), a4 = __ldg(a + 4);
+            const double *q = tab + k;
+            const double a0 = __ldg(q), a1 = __ldg(q + 64), a2 = __ldg(q + 128), a3 = __ldg(q + 192),
+                         a4 = __ldg(q + 256);
             const double cpR = a0 + T * (a1 + T * (a2 + T * (a3 + T * a4)));
-            const double HRT = __ldg(b) + T * (__ldg(b + 1) + T * (__ldg(b + 2) + T * (__ldg(b + 3) + T * __ldg(b + 4))))
-                               + __ldg(b + 5) * invT;
-            const double SR = __ldg(e) * lnT + T * (__ldg(e + 1) + T * (__ldg(e + 2) + T * (__ldg(e + 3) + T * __ldg(e + 4))))
-                              + __ldg(e + 5);
+            q += 5 * 64;
+            const double HRT = __ldg(q) + T * (__ldg(q + 64) + T * (__ldg(q + 128) + T * (__ldg(q + 192) + T * __ldg(q + 256))))
+                               + __ldg(q + 320) * invT;
+            q += 6 * 64;
+            const double SR = __ldg(q) * lnT + T * (__ldg(q + 64) + T * (__ldg(q + 128) + T * (__ldg(q + 192) + T * __ldg(q + 256))))
+                              + __ldg(q + 320);
             const double yw = y[s] * __ldg(m.f64.invW + k);
             yw_s[s] = yw;
             S += yw;
             cp += yw * cpR;
             if (wr) {
-                sh.HRT[k] = HRT;
-                sh.SR[k] = SR;
-                sh.cpR[k] = cpR;
+                sh.H[k] = HRT;
+                sh.g[k] = SR - HRT;
+                if (JAC) sh.cpR[k] = rd<mreal>(cpR);
             }
-            if (jac) dcp += yw * (a1 + T * (2.0 * a2 + T * (3.0 * a3 + T * 4.0 * a4)));
+            if (JAC) dcp += yw * (a1 + T * (2.0 * a2 + T * (3.0 * a3 + T * 4.0 * a4)));
         }
     }
-    S = warp_sum(S);
-    cp = warp_sum(cp) * kR;
-    if (jac) dcp = warp_sum(dcp) * kR;
+    if (JAC) warp_sum3(S, cp, dcp, lane);
+    else warp_sum2(S, cp, lane);
+    cp *= kR;
     const double Wbar = 1.0 / S;
     const double rho = p * invT * Wbar * (1.0 / kR);
-    const double invrho = 1.0 / rho;
+    // FP64 mode: 1 / rho without another division. The mixed mode keeps every FP64 rounding as it is
+    // (see the error norm below)
+    const double invrho = MX ? 1.0 / rho : Rinvp * (T * S);
     info.rho = rho;
-    info.invrho = invrho;
     info.cp = cp;
-    info.dcpdT = dcp;
+    info.dcpdT = JAC ? dcp * kR : 0.0;
     info.Wbar = Wbar;
-    // the mixed mode's FP32 concentrations for the third-body sums, in the space of V (written
-    // only by the gather below, after the reaction pass has used them)
-    float *Cf = reinterpret_cast<float *>(sh.V);
-    if (wr)
-        for (int s = 0; s < 2; ++s) {
+    if (wr) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
             const int c = lane + 32 * s;
             if (c >= 1 && c < n) {
-                sh.C[c - 1] = rho * yw_s[s];
-                if (MX) Cf[c - 1] = f64_to_f32_trunc(rho * yw_s[s]);
+                const double C = rho * yw_s[s];
+                sh.C[c - 1] = C;
+                if (MX) sh.Cf[c - 1] = f64_to_f32_trunc(C);
             }
         }
+        if (lane == 0) {                             // the absent species
+            sh.C[N] = 1.0;
+            sh.g[N] = 0.0;
+            sh.H[N] = 0.0;
+        }
+    }
     tm.sync();
     // reaction pass (thread per reaction over the team's lanes)
     const double lnPRT = m.lnPR - lnT;
     for (int j = tm.wt * 32 + lane; j < R; j += 32 * W) {
-        const int *re = m.reac + 3 * j;
-        const int *pr = m.prod + 3 * j;
-        const int r0 = __ldg(re), r1 = __ldg(re + 1), r2 = __ldg(re + 2);
-        const int p0 = __ldg(pr), p1 = __ldg(pr + 1), p2 = __ldg(pr + 2);
+        const uint2 sp = __ldg(m.rspec + j);
+        const int r0 = sp.x & 255, r1 = (sp.x >> 8) & 255, p0 = sp.y & 255, p1 = (sp.y >> 8) & 255;
         const double beta = __ldg(m.beta + j), EaR = __ldg(m.EaR + j);
         const double lnkf = __ldg(m.lnA + j) + beta * lnT - EaR * invT;
         const double kf = MX ? exp_mx(lnkf) : exp(lnkf);
-        double lnKp = 0.0, dH = 0.0;
-        if (p0 >= 0) { lnKp += sh.SR[p0] - sh.HRT[p0]; dH += sh.HRT[p0]; }
-        if (r0 >= 0) { lnKp -= sh.SR[r0] - sh.HRT[r0]; dH -= sh.HRT[r0]; }
-        if (p1 >= 0) { lnKp += sh.SR[p1] - sh.HRT[p1]; dH += sh.HRT[p1]; }
-        if (r1 >= 0) { lnKp -= sh.SR[r1] - sh.HRT[r1]; dH -= sh.HRT[r1]; }
-        if (p2 >= 0) { lnKp += sh.SR[p2] - sh.HRT[p2]; dH += sh.HRT[p2]; }
-        if (r2 >= 0) { lnKp -= sh.SR[r2] - sh.HRT[r2]; dH -= sh.HRT[r2]; }
-        const double dnu = (double)__ldg(m.dnu + j);
+        double lnKp = sh.g[p0] - sh.g[r0];
+        lnKp += sh.g[p1];
+        lnKp -= sh.g[r1];
+        double C0 = sh.C[r0], C1 = sh.C[r1], D0 = sh.C[p0], D1 = sh.C[p1];
+        double Pf = C0 * C1, Pr = D0 * D1, C2 = 1.0, D2 = 1.0;
+        const int r2 = (sp.x >> 16) & 255, p2 = (sp.y >> 16) & 255;
+        if (m.three) {
+            C2 = sh.C[r2];
+            D2 = sh.C[p2];
+            lnKp += sh.g[p2];
+            lnKp -= sh.g[r2];
+            Pf *= C2;
+            Pr *= D2;
+        }
+        const double dnu = __ldg(m.dnu_d + j);
         // k_r = k_f / K_c, ln K_c = ln K_p + dnu ln(P_std / RT)
         const double kr = MX ? exp_mx(lnkf - lnKp - dnu * lnPRT) : exp(lnkf - lnKp - dnu * lnPRT);
-        double Pf = 1.0, Pr = 1.0;
-        if (r0 >= 0) Pf *= sh.C[r0];
-        if (r1 >= 0) Pf *= sh.C[r1];
-        if (r2 >= 0) Pf *= sh.C[r2];
-        if (p0 >= 0) Pr *= sh.C[p0];
-        if (p1 >= 0) Pr *= sh.C[p1];
-        if (p2 >= 0) Pr *= sh.C[p2];
         const int type = __ldg(m.rtype + j);
         const double dlnkf = (beta + EaR * invT) * invT;
         double F = 1.0, dFdC = 0.0, dFdT = 0.0;
         if (type != 0) {
-            const double *e = m.eff + (size_t)__ldg(m.tb_row + j) * N;
             double M = 0.0;
             if (MX) {
+                const float *e = m.eff_f + (size_t)j * N;
                 float Mf = 0.0f;
-                for (int k = 0; k < N; ++k) Mf = fmaf(f64_to_f32_trunc(__ldg(e + k)), Cf[k], Mf);
+#pragma unroll 8
+                for (int k = 0; k < N; ++k) Mf = fmaf(__ldg(e + k), sh.Cf[k], Mf);
                 M = f32_to_f64_int(Mf);
             } else {
+                const double *e = m.eff + (size_t)j * N;
+#pragma unroll 8
                 for (int k = 0; k < N; ++k) M += __ldg(e + k) * sh.C[k];
             }
             if (type == 1) {
@@ -286,185 +373,336 @@ __device__ EvalInfo eval_rhs(const DevMech &m, const Slice &sh, Team<W> tm, int 
                 }
                 const double ip = 1.0 / (1.0 + Prd);
                 const double blend = Prd * ip;
-                const double dF_dPrd = Ft * ip * (ip + glg);
                 F = blend * Ft;
-                dFdC = dF_dPrd * ratio;
-                const double dlnk0 = (beta0 + Ea0R * invT) * invT;
-                dFdT = dF_dPrd * Prd * (dlnk0 - dlnkf) + blend * dFtdT;
+                if (JAC) {
+                    const double dF_dPrd = Ft * ip * (ip + glg);
+                    dFdC = dF_dPrd * ratio;
+                    const double dlnk0 = (beta0 + Ea0R * invT) * invT;
+                    dFdT = dF_dPrd * Prd * (dlnk0 - dlnkf) + blend * dFtdT;
+                }
             }
         }
-        const double rop = kf * Pf - kr * Pr;
-        sh.rq[j] = F * rop;
-        if (jac) {
+        const double rop = fma(kf, Pf, -__dmul_rn(kr, Pr));
+        double q = rop;
+        if (type != 0) q = F * rop;
+        sh.rq[j] = q;
+        if (JAC) {
+            double dH = sh.H[p0] - sh.H[r0];
+            dH += sh.H[p1];
+            dH -= sh.H[r1];
+            if (m.three) {
+                dH += sh.H[p2];
+                dH -= sh.H[r2];
+            }
             const double dlnKc = (dH - dnu) * invT;
-            const double dkfdT = kf * dlnkf;
-            const double dkrdT = kr * (dlnkf - dlnKc);
-            sh.rdqT[j] = F * (dkfdT * Pf - dkrdT * Pr) + rop * dFdT;
-            sh.rc3[j] = (type != 0) ? rop * dFdC : 0.0;
+            const double dkfdT = kf * dlnkf, dkrdT = kr * (dlnkf - dlnKc);
+            double dq = dkfdT * Pf - dkrdT * Pr;
+            if (type != 0) {
+                dq = F * dq + rop * dFdT;
+                sh.rc3[j] = rd<mreal>(rop * dFdC);
+            }
+            sh.rdqT[j] = dq;
             // d q / d C_l through the mass-action products, for the distinct species l
-            for (int u = 0; u < 6; ++u) {
-                const int l = __ldg(m.rsp + 6 * j + u);
-                if (l < 0) break;
-                double dPf = 0.0, dPr = 0.0;
-                if (r0 == l) dPf += (r1 >= 0 ? sh.C[r1] : 1.0) * (r2 >= 0 ? sh.C[r2] : 1.0);
-                if (r1 == l) dPf += (r0 >= 0 ? sh.C[r0] : 1.0) * (r2 >= 0 ? sh.C[r2] : 1.0);
-                if (r2 == l) dPf += (r0 >= 0 ? sh.C[r0] : 1.0) * (r1 >= 0 ? sh.C[r1] : 1.0);
-                if (p0 == l) dPr += (p1 >= 0 ? sh.C[p1] : 1.0) * (p2 >= 0 ? sh.C[p2] : 1.0);
-                if (p1 == l) dPr += (p0 >= 0 ? sh.C[p0] : 1.0) * (p2 >= 0 ? sh.C[p2] : 1.0);
-                if (p2 == l) dPr += (p0 >= 0 ? sh.C[p0] : 1.0) * (p1 >= 0 ? sh.C[p1] : 1.0);
-                sh.rdq[6 * j + u] = F * (kf * dPf - kr * dPr);
+            mreal *o = sh.rdq + (size_t)j * m.nslot;
+            auto put = [&](int u, double d) { o[u] = rd<mreal>(type != 0 ? F * d : d); };
+            if (sp.x >> 24) {                        // every species once, in slot order
+                put(0, kf * (m.three ? C1 * C2 : C1));
+                int u = 1;
+                if (r1 < N) put(u++, kf * (m.three ? C0 * C2 : C0));
+                if (m.three && r2 < N) put(u++, kf * (C0 * C1));
+                if (p0 < N) put(u++, -(kr * (m.three ? D1 * D2 : D1)));
+                if (p1 < N) put(u++, -(kr * (m.three ? D0 * D2 : D0)));
+                if (m.three && p2 < N) put(u++, -(kr * (D0 * D1)));
+            } else {
+                for (int u = 0; u < 6; ++u) {
+                    const int l = __ldg(m.rsp + 6 * j + u);
+                    if (l < 0) break;
+                    double dPf = 0.0, dPr = 0.0;
+                    if (r0 == l) dPf += C1 * C2;
+                    if (r1 == l) dPf += C0 * C2;
+                    if (r2 == l) dPf += C0 * C1;
+                    if (p0 == l) dPr += D1 * D2;
+                    if (p1 == l) dPr += D0 * D2;
+                    if (p2 == l) dPr += D0 * D1;
+                    put(u, kf * dPf - kr * dPr);
+                }
             }
         }
     }
     tm.sync();
     // species gather: wdot_k = sum_j nu_kj q_j (reactions ascending)
+    double w[NS], wt[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const unsigned *lst = m.gath + lane + 32 * s - 1;    // species c - 1
+        const bool on = lane + 32 * s >= 1 && lane + 32 * s < n;
+        w[s] = 0.0;
+        wt[s] = 0.0;
+        if (on)
+            for (int t = 0; t < m.gath_len; t += 4) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned e = __ldg(lst + (t + u) * 64);
+                    const double nu = code_value<double>(e);
+                    w[s] += nu * sh.rq[e & 0xFFFFu];
+                    if (JAC) wt[s] += nu * sh.rdqT[e & 0xFFFFu];
+                }
+            }
+    }
     double Q = 0.0;
     const double RT = kR * T;
-    for (int s = 0; s < 2; ++s) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
         const int c = lane + 32 * s;
         if (c >= 1 && c < n) {
             const int k = c - 1;
-            double w = 0.0, wt = 0.0;
-            const int b = __ldg(m.inc_ptr + k), e = __ldg(m.inc_ptr + k + 1);
-            for (int t = b; t < e; ++t) {
-                const int2 ent = __ldg(m.inc + t);
-                w += (double)ent.y * sh.rq[ent.x];
-                if (jac) wt += (double)ent.y * sh.rdqT[ent.x];
-            }
             const double Wk = __ldg(m.W + k);
-            if (jac && wr) {
-                sh.wdot[k] = w;
-                sh.wT[k] = wt;
-                sh.U[k] = Wk * invrho;
-                sh.V[k] = Wk * w * Wbar * invrho;
+            const double H = sh.H[k];
+            if (JAC && wr) {
+                sh.wdot[k] = rd<mreal>(w[s]);
+                sh.wT[k] = rd<mreal>(wt[s]);
+                sh.U[k] = rd<mreal>(Wk * invrho);
+                sh.V[k] = rd<mreal>(Wk * w[s] * Wbar * invrho);
+                sh.HR[k] = rd<mreal>(H) * ((mreal)kR * rd<mreal>(T));
             }
-            f[s] = Wk * w * invrho;
-            Q += sh.HRT[k] * RT * w;
+            f[s] = Wk * w[s] * invrho;
+            Q += H * RT * w[s];
         }
     }
     Q = warp_sum(Q);
     info.Q = Q;
-    if (lane == 0) f[0] = -Q / (rho * cp);
+    if (lane == 0) f[0] = MX ? -Q / (rho * cp) : -(Q * invrho) / cp;
     return info;
 }
 
-// shared-memory FP64 value in the working type of the matrix assembly (FP32: by truncation on
-// the integer pipe)
-template <typename real>
-__device__ __forceinline__ real rd(double x) {
-    if constexpr (sizeof(real) == 4) return f64_to_f32_trunc(x);
-    else return x;
-}
+// a b + c d and a b - c d with the first product rounded; FP32 written out, so that the mixed mode's
+// results do not depend on how the compiler contracts sums of two products (a last-bit change of the
+// matrix moves T by up to 1e-8 relative in a step)
+__device__ __forceinline__ float mul_add(float a, float b, float c, float d) { return fmaf(c, d, __fmul_rn(a, b)); }
+__device__ __forceinline__ double mul_add(double a, double b, double c, double d) { return a * b + c * d; }
+__device__ __forceinline__ float mul_sub(float a, float b, float c, float d) { return fmaf(-c, d, __fmul_rn(a, b)); }
+__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) { return a * b - c * d; }
 
-// G = I/(h g) - J from the data of eval_rhs(..., jac = true), built by one warp into Gm (the FP64
-// matrix sh.G, or in the mixed mode its FP32 counterpart in the same space: the Jacobian then
-// carries FP32 rounding, about 1e-7 relative, which the mixed mode's loose tolerances absorb).
-template <typename real>
-__device__ void build_matrix_warp(const DevMech &m, const Slice &sh, real *G, int lane, const EvalInfo &in, double h) {
+// G = I/(h g) - J from the data of eval_rhs<JAC> (the FP64 matrix, or in the mixed mode an FP32 one:
+// the Jacobian then carries FP32 rounding, about 1e-7 relative, which the mixed mode's loose
+// tolerances absorb). In a team the entry lists and the third-body rows are split over the warps and
+// the first warp does the rest.
+template <int W, int NS, bool MX>
+__device__ void build_matrix(const DevMech &m, const Slice<MX> &sh, Team<W> tm, int lane, const EvalInfo &in, double ih) {
+    using real = typename Slice<MX>::mreal;
     const int N = m.N, n = N + 1;
-    for (int s = 0; s < 2; ++s) {            // zero the species block (column owners)
-        const int c = lane + 32 * s;
-        if (c >= 1 && c < n)
-            for (int r = 1; r < n; ++r) G[r * n + c] = 0;
+    real *G = sh.G;
+    if (!MX) tm.sync();                      // FP64: the matrix may share its space with the rates read above
+    for (int r = 1 + tm.wt; r < n; r += W) { // zero the species block
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            if (lane + 32 * s < n) G[r * n + lane + 32 * s] = 0;
     }
-    __syncwarp();
-    // sparse part of JC = d wdot / d C: row owners gather their reactions (ascending)
-    for (int s = 0; s < 2; ++s) {
-        const int c = lane + 32 * s;
-        if (c >= 1 && c < n) {
-            const int k = c - 1;
-            real *row = G + (size_t)c * n + 1;
-            const int b = __ldg(m.inc_ptr + k), e = __ldg(m.inc_ptr + k + 1);
-            for (int t = b; t < e; ++t) {
-                const int2 ent = __ldg(m.inc + t);
-                const real nu = (real)ent.y;
-                for (int u = 0; u < 6; ++u) {
-                    const int l = __ldg(m.rsp + 6 * ent.x + u);
-                    if (l < 0) break;
-                    row[l] += nu * rd<real>(sh.rdq[6 * ent.x + u]);
+    tm.sync();
+    // sparse part of JC = d wdot / d C: an entry per lane, its reactions ascending
+    const unsigned *ell = MX ? m.ell_f : m.ell_d;
+    for (int q = tm.wt; q < m.ell_groups; q += W) {
+        const int pos = __ldg(m.ell_pos + 32 * q + lane), len = __ldg(m.ell_len + q);
+        const unsigned *p = ell + __ldg(m.ell_off + q) + lane;
+        real acc = 0;
+        for (int t = 0; t < len; ++t) {
+            const unsigned e = __ldg(p + 32 * t);
+            if (e >> 16) acc += code_value<real>(e) * sh.rdq[e & 0xFFFFu];
+        }
+        if (pos >= 0) G[pos] = acc;
+    }
+    tm.sync();
+    // dense third-body part: row k takes nu_kj (rop dF/dM)_j eff_j of its reactions j, columns over lanes
+    if (m.n_tb > 0) {
+        const unsigned *tbc = MX ? m.tbrow_f : m.tbrow_d;
+        for (int k = tm.wt; k < N; k += W) {
+            const int b = __ldg(m.tbrow_ptr + k), e = __ldg(m.tbrow_ptr + k + 1);
+            if (b == e) continue;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                const int c = lane + 32 * s;
+                if (c >= 1 && c < n) {
+                    real acc = G[(1 + k) * n + c];
+                    for (int t = b; t < e; ++t) {
+                        const unsigned w = __ldg(tbc + t);
+                        const int j = w & 0xFFFFu;
+                        real ef;
+                        if constexpr (MX) ef = __ldg(m.eff_f + (size_t)j * N + c - 1);
+                        else ef = __ldg(m.eff + (size_t)j * N + c - 1);
+                        acc += code_value<real>(w) * (sh.rc3[j] * ef);
+                    }
+                    G[(1 + k) * n + c] = acc;
                 }
             }
         }
+        tm.sync();
     }
-    __syncwarp();
-    // dense third-body part: rank-1 terms nu_j (rop dF/dM) eff_j (column owners)
-    for (int t = 0; t < m.n_tb; ++t) {
-        const int j = __ldg(m.tb_list + t);
-        const real c3 = rd<real>(sh.rc3[j]);
-        const double *e = m.eff + (size_t)__ldg(m.tb_row + j) * N;
-        for (int s = 0; s < 2; ++s) {
+    if (tm.lead()) {
+        // JCC[k] = sum_l JC[k][l] C_l (row owners)
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
             const int c = lane + 32 * s;
             if (c >= 1 && c < n) {
-                const real v = c3 * rd<real>(__ldg(e + c - 1));
-                for (int u = 0; u < 6; ++u) {
-                    const int k = __ldg(m.rsp + 6 * j + u);
-                    if (k < 0) break;
-                    G[(1 + k) * n + c] += (real)__ldg(m.rnu + 6 * j + u) * v;
+                real acc = 0;
+                for (int l = 0; l < N; ++l) {
+                    real C;
+                    if constexpr (MX) C = sh.Cf[l];
+                    else C = sh.C[l];
+                    acc += G[c * n + 1 + l] * C;
                 }
+                sh.JCC[c - 1] = acc;
             }
         }
-    }
-    __syncwarp();
-    // JCC[k] = sum_l JC[k][l] C_l (row owners)
-    for (int s = 0; s < 2; ++s) {
-        const int c = lane + 32 * s;
-        if (c >= 1 && c < n) {
-            real acc = 0;
-            for (int l = 0; l < N; ++l) acc += G[c * n + 1 + l] * rd<real>(sh.C[l]);
-            sh.JCC[c - 1] = (double)acc;
-        }
-    }
-    __syncwarp();
-    // chain rule through C(T, Y) and rho(T, Y); then G = I/(h g) - J
-    const real T = rd<real>(in.T), invT = rd<real>(in.invT), cp = rd<real>(in.cp), Wbar = rd<real>(in.Wbar);
-    const real Q = rd<real>(in.Q), rho = rd<real>(in.rho), dcpdT = rd<real>(in.dcpdT);
-    const real invrcp = (real)1 / (rho * cp);
-    const real qq = Q * invrcp / cp;              // Q / (rho cp^2)
-    const real Rr = (real)kR;
-    const real RT = Rr * T;
-    const real ghinv = rd<real>(1.0 / (h * kGam));
-    real sT = 0;
-    for (int s = 0; s < 2; ++s) {
-        const int c = lane + 32 * s;
-        if (c < 1 || c >= n) continue;
-        // species column c (column owner)
-        const int mm = c - 1;
-        const real iWm = rd<real>(__ldg(m.f64.invW + mm));
-        const real a = rho * iWm, b = Wbar * iWm;
-        real sTr = 0;
-        for (int k = 0; k < N; ++k) {
-            real *g = G + (size_t)(1 + k) * n + c;
-            const real dw = *g * a - b * rd<real>(sh.JCC[k]);
-            sTr += rd<real>(sh.HRT[k]) * RT * dw;
-            const real J = rd<real>(sh.U[k]) * dw + rd<real>(sh.V[k]) * iWm;
-            *g = (1 + k == c) ? ghinv - J : -J;
-        }
-        G[c] = sTr * invrcp + qq * (cp * Wbar - rd<real>(sh.cpR[mm]) * Rr) * iWm;   // -J[0][c]
-        // temperature column entry of row c (row owner)
-        const real dwdT = rd<real>(sh.wT[mm]) - rd<real>(sh.JCC[mm]) * invT;
-        const real Um = rd<real>(sh.U[mm]), wm = rd<real>(sh.wdot[mm]);
-        G[(size_t)c * n] = -(Um * dwdT + Um * wm * invT);
-        sT += rd<real>(sh.cpR[mm]) * Rr * wm + rd<real>(sh.HRT[mm]) * RT * dwdT;
-    }
+        __syncwarp();
+        // chain rule through C(T, Y) and rho(T, Y); then G = I/(h g) - J
+        const real invT = rd<real>(in.invT), cp = rd<real>(in.cp), Wbar = rd<real>(in.Wbar);
+        const real Q = rd<real>(in.Q), rho = rd<real>(in.rho), dcpdT = rd<real>(in.dcpdT);
+        const real invrcp = (real)1 / (rho * cp);
+        const real qq = Q * invrcp / cp;              // Q / (rho cp^2)
+        const real Rr = (real)kR;
+        const real ghinv = rd<real>(ih * (1.0 / kGam));         // 1 / (h g), g a power of two
+        real sT = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sT += __shfl_xor_sync(kFull, sT, o);
-    if (lane == 0) G[0] = ghinv + sT * invrcp + qq * (cp * invT - dcpdT);
-    __syncwarp();
-}
-
-template <int W, typename real>
-__device__ void build_matrix(const DevMech &m, const Slice &sh, real *G, Team<W> tm, int lane, const EvalInfo &in,
-                             double h) {
-    if (tm.lead()) build_matrix_warp<real>(m, sh, G, lane, in, h);
+        for (int s = 0; s < NS; ++s) {
+            const int c = lane + 32 * s;
+            if (c < 1 || c >= n) continue;
+            // species column c (column owner)
+            const int mm = c - 1;
+            const real iWm = rd<real>(__ldg(m.f64.invW + mm));
+            const real a = rho * iWm, b = Wbar * iWm;
+            real sTr = 0;
+            for (int k = 0; k < N; ++k) {
+                real *g = G + (size_t)(1 + k) * n + c;
+                const real dw = mul_add(-b, sh.JCC[k], *g, a);
+                sTr += sh.HR[k] * dw;
+                const real J = mul_add(sh.U[k], dw, sh.V[k], iWm);
+                *g = (1 + k == c) ? ghinv - J : -J;
+            }
+            G[c] = mul_add(qq * mul_sub(cp, Wbar, sh.cpR[mm], Rr), iWm, sTr, invrcp);   // -J[0][c]
+            // temperature column entry of row c (row owner)
+            const real dwdT = sh.wT[mm] - sh.JCC[mm] * invT;
+            const real Um = sh.U[mm], wm = sh.wdot[mm];
+            G[(size_t)c * n] = -mul_add(Um * wm, invT, Um, dwdT);
+            sT += mul_add(sh.cpR[mm] * Rr, wm, sh.HR[mm], dwdT);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sT += __shfl_xor_sync(kFull, sT, o);
+        if (lane == 0) G[0] = ghinv + sT * invrcp + qq * (cp * invT - dcpdT);
+    }
     tm.sync();
 }
 
-// In-place LU with partial pivoting of G (FP64, or its FP32 copy in the mixed mode), the
-// reciprocal pivots in invd and the pivot rows in sh.piv; false for a zero or non-finite pivot
-// column. In a team every warp searches the pivot (same data, same choice), the first warp swaps
-// and scales, and the trailing update splits the rows over the warps.
+// The largest of the lanes' non-negative values (FP32 or FP64 patterns compare as integers) among those
+// with `valid`, the smallest `pos` among equals: the lane that holds it, or -1 when it is zero, not
+// finite or none is valid.
+__device__ __forceinline__ int pivot_lane(float v, bool valid, int pos, int lane) {
+    const unsigned key = valid && v == v ? __float_as_uint(v) : 0u;
+    const unsigned top = __reduce_max_sync(kFull, key);
+    if (top == 0u || top >= 0x7F800000u) return -1;
+    const bool cand = valid && key == top;
+    const unsigned first = __reduce_min_sync(kFull, cand ? (unsigned)pos : 64u);
+    return __ffs(__ballot_sync(kFull, cand && (unsigned)pos == first)) - 1;
+}
+__device__ __forceinline__ int pivot_lane(double v, bool valid, int pos, int lane) {
+    valid = valid && v == v;
+    const unsigned hi = valid ? (unsigned)__double2hiint(v) : 0u, lo = (unsigned)__double2loint(v);
+    const unsigned top = __reduce_max_sync(kFull, hi);
+    if (top >= 0x7FF00000u) return -1;
+    const unsigned low = __reduce_max_sync(kFull, valid && hi == top ? lo : 0u);
+    if ((top | low) == 0u) return -1;
+    const bool cand = valid && hi == top && lo == low;
+    const unsigned first = __reduce_min_sync(kFull, cand ? (unsigned)pos : 64u);
+    return __ffs(__ballot_sync(kFull, cand && (unsigned)pos == first)) - 1;
+}
+
+// LU with partial pivoting of an n x n matrix, n <= NC <= 32, in registers: lane i holds row i of the
+// matrix, then (moved once, after the factorisation) the factors' row of its pivoted place i.
+template <typename real, int NC>
+struct RowLU {
+    real row[NC];
+    real rinv;                 // reciprocal pivot of this lane's row
+    int mine;                  // the row of the matrix that this lane's factors come from
+
+    __device__ __forceinline__ bool factor(const real *G, int lane, int n) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) row[c] = (lane < n && c < n) ? G[lane * n + c] : (real)0;
+        int pos = lane;            // place of this lane's row
+        mine = lane;
+        rinv = 0;
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            if (k < n && ok) {
+                const int p = pivot_lane((real)fabs(row[k]), pos >= k && lane < n, pos, lane);
+                if (p < 0) {
+                    ok = false;
+                } else {
+                    const int was = __shfl_sync(kFull, pos, p);
+                    if (pos == k) pos = was;          // the row that stood there takes the pivot's place
+                    if (lane == p) pos = k;
+                    if (lane == k) mine = p;
+                    const real rp = (real)1 / __shfl_sync(kFull, row[k], p);
+                    if (lane == p) rinv = rp;
+                    const bool below = pos > k;
+                    if (below) row[k] *= rp;
+#pragma unroll
+                    for (int cb = (k + 1) & ~3; cb < NC; cb += 4) {
+                        if (cb < n) {
+#pragma unroll
+                            for (int c = cb; c < cb + 4; ++c)
+                                if (c > k) {
+                                    const real akc = __shfl_sync(kFull, row[c], p);
+                                    if (below) row[c] -= row[k] * akc;
+                                }
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < n) row[c] = __shfl_sync(kFull, row[c], mine);
+        rinv = __shfl_sync(kFull, rinv, mine);
+        if constexpr (sizeof(real) == 8) {
+            // FP64: the rows of U divided by their pivots once, instead of each unknown in every solve
+#pragma unroll
+            for (int k = 1; k < NC; ++k)
+                if (lane < k) row[k] *= rinv;
+        }
+        return ok;
+    }
+
+    // x = A^-1 b, component c in lane c
+    __device__ __forceinline__ real solve(real b, int lane, int n) const {
+        b = __shfl_sync(kFull, b, mine);
+#pragma unroll
+        for (int k = 0; k < NC - 1; ++k) {
+            if (k < n - 1) {
+                const real bk = __shfl_sync(kFull, b, k);
+                if (lane > k) b -= row[k] * bk;
+            }
+        }
+        if constexpr (sizeof(real) == 8) b *= rinv;
+#pragma unroll
+        for (int k = NC - 1; k >= 0; --k) {
+            if (k < n) {
+                if constexpr (sizeof(real) == 4) {
+                    if (lane == k) b *= rinv;
+                }
+                const real bk = __shfl_sync(kFull, b, k);
+                if (lane < k) b -= row[k] * bk;
+            }
+        }
+        return b;
+    }
+};
+
+// In-place LU with partial pivoting in shared memory (n > 32), the reciprocal pivots in invd and the
+// pivot rows in sh.piv; false for a zero or non-finite pivot column. In a team every warp searches the
+// pivot (same data, same choice), the first warp swaps and scales, and the trailing update splits
+// the rows over the warps.
 template <int W, typename real>
-__device__ bool lu_factor(const Slice &sh, real *G, real *invd, Team<W> tm, int lane, int n) {
+__device__ bool lu_factor(int *piv, real *G, real *invd, Team<W> tm, int lane, int n) {
     for (int k = 0; k < n; ++k) {
         real best = -1;
         int bi = n;
@@ -483,7 +721,7 @@ __device__ bool lu_factor(const Slice &sh, real *G, real *invd, Team<W> tm, int 
         }
         if (!(best > 0) || !(best < (real)INFINITY) || bi >= n) return false;
         if (tm.lead()) {
-            if (lane == 0) sh.piv[k] = bi;
+            if (lane == 0) piv[k] = bi;
             if (bi != k) {
                 for (int s = 0; s < 2; ++s) {
                     const int c = lane + 32 * s;
@@ -517,11 +755,10 @@ __device__ bool lu_factor(const Slice &sh, real *G, real *invd, Team<W> tm, int 
     return true;
 }
 
-// b <- G^-1 b with the stored factors G, invd (FP64, or FP32 in the mixed mode); b is
-// lane-distributed. bsw is this warp's own permutation buffer (every warp of a team solves on
-// its own).
+// b <- G^-1 b with the factors G, invd in shared memory (n > 32); b is lane-distributed, bsw this
+// warp's own buffer.
 template <typename real>
-__device__ void tri_solve(const Slice &sh, const real *G, const real *invd, real *bsw, int lane, int n, real b[2]) {
+__device__ void tri_solve(const int *piv, const real *G, const real *invd, real *bsw, int lane, int n, real (&b)[2]) {
     for (int s = 0; s < 2; ++s) {
         const int c = lane + 32 * s;
         if (c < n) bsw[c] = b[s];
@@ -529,7 +766,7 @@ __device__ void tri_solve(const Slice &sh, const real *G, const real *invd, real
     __syncwarp();
     if (lane == 0) {
         for (int k = 0; k < n; ++k) {
-            const int p = sh.piv[k];
+            const int p = piv[k];
             if (p != k) { const real t = bsw[k]; bsw[k] = bsw[p]; bsw[p] = t; }
         }
     }
@@ -559,60 +796,112 @@ __device__ void tri_solve(const Slice &sh, const real *G, const real *invd, real
     __syncwarp();
 }
 
-// b <- G^-1 b with the FP64 factors (the default, FP64 mode)
-__device__ __forceinline__ void lu_solve(const Slice &sh, double *bsw, int lane, int n, double b[2]) {
-    tri_solve<double>(sh, sh.G, sh.invd, bsw, lane, n, b);
+// FP32 -> FP64 of a finite value (subnormals become signed zero). A matrix with an infinity or a NaN has
+// no finite pivot or solution, whatever this makes of it.
+__device__ __forceinline__ double f32_to_f64_finite(float x) {
+    const unsigned b = __float_as_uint(x);
+    const bool zero = (b & 0x7F800000u) == 0u;
+    const unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)((zero ? 0u : hi) | (b & 0x80000000u)), (int)(zero ? 0u : b << 29));
 }
 
-// The mixed mode's stage solve with the FP32 matrix Gc and its FP32 LU factors Gf (both in the
-// space of the FP64 matrix: n^2 floats each): x = Gf^-1 b, then one step of iterative refinement,
-// r = b - Gc x in FP64 arithmetic and x += Gf^-1 r. The correction solves the residual to FP32's
-// relative accuracy, so the refined x carries about cond(G) 2^-24 times that error. The
-// conversions between FP64 and FP32 run on the integer pipe (truncation; magnitudes below
-// 2^-126 become 0).
-__device__ void lu_solve_mixed(const Slice &sh, const float *Gf, const float *invdf, const float *Gc, double *bsw,
-                               int lane, int n, double b[2]) {
-    float v[2] = {f64_to_f32_trunc(b[0]), f64_to_f32_trunc(b[1])};
-    tri_solve<float>(sh, Gf, invdf, reinterpret_cast<float *>(bsw), lane, n, v);
-    const double x[2] = {f32_to_f64_int(v[0]), f32_to_f64_int(v[1])};
-    __syncwarp();
-    for (int s = 0; s < 2; ++s) {
-        const int c = lane + 32 * s;
-        if (c < n) bsw[c] = x[s];
-    }
-    __syncwarp();
-    double r[2] = {0.0, 0.0};
-    for (int s = 0; s < 2; ++s) {
-        const int c = lane + 32 * s;
-        if (c < n) {
-            const float *row = Gc + (size_t)c * n;
-            double acc = b[s];
-            for (int j = 0; j < n; ++j) acc = fma(-f32_to_f64_int(row[j]), bsw[j], acc);
-            r[s] = acc;
+// The factored system of one step: NC <= 32 in registers, NC = 64 in shared memory.
+template <int W, int NC, bool MX>
+struct Factors {
+    using real = typename Slice<MX>::mreal;
+    static constexpr bool kBig = NC > 32;
+    typename std::conditional<kBig, int, RowLU<real, kBig ? 4 : NC>>::type lu;
+
+    __device__ __forceinline__ bool factor(const Slice<MX> &sh, Team<W> tm, int lane, int n) {
+        if constexpr (kBig) {
+            if (MX) {                        // the matrix is kept for the refinement; its factors take rdq's space
+                for (int r = tm.wt; r < n; r += W)
+                    for (int c = lane; c < n; c += 32) sh.F[r * n + c] = sh.G[r * n + c];
+                tm.sync();
+            }
+            return lu_factor<W, real>(sh.piv, sh.F, sh.invd, tm, lane, n);
+        } else {
+            return lu.factor(sh.G, lane, n);
         }
     }
-    __syncwarp();
-    float w[2] = {f64_to_f32_trunc(r[0]), f64_to_f32_trunc(r[1])};
-    tri_solve<float>(sh, Gf, invdf, reinterpret_cast<float *>(bsw), lane, n, w);
-    for (int s = 0; s < 2; ++s) b[s] = x[s] + f32_to_f64_int(w[s]);
-}
+    template <int NS>
+    __device__ __forceinline__ void tri(const Slice<MX> &sh, real *buf, int lane, int n, real (&v)[NS]) const {
+        if constexpr (kBig) tri_solve<real>(sh.piv, sh.F, sh.invd, buf, lane, n, v);
+        else v[0] = lu.solve(v[0], lane, n);
+    }
+    // b <- A^-1 b. The mixed mode: x = Gf^-1 b with the FP32 factors, then one step of iterative
+    // refinement, r = b - G x in FP64 arithmetic and x += Gf^-1 r. The correction solves the residual to
+    // FP32's relative accuracy, so the refined x carries about cond(G) 2^-24 times that error. The
+    // conversions between FP64 and FP32 run on the integer pipe (truncation; magnitudes below 2^-126
+    // become 0).
+    template <int NS>
+    __device__ __forceinline__ void solve(const Slice<MX> &sh, double *xs, int lane, int n, double (&b)[NS]) const {
+        if constexpr (!MX) {
+            tri(sh, xs, lane, n, b);
+        } else {
+            double x[NS];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) x[s] = 0.0;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                float v[NS];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) v[s] = f64_to_f32_trunc(b[s]);
+                tri(sh, reinterpret_cast<float *>(xs), lane, n, v);
+                if (pass == 1) {
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) b[s] = x[s] + f32_to_f64_int(v[s]);
+                    break;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    const int c = lane + 32 * s;
+                    x[s] = f32_to_f64_int(v[s]);
+                    if (c < n) xs[c] = x[s];
+                }
+                __syncwarp();
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    const int c = lane + 32 * s;
+                    if (c < n) {
+                        const float *row = sh.G + (size_t)c * n;
+                        double acc = b[s];
+#pragma unroll 4
+                        for (int j = 0; j < n; ++j) acc = fma(-f32_to_f64_finite(row[j]), xs[j], acc);
+                        b[s] = acc;
+                    } else {
+                        b[s] = 0.0;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+};
 
 // Integrates cells popped from the work queue until it is exhausted; W warps per cell. MX: the
 // mixed mode (FP32 rate exponentials and fall-off blending; FP32 LU with one FP64 refinement).
-template <int W, bool MX>
-__device__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int64_t limit, int64_t ld, double dt,
-                                const chem_ode_opts &o, double *__restrict__ Tg, const double *__restrict__ pg,
-                                double *__restrict__ Yg, int32_t *__restrict__ status,
-                                int32_t *__restrict__ nsteps_out, unsigned int *__restrict__ queue,
-                                const int32_t *__restrict__ list, int ok_status) {
+template <int W, int NC, bool MX>
+__device__ __forceinline__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int64_t limit, int64_t ld,
+                                                double dt, const chem_ode_opts &o, double *__restrict__ Tg,
+                                                const double *__restrict__ pg, double *__restrict__ Yg,
+                                                int32_t *__restrict__ status, int32_t *__restrict__ nsteps_out,
+                                                unsigned int *__restrict__ queue, const int32_t *__restrict__ list,
+                                                int ok_status) {
+    constexpr int NS = NC > 32 ? 2 : 1;
+    constexpr bool BIG = NC > 32;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int N = m.N, n = N + 1;
-    const size_t sb = slice_bytes(N, m.R);
+    const size_t sb = make_slice<MX, BIG>(nullptr, N, m.R, m.n_tb, m.nslot, nullptr);
     Team<W> tm{W == 1 ? 0 : warp};
-    // the team's shared data live in its first warp's slice; every warp keeps its own permutation buffer
-    Slice sh = make_slice(smem + (size_t)(W == 1 ? warp : 0) * sb, N, m.R);
-    double *bsw = make_slice(smem + (size_t)warp * sb, N, m.R).bsw;
+    // the team's shared data live in its first warp's slice; every warp keeps its own vector buffer
+    Slice<MX> sh, own;
+    make_slice<MX, BIG>(smem + (size_t)(W == 1 ? warp : 0) * sb, N, m.R, m.n_tb, m.nslot, &sh);
+    make_slice<MX, BIG>(smem + (size_t)warp * sb, N, m.R, m.n_tb, m.nslot, &own);
+    double *xs = own.xs;
+    const double rn = 1.0 / (double)n;
     for (;;) {
         unsigned int pos = 0;
         if (W == 1) {
@@ -622,17 +911,17 @@ __device__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int6
             if (tm.lead() && lane == 0) *blk_pos = (int)atomicAdd(queue, 1u);
             tm.sync();
             pos = (unsigned int)*blk_pos;
-            // the next write of *blk_pos comes after this cell's evaluations, whose barriers
-            // order it after every warp's read above
+            tm.sync();                       // every warp has its ticket before the next one is drawn
         }
         if ((int64_t)pos >= limit) break;
         const int64_t cell = list ? (int64_t)list[pos] : (int64_t)pos;
-        double y[2], yn[2], f0[2], K1[2], K2[2], K3[2], K4[2], ys[2], fs[2];
-        for (int s = 0; s < 2; ++s) {
-            int c = lane + 32 * s;
+        double y[NS], f0[NS], K1[NS], K2[NS], K3[NS], K4[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const int c = lane + 32 * s;
             y[s] = (c == 0) ? Tg[cell] : (c < n ? Yg[(int64_t)(c - 1) * ld + cell] : 0.0);
         }
-        const double p = pg[cell];
+        const double p = pg[cell], Rinvp = kR / p;
         double t = 0.0, h = (o.h0 < dt) ? o.h0 : dt;
         int nst = 0, rejected_last = 0, stat = CHEM_CELL_OK;
         while (t < dt) {
@@ -641,103 +930,92 @@ __device__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int6
             const double rem = dt - t;
             bool last = false;
             if (h >= rem) { h = rem; last = true; }
-            EvalInfo info = eval_rhs<W, MX>(m, sh, tm, lane, p, y, f0, true);
+            const EvalInfo info = eval_rhs<W, NS, MX, true>(m, sh, tm, lane, p, Rinvp, y, f0);
             bool bad = false;
-            for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
                 if (lane + 32 * s < n && !isfinite(f0[s])) bad = true;
             if (__any_sync(kFull, bad)) { stat = CHEM_CELL_NONFINITE; break; }
-            // the mixed mode assembles an FP32 matrix Gc and factors its copy Gf, both in the space
-            // of the FP64 matrix
-            float *Gc = reinterpret_cast<float *>(sh.G);
-            float *Gf = Gc + n * n;
-            float *invdf = reinterpret_cast<float *>(sh.invd);
-            bool factored;
-            if (MX) {
-                build_matrix<W, float>(m, sh, Gc, tm, lane, info, h);
-                ++nst;
-                if (tm.lead()) {
-                    for (int s = 0; s < 2; ++s) {
-                        const int c = lane + 32 * s;
-                        if (c < n)
-                            for (int r = 0; r < n; ++r) Gf[r * n + c] = Gc[r * n + c];
+            const double ih = 1.0 / h;
+            build_matrix<W, NS, MX>(m, sh, tm, lane, info, ih);
+            ++nst;
+            Factors<W, NC, MX> A;
+            if (!A.factor(sh, tm, lane, n)) { h *= 0.2; rejected_last = 1; continue; }
+#pragma unroll
+            for (int s = 0; s < NS; ++s) K1[s] = K2[s] = K3[s] = K4[s] = 0.0;
+            // stages 1 .. 4 in one body: the stage points are y, y, y + 2 K1, y + 2 K1 + K3
+#pragma unroll 1
+            for (int st = 0; st < 4; ++st) {
+                double v[NS];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) v[s] = f0[s];
+                if (st >= 2) {
+                    double ys[NS];
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) ys[s] = y[s] + 2.0 * K1[s] + K3[s];
+                    eval_rhs<W, NS, MX, false>(m, sh, tm, lane, p, Rinvp, ys, v);
+                }
+                if (st >= 1) {
+                    const double c1 = (st == 1 ? kC21 : (st == 2 ? kC31 : kC41)) * ih;
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) v[s] += c1 * K1[s];
+                }
+                if (st >= 2) {
+                    const double c2 = (st == 2 ? kC32 : kC42) * ih, c3 = (st == 3 ? kC43 : 0.0) * ih;
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        v[s] += c2 * K2[s];
+                        v[s] += c3 * K3[s];
                     }
                 }
-                tm.sync();
-                factored = lu_factor<W, float>(sh, Gf, invdf, tm, lane, n);
-            } else {
-                build_matrix<W, double>(m, sh, sh.G, tm, lane, info, h);
-                ++nst;
-                factored = lu_factor<W, double>(sh, sh.G, sh.invd, tm, lane, n);
+                A.solve(sh, xs, lane, n, v);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    if (st == 0) K1[s] = v[s];
+                    else if (st == 1) K2[s] = v[s];
+                    else if (st == 2) K3[s] = v[s];
+                    else K4[s] = v[s];
+                }
             }
-            if (!factored) { h *= 0.2; rejected_last = 1; continue; }
-            auto solve = [&](double b[2]) {
-                if (MX) lu_solve_mixed(sh, Gf, invdf, Gc, bsw, lane, n, b);
-                else lu_solve(sh, bsw, lane, n, b);
-            };
-            const double ih = 1.0 / h;
-            // stage 1
-            for (int s = 0; s < 2; ++s) K1[s] = f0[s];
-            solve(K1);
-            // stage 2: the stage point is y itself (a21 = 0)
-            for (int s = 0; s < 2; ++s) K2[s] = f0[s] + (kC21 * ih) * K1[s];
-            solve(K2);
-            // stage 3: y + 2 K1
-            for (int s = 0; s < 2; ++s) ys[s] = y[s] + kA31 * K1[s];
-            eval_rhs<W, MX>(m, sh, tm, lane, p, ys, fs, false);
-            for (int s = 0; s < 2; ++s) {
-                double v = fs[s];
-                v += (kC31 * ih) * K1[s];
-                v += (kC32 * ih) * K2[s];
-                K3[s] = v;
-            }
-            solve(K3);
-            // stage 4: y + 2 K1 + K3
-            for (int s = 0; s < 2; ++s) ys[s] = y[s] + kA41 * K1[s] + kA43 * K3[s];
-            eval_rhs<W, MX>(m, sh, tm, lane, p, ys, fs, false);
-            for (int s = 0; s < 2; ++s) {
-                double v = fs[s];
-                v += (kC41 * ih) * K1[s];
-                v += (kC42 * ih) * K2[s];
-                v += (kC43 * ih) * K3[s];
-                K4[s] = v;
-            }
-            solve(K4);
             // y_new = y + 2 K1 + K3 + K4, error = K4
-            double acc = 0.0;
+            double acc = 0.0, yn[NS];
             bool nonfinite = false;
-            for (int s = 0; s < 2; ++s) {
-                int c = lane + 32 * s;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                const int c = lane + 32 * s;
+                yn[s] = 0.0;
                 if (c < n) {
                     double v = y[s];
                     v += 2.0 * K1[s];
                     v += K3[s];
                     v += K4[s];
                     yn[s] = v;
-                    double e = K4[s];
-                    double ay = fabs(y[s]), ayn = fabs(v);
-                    double sc = ((c == 0) ? o.atol_T : o.atol_Y) + o.rtol * (ay > ayn ? ay : ayn);
-                    double r = e / sc;
+                    const double e = K4[s];
+                    const double ay = fabs(y[s]), ayn = fabs(v);
+                    const double sc = ((c == 0) ? o.atol_T : o.atol_Y) + o.rtol * (ay > ayn ? ay : ayn);
+                    const double r = e / sc;
                     acc += r * r;
                     if (!isfinite(v) || !isfinite(e)) nonfinite = true;
-                } else {
-                    yn[s] = 0.0;
                 }
             }
             acc = warp_sum(acc);
             nonfinite = __any_sync(kFull, nonfinite);
-            double err = sqrt(acc / (double)n);
+            // The mixed mode's exponentials cut their FP64 arguments to FP32: where a last-bit change of T
+            // or of the step moves an argument across a cut, a rate jumps by 2e-6 and T by up to 6e-8. So
+            // that mode's FP64 operations are never reformulated, only the FP64 mode's.
+            double err = sqrt(MX ? acc / (double)n : acc * rn);
             double fac;
             if (nonfinite || !isfinite(err)) {
                 fac = 0.2;
                 err = 2.0;
             } else {
-                fac = (err > 0.0) ? 0.9 * pow(err, -1.0 / 3.0) : 5.0;
+                fac = (err > 0.0) ? 0.9 * (MX ? pow(err, -1.0 / 3.0) : rcbrt(err)) : 5.0;
                 fac = fmin(5.0, fmax(0.2, fac));
             }
             if (err <= 1.0) {
                 t = last ? dt : t + h;
-                y[0] = yn[0];
-                y[1] = yn[1];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) y[s] = yn[s];
                 if (rejected_last && fac > 1.0) fac = 1.0;
                 h *= fac;
                 rejected_last = 0;
@@ -747,8 +1025,9 @@ __device__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int6
             }
         }
         if (tm.lead()) {
-            for (int s = 0; s < 2; ++s) {
-                int c = lane + 32 * s;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                const int c = lane + 32 * s;
                 if (c == 0) Tg[cell] = y[s];
                 else if (c < n) Yg[(int64_t)(c - 1) * ld + cell] = y[s];
             }
@@ -764,43 +1043,93 @@ __device__ void integrate_cells(const DevMech &m, char *smem, int *blk_pos, int6
 // grid are spread over the SMs), at most the grid.
 inline int team_blocks(int sms, int blocks) { return sms < blocks ? sms : blocks; }
 
+// Resident blocks the registers are budgeted for: the mixed mode (32 FP32 row registers) runs 16 warps
+// per SM, the FP64 mode (64 row registers) 12; above 31 species shared memory decides (5 to 8 warps).
+constexpr int stiff_min_blocks(int NC, bool MX) { return NC > 32 ? 1 : (MX ? 4 : 3); }
+constexpr int kBigWarps = 8;         // most warps of a block above 31 species
+
 // Cells 0..ncells-1, or (list != null) the *list_count cells list[0..) of a
 // device-built queue; status of a successful cell = ok_status. When the cells
 // number at most team_blocks, the first team_blocks blocks integrate them with
-// all kWarps warps per cell and the other blocks return at once; otherwise
+// kWarps warps per cell and the other blocks return at once; otherwise
 // every warp takes cells of its own.
-__global__ void __launch_bounds__(kWarps * 32) stiff_kernel(DevMech m, int64_t ncells, int64_t ld, double dt,
-                                                             chem_ode_opts o, double *__restrict__ Tg,
-                                                             const double *__restrict__ pg, double *__restrict__ Yg,
-                                                             int32_t *__restrict__ status,
-                                                             int32_t *__restrict__ nsteps_out,
-                                                             unsigned int *__restrict__ queue,
-                                                             const int32_t *__restrict__ list,
-                                                             const unsigned int *__restrict__ list_count,
-                                                             int ok_status, int team_blocks) {
+template <int NC, bool MX>
+__global__ void __launch_bounds__(NC > 32 ? 32 * kBigWarps : 32 * kWarps, stiff_min_blocks(NC, MX))
+    stiff_kernel(const __grid_constant__ DevMech m, int64_t ncells, int64_t ld, double dt, chem_ode_opts o,
+                 double *__restrict__ Tg, const double *__restrict__ pg, double *__restrict__ Yg,
+                 int32_t *__restrict__ status, int32_t *__restrict__ nsteps_out, unsigned int *__restrict__ queue,
+                 const int32_t *__restrict__ list, const unsigned int *__restrict__ list_count, int ok_status,
+                 int team_blocks) {
     extern __shared__ __align__(16) char smem_raw[];
     int *blk_pos = reinterpret_cast<int *>(smem_raw);
     char *smem = smem_raw + kSmemHeader;
     const int64_t limit = list ? (int64_t)(*list_count < (unsigned int)ncells ? *list_count : (unsigned int)ncells)
                                : ncells;
-    // the mixed mode takes tolerances no tighter than kMixedMinRtol (its FP32 rates carry about
-    // 1e-6 relative noise)
-    const bool mx = o.mode == CHEM_ODE_MIXED && o.rtol >= kMixedMinRtol;
     if (limit <= (int64_t)team_blocks) {
-        if ((int)blockIdx.x >= team_blocks) return;
-        if (mx)
-            integrate_cells<kWarps, true>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue,
-                                          list, ok_status);
-        else
-            integrate_cells<kWarps, false>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue,
-                                           list, ok_status);
-    } else if (mx) {
-        integrate_cells<1, true>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
-                                 ok_status);
+        if ((int)blockIdx.x >= team_blocks || threadIdx.x >= 32 * kWarps) return;
+        integrate_cells<kWarps, NC, MX>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue,
+                                        list, ok_status);
     } else {
-        integrate_cells<1, false>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
-                                  ok_status);
+        integrate_cells<1, NC, MX>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
+                                   ok_status);
     }
+}
+
+// The launch of one kernel variant: warps per block and resident blocks for this mechanism.
+template <int NC, bool MX>
+int launch_stiff_nc(const chem_mech *m, int64_t capacity, int64_t ld, double dt, const chem_ode_opts &o, double *T,
+                    const double *p, double *Y, int32_t *status, int32_t *nsteps, unsigned int *queue,
+                    const int32_t *list, const unsigned int *count, int ok_status, cudaStream_t st, const char *who) {
+    constexpr size_t kSmemMax = 227 * 1024;
+    const size_t slice = make_slice<MX, (NC > 32)>(nullptr, m->N, m->R, m->dev.n_tb, m->dev.nslot, nullptr);
+    int warps = kWarps;
+    // above 31 species one block of up to kBigWarps warps where two blocks of kWarps do not fit
+    if (NC > 32 && 2 * (kSmemHeader + kWarps * slice) > kSmemMax)
+        while (warps < kBigWarps && kSmemHeader + (warps + 1) * slice <= kSmemMax) ++warps;
+    const size_t smem = kSmemHeader + slice * warps;
+    if (smem > kSmemMax)
+        return set_error(CHEM_EUNSUPPORTED, std::string(who) + ": mechanism too large for shared memory");
+    auto kernel = stiff_kernel<NC, MX>;
+    int rc = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
+    if (rc) return rc;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, warps * 32, smem);
+    if (per_sm < 1) per_sm = 1;
+    const int64_t need = (capacity + warps - 1) / warps;
+    int blocks = (int)((int64_t)sms * per_sm < need ? (int64_t)sms * per_sm : need);
+    if (!list && capacity <= sms) blocks = (int)capacity;      // one block (a team of warps) per cell
+    if (blocks < 1) blocks = 1;
+    rc = check_cuda(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st), who);
+    if (rc) return rc;
+    kernel<<<blocks, warps * 32, smem, st>>>(m->dev, capacity, ld, dt, o, T, p, Y, status, nsteps, queue, list, count,
+                                             ok_status, team_blocks(sms, blocks));
+    return check_cuda(cudaGetLastError(), who);
+}
+
+// Stiff integration of cells 0..capacity-1 (list null) or of a device-built list; queue: a work-queue
+// counter that this call clears on its stream. The mixed mode takes tolerances no tighter than
+// kMixedMinRtol (its FP32 rates carry about 1e-6 relative noise).
+int launch_stiff(const chem_mech *m, int64_t capacity, int64_t ld, double dt, const chem_ode_opts &o, double *T,
+                 const double *p, double *Y, int32_t *status, int32_t *nsteps, unsigned int *queue,
+                 const int32_t *list, const unsigned int *count, int ok_status, cudaStream_t st, const char *who) {
+    const bool mx = o.mode == CHEM_ODE_MIXED && o.rtol >= kMixedMinRtol;
+    const int n = m->N + 1;
+#define CHEMGB_STIFF(NC_, MX_)                                                                                      \
+    return launch_stiff_nc<NC_, MX_>(m, capacity, ld, dt, o, T, p, Y, status, nsteps, queue, list, count, ok_status, \
+                                     st, who)
+    if (n <= 16) {
+        if (mx) CHEMGB_STIFF(16, true);
+        CHEMGB_STIFF(16, false);
+    }
+    if (n <= 32) {
+        if (mx) CHEMGB_STIFF(32, true);
+        CHEMGB_STIFF(32, false);
+    }
+    if (mx) CHEMGB_STIFF(64, true);
+    CHEMGB_STIFF(64, false);
+#undef CHEMGB_STIFF
 }
 
 // PaSR scaling (Sec. 4.1), one warp per cell. The species times Y_k / |dY_k/dt| come from the
@@ -809,8 +1138,10 @@ __global__ void __launch_bounds__(kWarps * 32) stiff_kernel(DevMech m, int64_t n
 // (the slowest formation rate), +inf when none qualifies; tau_mix = sqrt(tau_T tau_K);
 // kappa = tau_c / (tau_c + tau_mix), 1 for an infinite tau_c. With T, Y given (the chemistry
 // step's result), they become T0 + kappa (T - T0), Y0 + kappa (Y - Y0).
-__global__ void __launch_bounds__(kWarps * 32) pasr_kernel(DevMech m, int64_t ncells, int64_t ld, double y_min,
-                                                            const double *__restrict__ T0,
+__host__ __device__ inline size_t pasr_slice_bytes(int N, int R) { return (size_t)(3 * (N + 1) + R) * 8; }
+template <int NS>
+__global__ void __launch_bounds__(kWarps * 32) pasr_kernel(const __grid_constant__ DevMech m, int64_t ncells,
+                                                            int64_t ld, double y_min, const double *__restrict__ T0,
                                                             const double *__restrict__ pg,
                                                             const double *__restrict__ Y0,
                                                             const double *__restrict__ tau_t,
@@ -820,17 +1151,23 @@ __global__ void __launch_bounds__(kWarps * 32) pasr_kernel(DevMech m, int64_t nc
     extern __shared__ __align__(16) char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int N = m.N, n = N + 1;
-    const Slice sh = make_slice(smem_raw + (size_t)warp * slice_bytes(N, m.R), N, m.R);
+    Slice<false> sh{};
+    sh.C = reinterpret_cast<double *>(smem_raw + (size_t)warp * pasr_slice_bytes(N, m.R));
+    sh.g = sh.C + N + 1;
+    sh.H = sh.g + N + 1;
+    sh.rq = sh.H + N + 1;
     const Team<1> tm{0};
     for (int64_t cell = (int64_t)blockIdx.x * kWarps + warp; cell < ncells; cell += (int64_t)gridDim.x * kWarps) {
-        double y[2], f[2];
-        for (int s = 0; s < 2; ++s) {
+        double y[NS], f[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
             const int c = lane + 32 * s;
             y[s] = (c == 0) ? T0[cell] : (c < n ? Y0[(int64_t)(c - 1) * ld + cell] : 0.0);
         }
-        eval_rhs<1, false>(m, sh, tm, lane, pg[cell], y, f, false);
+        eval_rhs<1, NS, false, false>(m, sh, tm, lane, pg[cell], kR / pg[cell], y, f);
         double tmax = -1.0;                       // species times are >= 0: -1 marks none
-        for (int s = 0; s < 2; ++s) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
             const int c = lane + 32 * s;
             if (c >= 1 && c < n) {
                 const double r = fabs(f[s]);
@@ -847,7 +1184,8 @@ __global__ void __launch_bounds__(kWarps * 32) pasr_kernel(DevMech m, int64_t nc
             if (kappa_out) kappa_out[cell] = kap;
         }
         if (T && Y)
-            for (int s = 0; s < 2; ++s) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
                 const int c = lane + 32 * s;
                 if (c == 0) T[cell] = y[s] + kap * (T[cell] - y[s]);
                 else if (c < n) {
@@ -879,26 +1217,23 @@ extern "C" int chem_pasr(const chem_mech *m, int64_t ncells, int64_t ld, double 
         if (q && !aligned16(q)) return set_error(CHEM_EINVAL, "chem_pasr: arrays must be 16-byte aligned");
     std::string why;
     if (!device_ok(&why)) return set_error(CHEM_EUNSUPPORTED, "chem_pasr: " + why);
-    const size_t smem = slice_bytes(m->N, m->R) * kWarps;
+    const size_t smem = pasr_slice_bytes(m->N, m->R) * kWarps;
     if (smem > 227 * 1024) return set_error(CHEM_EUNSUPPORTED, "chem_pasr: mechanism too large for shared memory");
-    static size_t configured = 0;
-    if (smem > configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(pasr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                            "chem_pasr: smem attribute");
-        if (rc) return rc;
-        configured = smem;
-    }
+    auto kernel = m->N <= 31 ? pasr_kernel<1> : pasr_kernel<2>;
+    int rc = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                        "chem_pasr: smem attribute");
+    if (rc) return rc;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pasr_kernel, kWarps * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWarps * 32, smem);
     if (per_sm < 1) per_sm = 1;
     const int64_t need = (ncells + kWarps - 1) / kWarps;
     const int blocks = (int)((int64_t)sms * per_sm < need ? (int64_t)sms * per_sm : need);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     void *pb = prof_begin(st);
-    pasr_kernel<<<blocks, kWarps * 32, smem, st>>>(m->dev, ncells, ld, y_min, T0, p, Y0, tau_taylor, tau_kolmogorov,
-                                                   T, Y, tau_c, kappa);
+    kernel<<<blocks, kWarps * 32, smem, st>>>(m->dev, ncells, ld, y_min, T0, p, Y0, tau_taylor, tau_kolmogorov, T, Y,
+                                              tau_c, kappa);
     prof_end(pb, st, "pasr_kernel", 0.0, (double)ncells * ((m->N + 2) * 8 + 2 * 8 + (T ? 2 * (m->N + 1) * 8 : 0)));
     return check_cuda(cudaGetLastError(), "chem_pasr launch");
 }
@@ -925,33 +1260,12 @@ extern "C" int chem_step_stiff(const chem_mech *m, int64_t ncells, int64_t ld, d
         return set_error(CHEM_EINVAL, "chem_step_stiff: mode must be CHEM_ODE_FP64 or CHEM_ODE_MIXED");
     std::string why;
     if (!device_ok(&why)) return set_error(CHEM_EUNSUPPORTED, "chem_step_stiff: " + why);
-    size_t per_warp = slice_bytes(m->N, m->R);
-    size_t smem = kSmemHeader + per_warp * kWarps;
-    if (smem > 227 * 1024) return set_error(CHEM_EUNSUPPORTED, "chem_step_stiff: mechanism too large for shared memory");
-    static size_t configured = 0;
-    if (smem > configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(stiff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                            "chem_step_stiff: smem attribute");
-        if (rc) return rc;
-        configured = smem;
-    }
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stiff_kernel, kWarps * 32, smem);
-    if (per_sm < 1) per_sm = 1;
-    int64_t need = (ncells + kWarps - 1) / kWarps;
-    int blocks = (int)((int64_t)sms * per_sm < need ? (int64_t)sms * per_sm : need);
-    if (ncells <= sms) blocks = (int)ncells;      // one block (a team of warps) per cell
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    unsigned int *queue = m->dev.counters;
-    int rc = check_cuda(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st), "chem_step_stiff: queue reset");
-    if (rc) return rc;
     void *pb = prof_begin(st);
-    stiff_kernel<<<blocks, kWarps * 32, smem, st>>>(m->dev, ncells, ld, dt, o, T, p, Y, status, nsteps, queue, nullptr,
-                                                    nullptr, CHEM_CELL_OK, team_blocks(sms, blocks));
+    const int rc = launch_stiff(m, ncells, ld, dt, o, T, p, Y, status, nsteps, m->dev.counters, nullptr, nullptr,
+                                CHEM_CELL_OK, st, "chem_step_stiff");
     prof_end(pb, st, "stiff_kernel", 0.0, 0.0);
-    return check_cuda(cudaGetLastError(), "chem_step_stiff launch");
+    return rc;
 }
 
 namespace chemgb {
@@ -962,25 +1276,8 @@ int launch_stiff_list(const chem_mech *m, int64_t capacity, int64_t ld, double d
                       const double *p, double *Y, int32_t *status, const int32_t *list, const unsigned int *count,
                       int ok_status, cudaStream_t st) {
     if (m->N > 63) return set_error(CHEM_EUNSUPPORTED, "fallback: at most 63 species");
-    size_t smem = kSmemHeader + slice_bytes(m->N, m->R) * kWarps;
-    if (smem > 227 * 1024) return set_error(CHEM_EUNSUPPORTED, "fallback: mechanism too large for shared memory");
-    int rc = check_cuda(cudaFuncSetAttribute(stiff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                        "fallback: smem attribute");
-    if (rc) return rc;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stiff_kernel, kWarps * 32, smem);
-    if (per_sm < 1) per_sm = 1;
-    int64_t need = (capacity + kWarps - 1) / kWarps;
-    int blocks = (int)((int64_t)sms * per_sm < need ? (int64_t)sms * per_sm : need);
-    if (blocks < 1) blocks = 1;
-    unsigned int *queue = m->dev.counters + 1;
-    rc = check_cuda(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st), "fallback: queue reset");
-    if (rc) return rc;
-    stiff_kernel<<<blocks, kWarps * 32, smem, st>>>(m->dev, capacity, ld, dt, o, T, p, Y, status, nullptr, queue, list,
-                                                    count, ok_status, team_blocks(sms, blocks));
-    return check_cuda(cudaGetLastError(), "fallback launch");
+    return launch_stiff(m, capacity, ld, dt, o, T, p, Y, status, nullptr, m->dev.counters + 1, list, count, ok_status,
+                        st, "fallback");
 }
 }  // namespace chemgb
 
@@ -1056,24 +1353,6 @@ extern "C" int chem_step_stiff_noalloc(const chem_mech *m, int64_t ncells, int64
     unsigned int *queue = nullptr;
     int rc = noalloc_scratch(&queue);
     if (rc) return rc;
-    size_t smem = kSmemHeader + slice_bytes(m->N, m->R) * kWarps;
-    if (smem > 227 * 1024)
-        return set_error(CHEM_EUNSUPPORTED, "chem_step_stiff_noalloc: mechanism too large for shared memory");
-    rc = check_cuda(cudaFuncSetAttribute(stiff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                    "chem_step_stiff_noalloc: smem attribute");
-    if (rc) return rc;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stiff_kernel, kWarps * 32, smem);
-    if (per_sm < 1) per_sm = 1;
-    int64_t need = (ncells + kWarps - 1) / kWarps;
-    int blocks = (int)((int64_t)sms * per_sm < need ? (int64_t)sms * per_sm : need);
-    if (ncells <= sms) blocks = (int)ncells;      // one block (a team of warps) per cell
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    rc = check_cuda(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st), "chem_step_stiff_noalloc: clear queue");
-    if (rc) return rc;
-    stiff_kernel<<<blocks, kWarps * 32, smem, st>>>(m->dev, ncells, ld, dt, o, T, p, Y, status, nsteps, queue, nullptr,
-                                                    nullptr, CHEM_CELL_OK, team_blocks(sms, blocks));
-    return check_cuda(cudaGetLastError(), "chem_step_stiff_noalloc launch");
+    return launch_stiff(m, ncells, ld, dt, o, T, p, Y, status, nsteps, queue, nullptr, nullptr, CHEM_CELL_OK,
+                        reinterpret_cast<cudaStream_t>(stream), "chem_step_stiff_noalloc");
 }
