@@ -129,9 +129,9 @@ __device__ __forceinline__ float gelu_exact(float z) {
     const float s = fmaf(y, e, 1.0f);                 // erf(sqrt(2) |h|)
     return fmaf(fabsf(h), s, h);
 }
-// GELU(v0 + b0), GELU(v1 + b1): the scalar operations above, two lanes at a time
-__device__ __forceinline__ void gelu_pair(float v0, float v1, float b0, float b1, float &g0, float &g1) {
-    const uint64_t h = mul2(add2(pk2(v0, v1), pk2(b0, b1)), pk2(0.5f, 0.5f));
+// GELU(z0), GELU(z1), and with biases added first: the scalar operations above, two lanes at a time
+__device__ __forceinline__ void gelu_pair(uint64_t z, float &g0, float &g1) {
+    const uint64_t h = mul2(z, pk2(0.5f, 0.5f));
     float h0, h1;
     upk2(h, h0, h1);
     const uint64_t y = neg_erfcx2(pk2(fminf(fabsf(h0), kGeluXmax), fminf(fabsf(h1), kGeluXmax)));
@@ -139,6 +139,9 @@ __device__ __forceinline__ void gelu_pair(float v0, float v1, float b0, float b1
     upk2(mul2(mul2(h, pk2(kNeg2Log2e, kNeg2Log2e)), h), m0, m1);
     const uint64_t s = fma2(y, pk2(ex2_approx(m0), ex2_approx(m1)), pk2(1.0f, 1.0f));
     upk2(fma2(pk2(fabsf(h0), fabsf(h1)), s, h), g0, g1);
+}
+__device__ __forceinline__ void gelu_pair(float v0, float v1, float b0, float b1, float &g0, float &g1) {
+    gelu_pair(add2(pk2(v0, v1), pk2(b0, b1)), g0, g1);
 }
 // dGELU/dz = Phi(z) + z phi(z), with the same erf and exp(-z^2 / 2) = exp(-2 h^2)
 __device__ __forceinline__ float gelu_grad(float z) {
@@ -280,7 +283,7 @@ struct EpiLinear {
 
 // Y = bf16(acc * GELU'(Z)), Z the FP32 pre-activation of the layer below (backward pass). With aligned
 // rows Z is read 16 bytes at a time and Y stored by TMA: the product of 4096 x 1600 x 800 took 138 us
-// with element loads and stores (32 rows' sectors per instruction) and GRADUS that way.
+// with element loads and stores (32 rows' sectors per instruction) and takes 25 us that way.
 struct EpiGeluGrad {
     static constexpr bool kBNMajor = true;
     static constexpr bool kF8 = false;
@@ -363,24 +366,26 @@ struct EpiGeluQ {
                 c[4 * i] = c[4 * i + 1] = c[4 * i + 2] = c[4 * i + 3] = 1.0f;
             }
         }
+        float g[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint64_t z = F8IN ? fma2(pk2(v[2 * i], v[2 * i + 1]), pk2(c[2 * i], c[2 * i + 1]), pk2(b[2 * i], b[2 * i + 1]))
+                                    : add2(pk2(v[2 * i], v[2 * i + 1]), pk2(b[2 * i], b[2 * i + 1]));
+            gelu_pair(z, g[2 * i], g[2 * i + 1]);
+        }
         if (F8OUT) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(
-                    make_float2(act(v[4 * i], c[4 * i], b[4 * i]) * inv_so,
-                                act(v[4 * i + 1], c[4 * i + 1], b[4 * i + 1]) * inv_so),
-                    __NV_SATFINITE, __NV_E4M3);
+                    make_float2(g[4 * i] * inv_so, g[4 * i + 1] * inv_so), __NV_SATFINITE, __NV_E4M3);
                 const __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(
-                    make_float2(act(v[4 * i + 2], c[4 * i + 2], b[4 * i + 2]) * inv_so,
-                                act(v[4 * i + 3], c[4 * i + 3], b[4 * i + 3]) * inv_so),
-                    __NV_SATFINITE, __NV_E4M3);
+                    make_float2(g[4 * i + 2] * inv_so, g[4 * i + 3] * inv_so), __NV_SATFINITE, __NV_E4M3);
                 w[i] = (uint32_t)lo | ((uint32_t)hi << 16);
             }
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                __nv_bfloat162 h = __floats2bfloat162_rn(act(v[2 * i], c[2 * i], b[2 * i]),
-                                                         act(v[2 * i + 1], c[2 * i + 1], b[2 * i + 1]));
+                __nv_bfloat162 h = __floats2bfloat162_rn(g[2 * i], g[2 * i + 1]);
                 w[i] = *reinterpret_cast<uint32_t *>(&h);
             }
         }

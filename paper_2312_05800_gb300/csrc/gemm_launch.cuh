@@ -229,14 +229,17 @@ int launch_gemm(int bn, const void *X, int64_t ldx, const void *W, int64_t ldw, 
                                K, epi, err, st, max_ctas);
 }
 
-// Default tile width for an output width N (fewest padded columns, then widest tile).
+// Default tile width for an output width N: a tile's time is about that of its columns plus 290 (the
+// operands' k-blocks and the tile's own start and end), so the width with the smallest sum over the
+// N tiles. Measured on 262,144 rows (us at 160 / 208 / 256): 800 x 1600 553 / 488 / 502, 1600 x 96 330 / 348 /
+// 310, 400 x 800 201 / 159 / 205, 1024 x 2048 954 / 766 / 671; the fewest padded columns, the rule before, took 160
+// for the first two.
 inline int default_tile_width(int N) {
     int best = 256;
-    long best_pad = -1;
+    long best_cost = -1;
     for (int bn : kTileWidths) {
-        if (bn < 64 && N > 64) continue;
-        long pad = (long)((N + bn - 1) / bn) * bn - N;
-        if (best_pad < 0 || pad < best_pad || (pad == best_pad && bn > best)) { best = bn; best_pad = pad; }
+        const long cost = (long)((N + bn - 1) / bn) * (bn + 290);
+        if (best_cost < 0 || cost < best_cost) { best = bn; best_cost = cost; }
     }
     return best;
 }
