@@ -140,4 +140,11 @@ __device__ __forceinline__ double f32_to_f64_int(float x) {
     const unsigned long long mant = static_cast<unsigned long long>(b & 0x7FFFFFu) << 29;
     return __longlong_as_double(static_cast<long long>(sign | (ed << 52) | mant));
 }
+// The same for a finite value.
+__device__ __forceinline__ double f32_to_f64_finite(float x) {
+    const unsigned b = __float_as_uint(x);
+    const bool zero = (b & 0x7F800000u) == 0u;
+    const unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)((zero ? 0u : hi) | (b & 0x80000000u)), (int)(zero ? 0u : b << 29));
+}
 }  // namespace chemgb

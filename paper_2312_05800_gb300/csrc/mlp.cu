@@ -145,7 +145,7 @@ __device__ __forceinline__ float f64_to_f32_near(double x) {
 // A block takes 32 cells, a warp 8 of their columns (lanes = cells, so the state rows are read
 // coalesced); the rows are put together in shared memory and written as one contiguous block.
 // A thread per cell wrote 16-byte pieces at a stride of a row and left small calls with a serial chain of
-// n_in powers: PROLOGUS.
+// n_in powers: 4,096 gathered rows took 28 us and take 7.4, 2,500 cells 23 and 5.
 __global__ void prologue_kernel(int64_t n, int64_t ld, const double *__restrict__ T, const double *__restrict__ p,
                                 const double *__restrict__ Y, const int32_t *__restrict__ idx, int N, int n_in_pad,
                                 const float *__restrict__ mu, const float *__restrict__ isd,
@@ -213,9 +213,8 @@ __device__ __forceinline__ int ood_bin(const float f[3], const float *range, int
 
 // Per cell: dY_k = sigma_k u_k + mu_k (output species), dY_bath = -sum dY_k,
 // Y' = max(Y + dY, 0) renormalised, T' from h(T', Y') = h(T, Y) by Newton.
-// dY and the provisional Y' live in FP32 registers (species loops unrolled to
-// the compile-time bound NMAX) for the enthalpy Newton iteration; the final
-// clamp and renormalisation are FP64 so that sum Y' = 1 to FP64 round-off.
+// The enthalpy Newton iteration is FP32; the final clamp and renormalisation are
+// FP64 so that sum Y' = 1 to FP64 round-off.
 struct OodRoute {
     const float *range;      // per grid lo[3], inv_width[3]; null: no test
     const uint8_t *mask[kOodMaxGrids];
@@ -229,26 +228,42 @@ struct OodRoute {
 // true when a cell with features (T, h/R) and the state Y is outside any grid's distribution
 __device__ __forceinline__ bool ood_outside(const OodRoute &ood, float T, float h, const double *Y, int64_t ld,
                                             int64_t i) {
-    for (int g = 0; g < ood.ngrids; ++g) {
-        const float f[3] = {T, h, f64_to_f32_trunc(Y[(int64_t)ood.species[g] * ld + i])};
-        const int b = ood_bin(f, ood.range + 6 * g, ood.nb);
-        if (b < 0 || ood.mask[g][b] == 0) return true;
+#pragma unroll
+    for (int g = 0; g < kOodMaxGrids; ++g) {
+        if (g < ood.ngrids) {
+            const float f[3] = {T, h, f64_to_f32_trunc(Y[(int64_t)ood.species[g] * ld + i])};
+            const int b = ood_bin(f, ood.range + 6 * g, ood.nb);
+            if (b < 0 || ood.mask[g][b] == 0) return true;
+        }
     }
     return false;
 }
 
-template <int NMAX>
-__global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int64_t n, int64_t ld, const float *__restrict__ u, int ldu,
+// Layout: a thread per cell; the state is read once, eight species' loads in flight, and kept with dY in
+// shared memory columns (conflict-free), from which the passes below take it. FP64 work is three
+// additions or multiplications per species, the FP64 pipe's floor of about 0.65 ms for 4,194,304 30-species
+// cells. Loads one by one under a test of k < N and the state re-read from L2 took 2.14 ms for them and
+// 38 us for 2,500 cells, EPIUS. Blocks of 32 cells where blocks of 128 would not fill the chip.
+template <int NMAX, int BD>
+struct EpiLayout {
+    static constexpr size_t tab = 2 * NMAX * 3 * sizeof(float4) + NMAX * sizeof(float2);
+    static size_t bytes(int N) { return tab + (size_t)N * BD * (sizeof(double) + sizeof(float)); }
+};
+template <int NMAX, int BD>
+__global__ void __launch_bounds__(BD) epilogue_kernel(int64_t n, int64_t ld, const float *__restrict__ u, int ldu,
                                                        int N, int bath, const float *__restrict__ mu_u,
                                                        const float *__restrict__ sd_u, PropTables<float> tb,
                                                        float T_mid, double *__restrict__ T, double *__restrict__ Y,
                                                        int32_t *__restrict__ status, OodRoute ood) {
-    // per species and range: cp/R coefficients (5), H/R coefficients (6), 1/W -> 3 float4
-    __shared__ float4 tab[2 * NMAX * 3];
-    // dY per species and thread (column per thread: conflict-free), so that only the provisional
-    // Y' stays in registers and the kernel keeps more warps resident
-    __shared__ float dyS[NMAX][128];
-    for (int e = threadIdx.x; e < 2 * N; e += blockDim.x) {
+    extern __shared__ __align__(16) unsigned char epi_smem[];
+    const int t = threadIdx.x;
+    // per species and range: cp/R coefficients (5), H/R coefficients (6), 1/W -> 3 float4; then the output
+    // statistics (sd, mu), zero for the bath
+    float4 *tab = reinterpret_cast<float4 *>(epi_smem);
+    float2 *stat = reinterpret_cast<float2 *>(tab + 2 * NMAX * 3);
+    double *yS = reinterpret_cast<double *>(epi_smem + EpiLayout<NMAX, BD>::tab) + t;      // [N][BD]
+    float *dyS = reinterpret_cast<float *>(yS - t + (size_t)N * BD) + t;                   // [N][BD]
+    for (int e = t; e < 2 * N; e += BD) {
         const int rg = e / N, k = e % N;
         const float *a = tb.nasa_cp + (rg * N + k) * 5;
         const float *b = tb.nasa_h + (rg * N + k) * 6;
@@ -257,30 +272,60 @@ __global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int
         o[1] = make_float4(a[4], b[0], b[1], b[2]);
         o[2] = make_float4(b[3], b[4], b[5], tb.invW[k]);
     }
+    for (int k = t; k < N; k += BD) {
+        const int j = k < bath ? k : k - 1;
+        stat[k] = k == bath ? make_float2(0.0f, 0.0f) : make_float2(sd_u[j], mu_u[j]);
+    }
     __syncthreads();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * BD + t;
     if (i >= n) return;
-    const int t = threadIdx.x;
     const float *ur = u + i * ldu;
-    const float T0 = (float)T[i];
+    double *Yi = Y + i;
+    const float T0 = f64_to_f32_near(T[i]);
     const int r0 = (T0 >= T_mid) ? 1 : 0;
-    float sum = 0.0f, h0 = 0.0f;
+    float sum = 0.0f, h0 = 0.0f, last = 0.0f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < N; k0 += 8) {
+        double yv[8];
+        const double *q0 = Yi + (int64_t)k0 * ld;
 #pragma unroll
-    for (int k = 0; k < NMAX; ++k) {
-        if (k < N) {
-            const float y = f64_to_f32_trunc(Y[(int64_t)k * ld + i]);
-            float d = 0.0f;
-            if (k != bath) {
-                const int j = (k < bath) ? k : k - 1;   // outputs: the non-bath species, ascending
-                d = fmaf(__ldg(sd_u + j), ur[j], __ldg(mu_u + j));
+        for (int q = 0; q < 8; ++q) {
+            yv[q] = k0 + q < N ? *q0 : 0.0;
+            q0 += ld;
+        }
+        // the row's outputs k0 .. k0 + 7; the outputs are the non-bath species, so species past the bath take the
+        // one before theirs
+        float o[8], uv[8];
+        if (k0 < ldu) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(ur + k0)), b = __ldg(reinterpret_cast<const float4 *>(ur + k0) + 1);
+            o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) o[q] = 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int k = k0 + q;
+            uv[q] = k < bath ? o[q] : (k > bath ? (q == 0 ? last : o[q == 0 ? 0 : q - 1]) : 0.0f);
+        }
+        last = o[7];
+        const float4 *r = tab + (r0 * NMAX + k0) * 3;
+        double *yo = yS + k0 * BD;
+        float *dq = dyS + k0 * BD;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if (k0 + q < N) {
+                yo[q * BD] = yv[q];
+                const float y = f64_to_f32_trunc(yv[q]);
+                const float2 st = stat[k0 + q];
+                const float d = fmaf(st.x, uv[q], st.y);       // 0 for the bath
                 sum += d;
+                dq[q * BD] = d;
+                const float4 q1 = r[3 * q + 1], q2 = r[3 * q + 2];
+                float hh = fmaf(fmaf(fmaf(fmaf(q2.y, T0, q2.x), T0, q1.w), T0, q1.z), T0, q1.y);
+                hh = hh * T0 + q2.z;                       // H_k / R
+                h0 = fmaf(y * q2.w, hh, h0);
             }
-            dyS[k][t] = d;
-            const float4 *q = tab + (r0 * NMAX + k) * 3;
-            const float4 q1 = q[1], q2 = q[2];
-            float hh = fmaf(fmaf(fmaf(fmaf(q2.y, T0, q2.x), T0, q1.w), T0, q1.z), T0, q1.y);
-            hh = hh * T0 + q2.z;                       // H_k / R
-            h0 = fmaf(y * q2.w, hh, h0);
         }
     }
     // a non-finite prediction (non-finite weights or statistics, an overflow) never reaches the
@@ -298,12 +343,11 @@ __global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int
         if (status) status[i] = CHEM_CELL_NONFINITE;     // without the guard: the state is kept
         return;
     }
-    dyS[bath][t] = -sum;
+    dyS[bath * BD] = -sum;
     // Newton on h(T', Y') = h0 with Y' = max(Y + dY, 0) / sum. The mixture's cp/R and H/R are
     // polynomials in T whose coefficients are sum_k (Y'_k / W_k) a_k: formed once per cell for the
-    // range in use (again, from the state and dY, only if T' crosses T_mid), so that an iteration
-    // is two polynomial evaluations instead of a pass over the species' NASA rows. The provisional
-    // Y' is not kept: the state is re-read from cache.
+    // range in use (again only if T' crosses T_mid), so that an iteration is two polynomial
+    // evaluations instead of a pass over the species' NASA rows.
     float mc[5], mh[6];
     auto mix = [&](int rg) {
 #pragma unroll
@@ -311,26 +355,24 @@ __global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int
 #pragma unroll
         for (int j = 0; j < 6; ++j) mh[j] = 0.0f;
         float s = 0.0f;
-#pragma unroll
-        for (int k = 0; k < NMAX; ++k) {
-            if (k < N) {
-                const float y = fmaxf(f64_to_f32_trunc(Y[(int64_t)k * ld + i]) + dyS[k][t], 0.0f);
-                s += y;
-                const float4 *q = tab + (rg * NMAX + k) * 3;
-                const float4 q0 = q[0], q1 = q[1], q2 = q[2];
-                const float yw = y * q2.w;
-                mc[0] = fmaf(yw, q0.x, mc[0]);
-                mc[1] = fmaf(yw, q0.y, mc[1]);
-                mc[2] = fmaf(yw, q0.z, mc[2]);
-                mc[3] = fmaf(yw, q0.w, mc[3]);
-                mc[4] = fmaf(yw, q1.x, mc[4]);
-                mh[0] = fmaf(yw, q1.y, mh[0]);
-                mh[1] = fmaf(yw, q1.z, mh[1]);
-                mh[2] = fmaf(yw, q1.w, mh[2]);
-                mh[3] = fmaf(yw, q2.x, mh[3]);
-                mh[4] = fmaf(yw, q2.y, mh[4]);
-                mh[5] = fmaf(yw, q2.z, mh[5]);
-            }
+#pragma unroll 4
+        for (int k = 0; k < N; ++k) {
+            const float y = fmaxf(f64_to_f32_trunc(yS[k * BD]) + dyS[k * BD], 0.0f);
+            s += y;
+            const float4 *q = tab + (rg * NMAX + k) * 3;
+            const float4 q0 = q[0], q1 = q[1], q2 = q[2];
+            const float yw = y * q2.w;
+            mc[0] = fmaf(yw, q0.x, mc[0]);
+            mc[1] = fmaf(yw, q0.y, mc[1]);
+            mc[2] = fmaf(yw, q0.z, mc[2]);
+            mc[3] = fmaf(yw, q0.w, mc[3]);
+            mc[4] = fmaf(yw, q1.x, mc[4]);
+            mh[0] = fmaf(yw, q1.y, mh[0]);
+            mh[1] = fmaf(yw, q1.z, mh[1]);
+            mh[2] = fmaf(yw, q1.w, mh[2]);
+            mh[3] = fmaf(yw, q2.x, mh[3]);
+            mh[4] = fmaf(yw, q2.y, mh[4]);
+            mh[5] = fmaf(yw, q2.z, mh[5]);
         }
         const float invs = 1.0f / s;
 #pragma unroll
@@ -338,7 +380,9 @@ __global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int
 #pragma unroll
         for (int j = 0; j < 6; ++j) mh[j] *= invs;
     };
-    float Tn = T0;
+    // An iteration is a function of Tn alone, so one that FP32 takes back to Tn or to the value before it
+    // decides all that follow: the loop ends with the value the thirtieth would have.
+    float Tn = T0, Tp = T0;
     int rc = -1;
     for (int it = 0; it < 30; ++it) {
         const int rg = (Tn >= T_mid) ? 1 : 0;
@@ -350,32 +394,35 @@ __global__ void __launch_bounds__(128, (NMAX <= 32 ? 8 : 4)) epilogue_kernel(int
         float h1 = fmaf(fmaf(fmaf(fmaf(mh[4], Tn, mh[3]), Tn, mh[2]), Tn, mh[1]), Tn, mh[0]);
         h1 = fmaf(h1, Tn, mh[5]);
         const float d = (h1 - h0) / c1;        // both in units of R
-        Tn -= d;
-        if (fabsf(d) < 1e-4f) break;
-    }
-    // FP64 update, clamp and renormalisation in two passes over the species (the state is
-    // re-read from cache): the widening of dY and the clamp test of the sign bit run on the
-    // integer pipe, leaving four FP64-pipe instructions per species
-    double s64 = 0.0;
-#pragma unroll
-    for (int k = 0; k < NMAX; ++k) {
-        if (k < N) {
-            double y = Y[(int64_t)k * ld + i] + f32_to_f64_int(dyS[k][t]);
-            if (__double_as_longlong(y) < 0) y = 0.0;
-            s64 += y;
+        const float Ta = Tn - d;
+        if (fabsf(d) < 1e-4f || Ta == Tn) {
+            Tn = Ta;
+            break;
         }
+        if (it > 0 && Ta == Tp) {              // it alternates between Tn and Ta
+            if (((29 - it) & 1) == 0) Tn = Ta;
+            break;
+        }
+        Tp = Tn;
+        Tn = Ta;
+    }
+    // FP64 update, clamp and renormalisation: the widening of dY and the clamp test of the sign bit run on
+    // the integer pipe, leaving three FP64-pipe instructions per species (every dY is finite: their sum is)
+    double s64 = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < N; ++k) {
+        double y = yS[k * BD] + f32_to_f64_finite(dyS[k * BD]);
+        if (__double2hiint(y) < 0) y = 0.0;
+        yS[k * BD] = y;
+        s64 += y;
     }
     const double inv = 1.0 / s64;
-#pragma unroll
-    for (int k = 0; k < NMAX; ++k) {
-        if (k < N) {
-            double *q = Y + (int64_t)k * ld + i;
-            double y = *q + f32_to_f64_int(dyS[k][t]);
-            if (__double_as_longlong(y) < 0) y = 0.0;
-            *q = y * inv;
-        }
+#pragma unroll 8
+    for (int k = 0; k < N; ++k) {
+        *Yi = yS[k * BD] * inv;
+        Yi += ld;
     }
-    T[i] = (double)Tn;
+    T[i] = f32_to_f64_int(Tn);
     if (status) status[i] = CHEM_CELL_OK;
 }
 
@@ -459,7 +506,7 @@ __device__ __forceinline__ float h_over_R(const float *b, float T) {
 
 // L1 loss of Eq. 5 on normalised outputs, dL/du = sign(u - u*)/B, plus the physics terms above
 // when their weights are non-zero; dL/du written as BF16, the per-sample loss to part. One warp per sample,
-// outputs over lanes (a thread per sample left 32 CTAs walking scattered rows: 42 us for 4096, LOSSUS now).
+// outputs over lanes (a thread per sample left 32 CTAs walking scattered rows: 42 us for 4096, 7.6 us now).
 __global__ void __launch_bounds__(128) l1_loss_kernel(int64_t B, const float *__restrict__ u, int ldu, const int32_t *__restrict__ idx,
                                int64_t ld, const double *__restrict__ Y0, const double *__restrict__ Y1, int n_out,
                                const int *__restrict__ out_sp, const float *__restrict__ mu_u,
@@ -630,8 +677,7 @@ __global__ void transpose_kernel(int rows, int cols, const __nv_bfloat16 *__rest
 
 // Adam (Kingma and Ba 2015) on every layer in one launch, four parameters of a weight row per thread
 // (rows are padded to 8; padding has zero gradients and stays zero), refreshing the BF16 copy. Memory
-// bound: 30 bytes per parameter (31 us in four launches with a scattered transposed copy, ADAMUS now for 1.67M
-// parameters).
+// bound: 30 bytes per parameter (34 us in four launches with a scattered transposed copy, 9 us now for 1.67M parameters).
 struct AdamLayer {
     float *W, *b, *mW, *vW, *mb, *vb;
     const float *gW, *gb;
@@ -1506,21 +1552,27 @@ int step_ann_impl(const chem_mech *mech, const chem_mlp *m, int64_t ncells, int6
             queued += n;
         }
         void *pb = prof_begin(st);
-        const unsigned eg = (unsigned)((n + 127) / 128);
+        auto epi = [&](auto kernel, size_t smem, int threads) -> int {
+            int r = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                               "chem_step_ann epilogue");
+            if (r) return r;
+            kernel<<<(unsigned)((n + threads - 1) / threads), threads, smem, st>>>(
+                n, ld, m->out, m->n_out_pad, m->N, m->bath, m->mu_u, m->sd_u, mech->dev.f32, (float)mech->T_mid, T + c0,
+                Y + c0, st_chunk, route);
+            return check_cuda(cudaGetLastError(), "chem_step_ann epilogue");
+        };
+        // blocks of 32 cells while blocks of 128 would leave SMs without one
+        const bool few = n < (int64_t)128 * num_sms();
         if (m->N <= 16)
-            epilogue_kernel<16><<<eg, 128, 0, st>>>(n, ld, m->out, m->n_out_pad, m->N, m->bath, m->mu_u, m->sd_u,
-                                                    mech->dev.f32, (float)mech->T_mid, T + c0, Y + c0,
-                                                    st_chunk, route);
+            rc = few ? epi(epilogue_kernel<16, 32>, EpiLayout<16, 32>::bytes(m->N), 32)
+                     : epi(epilogue_kernel<16, 128>, EpiLayout<16, 128>::bytes(m->N), 128);
         else if (m->N <= 32)
-            epilogue_kernel<32><<<eg, 128, 0, st>>>(n, ld, m->out, m->n_out_pad, m->N, m->bath, m->mu_u, m->sd_u,
-                                                    mech->dev.f32, (float)mech->T_mid, T + c0, Y + c0,
-                                                    st_chunk, route);
+            rc = few ? epi(epilogue_kernel<32, 32>, EpiLayout<32, 32>::bytes(m->N), 32)
+                     : epi(epilogue_kernel<32, 128>, EpiLayout<32, 128>::bytes(m->N), 128);
         else
-            epilogue_kernel<64><<<eg, 128, 0, st>>>(n, ld, m->out, m->n_out_pad, m->N, m->bath, m->mu_u, m->sd_u,
-                                                    mech->dev.f32, (float)mech->T_mid, T + c0, Y + c0,
-                                                    st_chunk, route);
+            rc = few ? epi(epilogue_kernel<64, 32>, EpiLayout<64, 32>::bytes(m->N), 32)
+                     : epi(epilogue_kernel<64, 128>, EpiLayout<64, 128>::bytes(m->N), 128);
         prof_end(pb, st, "epilogue_kernel", 0.0, (double)n * (m->N * 16 + 16 + m->n_out_pad * 4));
-        rc = check_cuda(cudaGetLastError(), "chem_step_ann epilogue");
         if (rc) return rc;
     }
     rc = flush(flush_base);

@@ -796,15 +796,6 @@ __device__ void tri_solve(const int *piv, const real *G, const real *invd, real 
     __syncwarp();
 }
 
-// FP32 -> FP64 of a finite value (subnormals become signed zero). A matrix with an infinity or a NaN has
-// no finite pivot or solution, whatever this makes of it.
-__device__ __forceinline__ double f32_to_f64_finite(float x) {
-    const unsigned b = __float_as_uint(x);
-    const bool zero = (b & 0x7F800000u) == 0u;
-    const unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u;
-    return __hiloint2double((int)((zero ? 0u : hi) | (b & 0x80000000u)), (int)(zero ? 0u : b << 29));
-}
-
 // The factored system of one step: NC <= 32 in registers, NC = 64 in shared memory.
 template <int W, int NC, bool MX>
 struct Factors {
@@ -833,7 +824,8 @@ struct Factors {
     // refinement, r = b - G x in FP64 arithmetic and x += Gf^-1 r. The correction solves the residual to
     // FP32's relative accuracy, so the refined x carries about cond(G) 2^-24 times that error. The
     // conversions between FP64 and FP32 run on the integer pipe (truncation; magnitudes below 2^-126
-    // become 0).
+    // become 0). A matrix with an infinity or a NaN has no finite pivot or solution, whatever the
+    // conversion of finite values makes of it.
     template <int NS>
     __device__ __forceinline__ void solve(const Slice<MX> &sh, double *xs, int lane, int n, double (&b)[NS]) const {
         if constexpr (!MX) {
