@@ -291,6 +291,122 @@ __global__ void __launch_bounds__(128) props_kernel(int N, int Np, real T_mid, P
     }
 }
 
+// The same in FP64 with G threads per cell (G lanes of a warp, species k = lane, lane + G, ...), for calls
+// whose cells do not fill the chip with a thread each: FP64 issues one warp instruction per 64 clocks and
+// SM sub-partition, so 4,096 cells of 9 species on 32 of the SMs took 80 us, a serial chain of about 1,800
+// such instructions, and take 33 us spread over all of them. Per species one exponential (r = sqrt(mu), mu =
+// r^2) and two divisions; X_j enters the sums as Y_j / W_j and 1 / Wbar cancels in mu and lambda. Beyond
+// kSplitWarps warps per SM the loop above does less work per cell (its scalars serve 32 cells a
+// warp).
+constexpr int kSplitWarps = 4;
+template <int G>
+__global__ void __launch_bounds__(128)
+    props_split_kernel(int N, int Np, double T_mid, PropTables<double> tb, int64_t ncells, int64_t ld,
+                       const double *__restrict__ Tg, const double *__restrict__ pg, const double *__restrict__ Yg,
+                       double *__restrict__ cpg, double *__restrict__ hg, double *__restrict__ mug,
+                       double *__restrict__ lamg, double *__restrict__ Dkg) {
+    extern __shared__ double split_smem[];                    // [128 / G][3][N]: Y / W, r, 1 / r
+    const int l = threadIdx.x & (G - 1), slot = threadIdx.x / G;
+    const int64_t cell = (int64_t)blockIdx.x * (128 / G) + slot;
+    const bool valid = cell < ncells;
+    const int64_t i = valid ? cell : ncells - 1;
+    const bool transport = (mug != nullptr) || (lamg != nullptr) || (Dkg != nullptr);
+    double *xs = split_smem + (size_t)slot * 3 * N, *rs = xs + N, *is = rs + N;
+    auto group_sum = [](double v) {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    const double T = Tg[i], p = pg[i];
+    const int rng = (T >= T_mid) ? 1 : 0;
+    const double iT = 1.0 / T;
+    const double x = log(T) - 6.907755278982137;              // ln(T / 1000)
+    double S = 0.0, cpm = 0.0, hm = 0.0;
+    for (int k = l; k < N; k += G) {
+        const double *a = tb.nasa_cp + (rng * N + k) * 5, *b = tb.nasa_h + (rng * N + k) * 6, *c = tb.visc + k * 5;
+        const double yw = Yg[(int64_t)k * ld + i] * __ldg(tb.invW + k);
+        const double cpR = fma(fma(fma(fma(__ldg(a + 4), T, __ldg(a + 3)), T, __ldg(a + 2)), T, __ldg(a + 1)), T, __ldg(a));
+        double hR = fma(fma(fma(fma(__ldg(b + 4), T, __ldg(b + 3)), T, __ldg(b + 2)), T, __ldg(b + 1)), T, __ldg(b));
+        hR = fma(__ldg(b + 5), iT, hR);                       // H_k / (R T)
+        S += yw;
+        cpm = fma(yw, cpR, cpm);
+        hm = fma(yw, hR, hm);
+        if (transport) {
+            const double lm = fma(fma(fma(fma(__ldg(c + 4), x, __ldg(c + 3)), x, __ldg(c + 2)), x, __ldg(c + 1)), x, __ldg(c));
+            const double r = exp(0.5 * lm);
+            xs[k] = yw;
+            rs[k] = r;
+            is[k] = 1.0 / r;
+        }
+    }
+    S = group_sum(S);
+    cpm = group_sum(cpm);
+    hm = group_sum(hm);
+    if (l == 0 && valid) {
+        if (cpg) cpg[i] = cpm * kR;
+        if (hg) hg[i] = hm * kR * T;
+    }
+    if (!transport) return;
+    __syncwarp();                                             // a cell's threads are one warp's
+    const double Wbar = 1.0 / S;
+    const double T15 = T * sqrt(T);
+    double mu = 0.0, lam = 0.0;
+    for (int k = l; k < N; k += G) {
+        const double rk = rs[k];
+        const double2 *t0 = reinterpret_cast<const double2 *>(tb.wilke + (size_t)k * Np);
+        const double2 *d0 = reinterpret_cast<const double2 *>(tb.diff + (size_t)k * Np);
+        const size_t s2 = (size_t)N * Np / 2;
+        double den = 0.0, ds = 0.0, gs = 0.0;
+        for (int j = 0; j < N; j += 2) {                      // tables are padded with zeros to Np
+            const double2 w0 = __ldg(t0 + j / 2), w1 = __ldg(t0 + s2 + j / 2), w2 = __ldg(t0 + 2 * s2 + j / 2);
+            const double2 g0 = __ldg(d0 + j / 2), g1 = __ldg(d0 + s2 + j / 2), g2 = __ldg(d0 + 2 * s2 + j / 2),
+                          g3 = __ldg(d0 + 3 * s2 + j / 2), g4 = __ldg(d0 + 4 * s2 + j / 2);
+            const double xa = xs[j], ta = rk * is[j];
+            den = fma(fma(ta, fma(ta, w2.x, w1.x), w0.x), xa, den);
+            const double ga = fma(fma(fma(fma(g4.x, x, g3.x), x, g2.x), x, g1.x), x, g0.x);
+            ds = fma(ga, xa, ds);
+            gs += ga;
+            if (j + 1 < N) {
+                const double xb = xs[j + 1], tb2 = rk * is[j + 1];
+                den = fma(fma(tb2, fma(tb2, w2.y, w1.y), w0.y), xb, den);
+                const double gb = fma(fma(fma(fma(g4.y, x, g3.y), x, g2.y), x, g1.y), x, g0.y);
+                ds = fma(gb, xb, ds);
+                gs += gb;
+            }
+        }
+        const double *a = tb.nasa_cp + (rng * N + k) * 5;
+        const double cpR = fma(fma(fma(fma(__ldg(a + 4), T, __ldg(a + 3)), T, __ldg(a + 2)), T, __ldg(a + 1)), T, __ldg(a));
+        const double wk = xs[k] / den * (rk * rk);            // X_k mu_k / sum_j X_j Phi_kj
+        mu += wk;
+        lam = fma(wk, (cpR + 1.25) * kR * __ldg(tb.invW + k), lam);   // Eucken
+        if (Dkg && valid) {
+            const double y = Yg[(int64_t)k * ld + i], Xk = xs[k] * Wbar;
+            ds *= Wbar;
+            Dkg[(int64_t)k * ld + i] = pure_species(Xk, y, ds, gs, N) ? T15 / (p * gs / double(N - 1)) : (1.0 - y) * T15 / (p * ds);
+        }
+    }
+    mu = group_sum(mu);
+    lam = group_sum(lam);
+    if (l == 0 && valid) {
+        if (mug) mug[i] = mu;
+        if (lamg) lamg[i] = lam;
+    }
+}
+
+template <int G>
+int launch_props_split(const chem_mech *m, int64_t ncells, int64_t ld, const void *T, const void *p, const void *Y,
+                       void *cp, void *h, void *mu, void *lam, void *Dk, cudaStream_t st) {
+    const int per = 128 / G;
+    void *pb = prof_begin(st);
+    props_split_kernel<G><<<(unsigned)((ncells + per - 1) / per), 128, (size_t)per * 3 * m->N * sizeof(double), st>>>(
+        m->N, m->dev.Np, m->T_mid, m->dev.f64, ncells, ld, static_cast<const double *>(T), static_cast<const double *>(p),
+        static_cast<const double *>(Y), static_cast<double *>(cp), static_cast<double *>(h), static_cast<double *>(mu),
+        static_cast<double *>(lam), static_cast<double *>(Dk));
+    prof_end(pb, st, "props_kernel<f64>", (double)ncells * (16.0 * m->N * m->N + 30.0 * m->N),
+             (double)ncells * ((m->N + 2) * 8 + (4 + m->N) * 8));
+    return check_cuda(cudaGetLastError(), "props_eval launch");
+}
+
 // Thermo only (cp and h; the memory-bound part of props_eval), FP32 arithmetic,
 // with the state staged through shared memory by bulk copies.
 //
@@ -1033,6 +1149,20 @@ int dispatch_props(const chem_mech *m, int64_t ncells, int64_t ld, const void *T
             return launch_props_tc<in_t, 64>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
         }
     } else {
+        // the fewest threads per cell that give every SM kSplitWarps warps, at most one per species
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int64_t want = (int64_t)sms * kSplitWarps * 32;
+        if (ncells < want && m->N >= 4) {
+            if (ncells * 4 >= want || m->N < 8)
+                return launch_props_split<4>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+            if (ncells * 8 >= want || m->N < 16)
+                return launch_props_split<8>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+            if (ncells * 16 >= want || m->N < 24)
+                return launch_props_split<16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+            return launch_props_split<32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+        }
         if (m->N <= 16) return launch_props<real, in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
         if (m->N <= 32) return launch_props<real, in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
     }
