@@ -4,7 +4,7 @@
 // replaces).
 //
 // Design for sm_103a:
-//  - One warp per cell. Cells are popped from a device work queue (one atomic
+//  - One warp per cell, or two (many cells of up to 15 species). Cells are popped from a device work queue (one atomic
 //    per cell), so cells with very different step counts balance across the
 //    persistent grid.
 //  - The state vector y = (T, Y_1..Y_N) is distributed over the lanes:
@@ -27,7 +27,7 @@
 //    8 warps per SM) took 54,000 warp instructions and 1,600 FP64 ones a step of the
 //    30-species mixed mode, with the FP64 pipe 44 % busy; this one 30,000 and 1,350 at 16
 //    warps per SM (12 KB each), 60 %. 65,536 cells at rtol 1e-2: 148 -> 87 ms; 4,096
-//    cells of the 9-species mechanism in FP64 at rtol 1e-6: 111 -> 76 ms; the 2 % fallback
+//    cells of the 9-species mechanism in FP64 at rtol 1e-6: 111 -> 76 ms, with two per warp 57 ms; the 2 % fallback
 //    of 262,144 learned cells: 14.5 -> 9.1 ms.
 //  - Few cells (at most one per SM, e.g. the learned step's out-of-distribution
 //    cells): a team of kWarps warps integrates each cell, one per SM
@@ -62,32 +62,37 @@ constexpr double kGam = 0.5;
 // a31 = a41 = 2, a43 = 1, the others 0; m = (2, 0, 1, 1), e = (0, 0, 0, 1)
 constexpr double kC21 = 4.0, kC31 = 1.0, kC32 = -1.0, kC41 = 1.0, kC42 = -1.0, kC43 = -8.0 / 3.0;
 
+// Lanes per cell, LPC: 32, or 16 with two cells in the halves of a warp (n <= 16). Every shuffle is a whole
+// warp's; sums over 16 lanes have the bits of sums over 32 whose upper lanes hold zeros.
+template <int LPC>
 __device__ __forceinline__ double warp_sum(double v) {
     // butterfly: every lane ends with the same bits (addition is commutative)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    for (int o = LPC / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
 }
 // Two (four) sums in one butterfly: the halves (quarters) of the warp carry one sum each, so the FP64
 // pipe sees 5 (6) additions instead of 10 (20). Every lane ends with all of them.
+template <int LPC>
 __device__ __forceinline__ void warp_sum2(double &a, double &b, int lane) {
-    const bool up = lane & 16;
-    double v = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, 16);
+    const bool up = lane & (LPC / 2);
+    double v = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, LPC / 2);
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    a = __shfl_sync(kFull, v, 0);
-    b = __shfl_sync(kFull, v, 16);
+    for (int o = LPC / 4; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0, LPC);
+    b = __shfl_sync(kFull, v, LPC / 2, LPC);
 }
+template <int LPC>
 __device__ __forceinline__ void warp_sum3(double &a, double &b, double &c, int lane) {
-    const bool up = lane & 16, mid = lane & 8;
-    const double ab = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, 16);
-    const double cc = c + __shfl_xor_sync(kFull, c, 16);
-    double v = (mid ? cc : ab) + __shfl_xor_sync(kFull, mid ? ab : cc, 8);
+    const bool up = lane & (LPC / 2), mid = lane & (LPC / 4);
+    const double ab = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, LPC / 2);
+    const double cc = c + __shfl_xor_sync(kFull, c, LPC / 2);
+    double v = (mid ? cc : ab) + __shfl_xor_sync(kFull, mid ? ab : cc, LPC / 4);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    a = __shfl_sync(kFull, v, 0);
-    b = __shfl_sync(kFull, v, 16);
-    c = __shfl_sync(kFull, v, 8);
+    for (int o = LPC / 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0, LPC);
+    b = __shfl_sync(kFull, v, LPC / 2, LPC);
+    c = __shfl_sync(kFull, v, LPC / 4, LPC);
 }
 
 // The warps integrating one cell: W = 1 (a lone warp) or W = kWarps (the block).
@@ -234,13 +239,13 @@ __device__ __forceinline__ double exp_mx(double x) { return f32_to_f64_int(expf(
 
 // f = f(y) for the warp's cell. JAC: also what build_matrix needs. MX (the mixed mode): the rate
 // constants' exponentials and the fall-off blending in FP32, the rest FP64.
-template <int W, int NS, bool MX, bool JAC>
+template <int W, int NS, bool MX, bool JAC, int LPC = 32>
 __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &sh, Team<W> tm, int lane, double p,
                                              double Rinvp, const double (&y)[NS], double (&f)[NS]) {
     using mreal = typename Slice<MX>::mreal;
     const int N = m.N, R = m.R, n = N + 1;
     EvalInfo info;
-    const double T = __shfl_sync(kFull, y[0], 0);
+    const double T = __shfl_sync(kFull, y[0], 0, LPC);
     const double invT = 1.0 / T;
     const double lnT = log(T);
     info.T = T;
@@ -281,8 +286,8 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
             if (JAC) dcp += yw * (a1 + T * (2.0 * a2 + T * (3.0 * a3 + T * 4.0 * a4)));
         }
     }
-    if (JAC) warp_sum3(S, cp, dcp, lane);
-    else warp_sum2(S, cp, lane);
+    if (JAC) warp_sum3<LPC>(S, cp, dcp, lane);
+    else warp_sum2<LPC>(S, cp, lane);
     cp *= kR;
     const double Wbar = 1.0 / S;
     const double rho = p * invT * Wbar * (1.0 / kR);
@@ -312,7 +317,7 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
     tm.sync();
     // reaction pass (thread per reaction over the team's lanes)
     const double lnPRT = m.lnPR - lnT;
-    for (int j = tm.wt * 32 + lane; j < R; j += 32 * W) {
+    for (int j = tm.wt * 32 + lane; j < R; j += LPC * W) {
         const uint2 sp = __ldg(m.rspec + j);
         const int r0 = sp.x & 255, r1 = (sp.x >> 8) & 255, p0 = sp.y & 255, p1 = (sp.y >> 8) & 255;
         const double beta = __ldg(m.beta + j), EaR = __ldg(m.EaR + j);
@@ -469,7 +474,7 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
             Q += H * RT * w[s];
         }
     }
-    Q = warp_sum(Q);
+    Q = warp_sum<LPC>(Q);
     info.Q = Q;
     if (lane == 0) f[0] = MX ? -Q / (rho * cp) : -(Q * invrho) / cp;
     return info;
@@ -487,7 +492,7 @@ __device__ __forceinline__ double mul_sub(double a, double b, double c, double d
 // the Jacobian then carries FP32 rounding, about 1e-7 relative, which the mixed mode's loose
 // tolerances absorb). In a team the entry lists and the third-body rows are split over the warps and
 // the first warp does the rest.
-template <int W, int NS, bool MX>
+template <int W, int NS, bool MX, int LPC = 32>
 __device__ void build_matrix(const DevMech &m, const Slice<MX> &sh, Team<W> tm, int lane, const EvalInfo &in, double ih) {
     using real = typename Slice<MX>::mreal;
     const int N = m.N, n = N + 1;
@@ -502,14 +507,18 @@ __device__ void build_matrix(const DevMech &m, const Slice<MX> &sh, Team<W> tm, 
     // sparse part of JC = d wdot / d C: an entry per lane, its reactions ascending
     const unsigned *ell = MX ? m.ell_f : m.ell_d;
     for (int q = tm.wt; q < m.ell_groups; q += W) {
-        const int pos = __ldg(m.ell_pos + 32 * q + lane), len = __ldg(m.ell_len + q);
-        const unsigned *p = ell + __ldg(m.ell_off + q) + lane;
-        real acc = 0;
-        for (int t = 0; t < len; ++t) {
-            const unsigned e = __ldg(p + 32 * t);
-            if (e >> 16) acc += code_value<real>(e) * sh.rdq[e & 0xFFFFu];
+        const int len = __ldg(m.ell_len + q);
+#pragma unroll
+        for (int half = 0; half < 32; half += LPC) {
+            const int pos = __ldg(m.ell_pos + 32 * q + half + lane);
+            const unsigned *p = ell + __ldg(m.ell_off + q) + half + lane;
+            real acc = 0;
+            for (int t = 0; t < len; ++t) {
+                const unsigned e = __ldg(p + 32 * t);
+                if (e >> 16) acc += code_value<real>(e) * sh.rdq[e & 0xFFFFu];
+            }
+            if (pos >= 0) G[pos] = acc;
         }
-        if (pos >= 0) G[pos] = acc;
     }
     tm.sync();
     // dense third-body part: row k takes nu_kj (rop dF/dM)_j eff_j of its reactions j, columns over lanes
@@ -586,7 +595,7 @@ __device__ void build_matrix(const DevMech &m, const Slice<MX> &sh, Team<W> tm, 
             sT += mul_add(sh.cpR[mm] * Rr, wm, sh.HR[mm], dwdT);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sT += __shfl_xor_sync(kFull, sT, o);
+        for (int o = LPC / 2; o > 0; o >>= 1) sT += __shfl_xor_sync(kFull, sT, o);
         if (lane == 0) G[0] = ghinv + sT * invrcp + qq * (cp * invT - dcpdT);
     }
     tm.sync();
@@ -615,9 +624,38 @@ __device__ __forceinline__ int pivot_lane(double v, bool valid, int pos, int lan
     return __ffs(__ballot_sync(kFull, cand && (unsigned)pos == first)) - 1;
 }
 
+// The same over 16 lanes (both halves of the warp at once): values as 64-bit keys, four shuffle steps.
+__device__ __forceinline__ int pivot_lane16(unsigned long long key, int pos, int lane) {
+    unsigned long long best = key;
+    int first = key ? pos : 64;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        const unsigned long long ob = __shfl_xor_sync(kFull, best, o);
+        const int of = __shfl_xor_sync(kFull, first, o);
+        if (ob > best || (ob == best && of < first)) {
+            best = ob;
+            first = of;
+        }
+    }
+    const unsigned who = __ballot_sync(kFull, key == best && pos == first && key != 0);
+    return (best == 0 || first == 64) ? -1 : __ffs((who >> (threadIdx.x & 16)) & 0xFFFFu) - 1;
+}
+__device__ __forceinline__ int pivot_lane16(double v, bool valid, int pos, int lane) {
+    const unsigned long long k = (unsigned long long)__double_as_longlong(v);
+    const int p = pivot_lane16(valid && k <= 0x7FF0000000000000ull ? k : 0ull, pos, lane);   // NaN: no candidate
+    const double top = __shfl_sync(kFull, v, p < 0 ? 0 : p, 16);
+    return p < 0 || __double2hiint(top) >= 0x7FF00000 ? -1 : p;
+}
+__device__ __forceinline__ int pivot_lane16(float v, bool valid, int pos, int lane) {
+    const unsigned k = __float_as_uint(v);
+    const int p = pivot_lane16(valid && k <= 0x7F800000u ? (unsigned long long)k : 0ull, pos, lane);
+    const float top = __shfl_sync(kFull, v, p < 0 ? 0 : p, 16);
+    return p < 0 || __float_as_uint(top) >= 0x7F800000u ? -1 : p;
+}
+
 // LU with partial pivoting of an n x n matrix, n <= NC <= 32, in registers: lane i holds row i of the
 // matrix, then (moved once, after the factorisation) the factors' row of its pivoted place i.
-template <typename real, int NC>
+template <typename real, int NC, int LPC = 32>
 struct RowLU {
     real row[NC];
     real rinv;                 // reciprocal pivot of this lane's row
@@ -632,16 +670,22 @@ struct RowLU {
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
-            if (k < n && ok) {
-                const int p = pivot_lane((real)fabs(row[k]), pos >= k && lane < n, pos, lane);
+            if (k < n && (LPC == 16 || ok)) {
+                int p;
+                if constexpr (LPC == 16) {
+                    p = pivot_lane16((real)fabs(row[k]), pos >= k && lane < n, pos, lane);
+                    if (p < 0) { ok = false; p = 0; }     // the other half goes on: this one's result is not used
+                } else {
+                    p = pivot_lane((real)fabs(row[k]), pos >= k && lane < n, pos, lane);
+                }
                 if (p < 0) {
                     ok = false;
                 } else {
-                    const int was = __shfl_sync(kFull, pos, p);
+                    const int was = __shfl_sync(kFull, pos, p, LPC);
                     if (pos == k) pos = was;          // the row that stood there takes the pivot's place
                     if (lane == p) pos = k;
                     if (lane == k) mine = p;
-                    const real rp = (real)1 / __shfl_sync(kFull, row[k], p);
+                    const real rp = (real)1 / __shfl_sync(kFull, row[k], p, LPC);
                     if (lane == p) rinv = rp;
                     const bool below = pos > k;
                     if (below) row[k] *= rp;
@@ -651,7 +695,7 @@ struct RowLU {
 #pragma unroll
                             for (int c = cb; c < cb + 4; ++c)
                                 if (c > k) {
-                                    const real akc = __shfl_sync(kFull, row[c], p);
+                                    const real akc = __shfl_sync(kFull, row[c], p, LPC);
                                     if (below) row[c] -= row[k] * akc;
                                 }
                         }
@@ -661,8 +705,8 @@ struct RowLU {
         }
 #pragma unroll
         for (int c = 0; c < NC; ++c)
-            if (c < n) row[c] = __shfl_sync(kFull, row[c], mine);
-        rinv = __shfl_sync(kFull, rinv, mine);
+            if (c < n) row[c] = __shfl_sync(kFull, row[c], mine, LPC);
+        rinv = __shfl_sync(kFull, rinv, mine, LPC);
         if constexpr (sizeof(real) == 8) {
             // FP64: the rows of U divided by their pivots once, instead of each unknown in every solve
 #pragma unroll
@@ -674,11 +718,11 @@ struct RowLU {
 
     // x = A^-1 b, component c in lane c
     __device__ __forceinline__ real solve(real b, int lane, int n) const {
-        b = __shfl_sync(kFull, b, mine);
+        b = __shfl_sync(kFull, b, mine, LPC);
 #pragma unroll
         for (int k = 0; k < NC - 1; ++k) {
             if (k < n - 1) {
-                const real bk = __shfl_sync(kFull, b, k);
+                const real bk = __shfl_sync(kFull, b, k, LPC);
                 if (lane > k) b -= row[k] * bk;
             }
         }
@@ -689,7 +733,7 @@ struct RowLU {
                 if constexpr (sizeof(real) == 4) {
                     if (lane == k) b *= rinv;
                 }
-                const real bk = __shfl_sync(kFull, b, k);
+                const real bk = __shfl_sync(kFull, b, k, LPC);
                 if (lane < k) b -= row[k] * bk;
             }
         }
@@ -797,11 +841,11 @@ __device__ void tri_solve(const int *piv, const real *G, const real *invd, real 
 }
 
 // The factored system of one step: NC <= 32 in registers, NC = 64 in shared memory.
-template <int W, int NC, bool MX>
+template <int W, int NC, bool MX, int LPC = 32>
 struct Factors {
     using real = typename Slice<MX>::mreal;
     static constexpr bool kBig = NC > 32;
-    typename std::conditional<kBig, int, RowLU<real, kBig ? 4 : NC>>::type lu;
+    typename std::conditional<kBig, int, RowLU<real, kBig ? 4 : NC, LPC>>::type lu;
 
     __device__ __forceinline__ bool factor(const Slice<MX> &sh, Team<W> tm, int lane, int n) {
         if constexpr (kBig) {
@@ -990,7 +1034,7 @@ __device__ __forceinline__ void integrate_cells(const DevMech &m, char *smem, in
                     if (!isfinite(v) || !isfinite(e)) nonfinite = true;
                 }
             }
-            acc = warp_sum(acc);
+            acc = warp_sum<32>(acc);
             nonfinite = __any_sync(kFull, nonfinite);
             // The mixed mode's exponentials cut their FP64 arguments to FP32: where a last-bit change of T
             // or of the step moves an argument across a cut, a rate jumps by 2e-6 and T by up to 6e-8. So
@@ -1031,6 +1075,152 @@ __device__ __forceinline__ void integrate_cells(const DevMech &m, char *smem, in
     }
 }
 
+// The same for n <= 16 with two cells per warp, one in each half (16 lanes): the FP64 pipe, which counts warp
+// instructions, then serves two cells with each. The halves run their steps in lock step; one that
+// has finished its cell (or finds its step rejected) goes on with its own next cell or step, so neither
+// waits for the other's step count. Operations and orders per cell are those of integrate_cells.
+template <int NC, bool MX>
+__device__ __forceinline__ void integrate_halves(const DevMech &m, char *smem, int64_t limit, int64_t ld, double dt,
+                                                 const chem_ode_opts &o, double *__restrict__ Tg,
+                                                 const double *__restrict__ pg, double *__restrict__ Yg,
+                                                 int32_t *__restrict__ status, int32_t *__restrict__ nsteps_out,
+                                                 unsigned int *__restrict__ queue, const int32_t *__restrict__ list,
+                                                 int ok_status) {
+    static_assert(NC <= 16, "a cell's components in 16 lanes");
+    const int lane = threadIdx.x & 15, slot = threadIdx.x >> 4;
+    const unsigned half = 0xFFFFu << (threadIdx.x & 16);
+    const int N = m.N, n = N + 1;
+    const Team<1> tm{0};
+    Slice<MX> sh;
+    make_slice<MX, false>(smem + (size_t)slot * make_slice<MX, false>(nullptr, N, m.R, m.n_tb, m.nslot, nullptr), N, m.R,
+                          m.n_tb, m.nslot, &sh);
+    const double rn = 1.0 / (double)n;
+    bool have = false, done = false;
+    int64_t cell = 0;
+    double y[1] = {lane == 0 ? 1000.0 : rn}, p = 101325.0, t = 0.0, h = dt;     // a state for an idle half to run on
+    int nst = 0, rejected_last = 0, stat = CHEM_CELL_OK;
+    for (;;) {
+        if (!have && !done) {
+            unsigned int pos = 0;
+            if (lane == 0) pos = atomicAdd(queue, 1u);
+            pos = __shfl_sync(half, pos, 0, 16);
+            if ((int64_t)pos < limit) {
+                cell = list ? (int64_t)list[pos] : (int64_t)pos;
+                y[0] = (lane == 0) ? Tg[cell] : (lane < n ? Yg[(int64_t)(lane - 1) * ld + cell] : 0.0);
+                p = pg[cell];
+                t = 0.0;
+                h = (o.h0 < dt) ? o.h0 : dt;
+                nst = 0;
+                rejected_last = 0;
+                stat = CHEM_CELL_OK;
+                have = true;
+            } else {
+                done = true;
+            }
+        }
+        __syncwarp();
+        if (__all_sync(kFull, done)) break;
+        bool fin = false;
+        if (have) {
+            if (nst >= o.max_steps) { stat = CHEM_CELL_MAXSTEPS; fin = true; }
+            else if (h < 1e-20 * dt) { stat = CHEM_CELL_UNDERFLOW; fin = true; }
+        }
+        if (!__any_sync(kFull, fin)) {
+            const double rem = dt - t;
+            bool last = false;
+            if (h >= rem) { h = rem; last = true; }
+            const double Rinvp = kR / p;
+            double f0[1];
+            const EvalInfo info = eval_rhs<1, 1, MX, true, 16>(m, sh, tm, lane, p, Rinvp, y, f0);
+            const bool bad = (__ballot_sync(kFull, lane < n && !isfinite(f0[0])) & half) != 0;
+            const double ih = 1.0 / h;
+            build_matrix<1, 1, MX, 16>(m, sh, tm, lane, info, ih);
+            Factors<1, NC, MX, 16> A;
+            const bool ok = A.factor(sh, tm, lane, n);
+            double K1 = 0.0, K2 = 0.0, K3 = 0.0, K4 = 0.0;
+#pragma unroll 1
+            for (int st = 0; st < 4; ++st) {
+                double v[1] = {f0[0]};
+                if (st >= 2) {
+                    const double ys[1] = {y[0] + 2.0 * K1 + K3};
+                    eval_rhs<1, 1, MX, false, 16>(m, sh, tm, lane, p, Rinvp, ys, v);
+                }
+                if (st >= 1) v[0] += ((st == 1 ? kC21 : (st == 2 ? kC31 : kC41)) * ih) * K1;
+                if (st >= 2) {
+                    v[0] += ((st == 2 ? kC32 : kC42) * ih) * K2;
+                    v[0] += ((st == 3 ? kC43 : 0.0) * ih) * K3;
+                }
+                A.solve(sh, sh.xs, lane, n, v);
+                if (st == 0) K1 = v[0];
+                else if (st == 1) K2 = v[0];
+                else if (st == 2) K3 = v[0];
+                else K4 = v[0];
+            }
+            // y_new = y + 2 K1 + K3 + K4, error = K4
+            double acc = 0.0, yn = 0.0;
+            bool nonfinite = false;
+            if (lane < n) {
+                double v = y[0];
+                v += 2.0 * K1;
+                v += K3;
+                v += K4;
+                yn = v;
+                const double ay = fabs(y[0]), ayn = fabs(v);
+                const double sc = ((lane == 0) ? o.atol_T : o.atol_Y) + o.rtol * (ay > ayn ? ay : ayn);
+                const double r = K4 / sc;
+                acc = r * r;
+                nonfinite = !isfinite(v) || !isfinite(K4);
+            }
+            acc = warp_sum<16>(acc);
+            nonfinite = (__ballot_sync(kFull, nonfinite) & half) != 0;
+            double err = sqrt(MX ? acc / (double)n : acc * rn);
+            double fac;
+            if (nonfinite || !isfinite(err)) {
+                fac = 0.2;
+                err = 2.0;
+            } else {
+                fac = (err > 0.0) ? 0.9 * (MX ? pow(err, -1.0 / 3.0) : rcbrt(err)) : 5.0;
+                fac = fmin(5.0, fmax(0.2, fac));
+            }
+            if (have) {
+                if (bad) {
+                    stat = CHEM_CELL_NONFINITE;
+                    fin = true;
+                } else {
+                    ++nst;
+                    if (!ok) {
+                        h *= 0.2;
+                        rejected_last = 1;
+                    } else if (err <= 1.0) {
+                        t = last ? dt : t + h;
+                        y[0] = yn;
+                        if (rejected_last && fac > 1.0) fac = 1.0;
+                        h *= fac;
+                        rejected_last = 0;
+                        fin = !(t < dt);
+                    } else {
+                        h *= fac;
+                        rejected_last = 1;
+                    }
+                }
+            }                                // an idle half's state stays as it is
+        }
+        if (fin) {
+            if (lane == 0) {
+                Tg[cell] = y[0];
+                status[cell] = (stat == CHEM_CELL_OK) ? ok_status : stat;
+                if (nsteps_out) nsteps_out[cell] = nst;
+            } else if (lane < n) {
+                Yg[(int64_t)(lane - 1) * ld + cell] = y[0];
+            }
+            have = false;
+            t = 0.0;
+            h = dt;
+        }
+        __syncwarp();
+    }
+}
+
 // Blocks that take a cell each in team mode: one per SM (the first blocks of a
 // grid are spread over the SMs), at most the grid.
 inline int team_blocks(int sms, int blocks) { return sms < blocks ? sms : blocks; }
@@ -1044,14 +1234,14 @@ constexpr int kBigWarps = 8;         // most warps of a block above 31 species
 // device-built queue; status of a successful cell = ok_status. When the cells
 // number at most team_blocks, the first team_blocks blocks integrate them with
 // kWarps warps per cell and the other blocks return at once; otherwise
-// every warp takes cells of its own.
+// every warp takes cells of its own, from halves_from cells on one in each half.
 template <int NC, bool MX>
 __global__ void __launch_bounds__(NC > 32 ? 32 * kBigWarps : 32 * kWarps, stiff_min_blocks(NC, MX))
     stiff_kernel(const __grid_constant__ DevMech m, int64_t ncells, int64_t ld, double dt, chem_ode_opts o,
                  double *__restrict__ Tg, const double *__restrict__ pg, double *__restrict__ Yg,
                  int32_t *__restrict__ status, int32_t *__restrict__ nsteps_out, unsigned int *__restrict__ queue,
                  const int32_t *__restrict__ list, const unsigned int *__restrict__ list_count, int ok_status,
-                 int team_blocks) {
+                 int team_blocks, int64_t halves_from) {
     extern __shared__ __align__(16) char smem_raw[];
     int *blk_pos = reinterpret_cast<int *>(smem_raw);
     char *smem = smem_raw + kSmemHeader;
@@ -1061,10 +1251,17 @@ __global__ void __launch_bounds__(NC > 32 ? 32 * kBigWarps : 32 * kWarps, stiff_
         if ((int)blockIdx.x >= team_blocks || threadIdx.x >= 32 * kWarps) return;
         integrate_cells<kWarps, NC, MX>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue,
                                         list, ok_status);
-    } else {
-        integrate_cells<1, NC, MX>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
-                                   ok_status);
+        return;
     }
+    if constexpr (NC <= 16) {
+        if (limit >= halves_from) {
+            integrate_halves<NC, MX>(m, smem, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
+                                     ok_status);
+            return;
+        }
+    }
+    integrate_cells<1, NC, MX>(m, smem, blk_pos, limit, ld, dt, o, Tg, pg, Yg, status, nsteps_out, queue, list,
+                               ok_status);
 }
 
 // The launch of one kernel variant: warps per block and resident blocks for this mechanism.
@@ -1078,7 +1275,9 @@ int launch_stiff_nc(const chem_mech *m, int64_t capacity, int64_t ld, double dt,
     // above 31 species one block of up to kBigWarps warps where two blocks of kWarps do not fit
     if (NC > 32 && 2 * (kSmemHeader + kWarps * slice) > kSmemMax)
         while (warps < kBigWarps && kSmemHeader + (warps + 1) * slice <= kSmemMax) ++warps;
-    const size_t smem = kSmemHeader + slice * warps;
+    // two slices per warp, where they cost no resident block
+    const bool halves = NC <= 16 && stiff_min_blocks(NC, MX) * (kSmemHeader + 2 * kWarps * slice) <= kSmemMax;
+    const size_t smem = kSmemHeader + slice * (halves ? 2 * warps : warps);
     if (smem > kSmemMax)
         return set_error(CHEM_EUNSUPPORTED, std::string(who) + ": mechanism too large for shared memory");
     auto kernel = stiff_kernel<NC, MX>;
@@ -1095,8 +1294,13 @@ int launch_stiff_nc(const chem_mech *m, int64_t capacity, int64_t ld, double dt,
     if (blocks < 1) blocks = 1;
     rc = check_cuda(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st), who);
     if (rc) return rc;
+    // Two cells per warp from 5/4 cells per resident warp on. Below, a warp of its own ends each cell sooner
+    // than the pipe, shared by fewer warps, gains. 9 species, one / two cells per warp: FP64 mode (1,824
+    // warps) rtol 1e-6 1,824 cells 38.0 / 39.3 ms, 2,600 54.3 / 47.4, 16,384 261 / 169; mixed mode (2,432
+    // warps) 2,600 cells 1.66 / 1.73 ms, 4,096 2.36 / 1.81, 16,384 8.2 / 5.1.
+    const int64_t from = halves ? (int64_t)sms * per_sm * warps * 5 / 4 : INT64_MAX;
     kernel<<<blocks, warps * 32, smem, st>>>(m->dev, capacity, ld, dt, o, T, p, Y, status, nsteps, queue, list, count,
-                                             ok_status, team_blocks(sms, blocks));
+                                             ok_status, team_blocks(sms, blocks), from);
     return check_cuda(cudaGetLastError(), who);
 }
 
