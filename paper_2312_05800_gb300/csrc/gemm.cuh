@@ -14,9 +14,13 @@
 //               accumulating in one of two TMEM buffers (columns 0 and 256).
 //   warps 2..17 epilogue: four warps per TMEM lane quadrant (warp w reads TMEM
 //               lanes 32 (w % 4) .. +31, i.e. output rows) split the 16-column
-//               chunks between them; tcgen05.ld, then the functor. BF16 or
-//               E4M3 GELU outputs are staged per warp in shared memory (double
-//               buffered) and written by TMA tensor stores.
+//               chunks (E4M3 outputs: pairs of them) between them; tcgen05.ld,
+//               then the functor. BF16 or E4M3 GELU outputs are staged per warp
+//               in shared memory (double buffered) and written by TMA tensor
+//               stores of 32-byte row pieces, whole sectors: E4M3 chunks stored
+//               one by one, 16 bytes a row, cost 5 % of the 88-species forward
+//               (500,001 rows 2.16 -> 2.05 ms). BF16 pairs, 64-byte pieces, gain
+//               nothing (dense 544 / 542 us, learned step 20.98 / 21.06 ms).
 // B may also be stored [K][N] (the layer's own weights for the backward product dZ W): its k-blocks are
 // then boxes of 64 columns x 64 rows and the instruction takes it N-major.
 // Ragged M, N and K: TMA fills out-of-range operand elements with zeros, TMA
@@ -41,7 +45,7 @@ namespace chemgb {
 
 constexpr int kEpiWarps = 16;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
-constexpr uint32_t kStageBytesPerWarp = 32 * 16 * 2;   // one 32 x 16 BF16 chunk
+constexpr uint32_t kStageBytesPerWarp = 32 * 32;        // 32 rows x 16 BF16 or 32 E4M3 columns
 constexpr int kBM = 128;
 constexpr int kBK = 64;                     // BF16 elements per k-block row (128 bytes)
 constexpr int kBK8 = 128;                   // E4M3 elements per k-block row (128 bytes)
@@ -412,7 +416,7 @@ struct EpiGeluQ {
 template <int BN, int STAGES, class Epi>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tn_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmC, int M, int N, int K, GemmGroups grp, Epi epi, int *err) {
+                   const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC1, int M, int N, int K, GemmGroups grp, Epi epi, int *err) {
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "UMMA N for M = 128");
     static_assert(!Epi::kBNMajor || (BN % 64 == 0 && !Epi::kF8), "N-major B comes in boxes of 64 columns");
     using L = GemmSmem<BN, STAGES>;
@@ -541,8 +545,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             const Epi ge = epi.group(g);
             const int row0 = m_blk * kBM + quad * 32;
             const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * 256u;
+            // chunks of this warp: with kPer = 2, c = 2 group, 2 group + 1, then 2 group + 8, ...; a tile or the
+            // matrix may end after the first chunk of a pair, which then goes out by itself (map tmC1)
+            constexpr int kPer = 32 / Epi::kOutBytes;
 #pragma unroll 1
-            for (int c = group; c < BN / 16; c += kEpiWarps / 4) {
+            for (int c = kPer * group; c < BN / 16; c += kPer == 2 && !(c & 1) ? 1 : kPer * (kEpiWarps / 4) + 1 - kPer) {
                 const int col0 = n_blk * BN + c * 16;
                 if (col0 >= N) break;               // warp-uniform
                 float v[16];
@@ -551,16 +558,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     if (row0 >= M) continue;            // warp-uniform: nothing of this slice is in range
                     uint32_t w[8];
                     ge.compute(row0 + lane, col0, v, w);
+                    const bool second = kPer == 2 && (c & 1);
+                    const bool single = kPer == 2 && !second && (c + 1 >= BN / 16 || col0 + 16 >= N);
                     uint8_t *buf = my_stage + (nstore & 1) * kStageBytesPerWarp;
-                    if (nstore >= 2 && lane == 0) tc::bulk_wait_read<1>();   // this buffer's previous store has read it
-                    __syncwarp();
-                    uint4 *dst = reinterpret_cast<uint4 *>(buf + lane * Epi::kOutBytes);
-                    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (Epi::kOutBytes == 32) dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    if (!second) {
+                        if (nstore >= 2 && lane == 0) tc::bulk_wait_read<1>();   // this buffer's previous store has read it
+                        __syncwarp();
+                    }
+                    uint4 *dst = reinterpret_cast<uint4 *>(buf + lane * (single ? 16 : 32));
+                    dst[second ? 1 : 0] = make_uint4(w[0], w[1], w[2], w[3]);
+                    if (kPer == 1) dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    if (kPer == 2 && !second && !single) continue;
                     tc::fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
-                        store_tile(&tmC, buf, grp.c, col0, row0, g);
+                        store_tile(single ? &tmC1 : &tmC, buf, grp.c, second ? col0 - 16 : col0, row0, g);
                         tc::bulk_commit();
                     }
                     ++nstore;

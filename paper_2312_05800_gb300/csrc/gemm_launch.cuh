@@ -116,13 +116,14 @@ inline int num_sms() {
 }
 
 // Output tensor map for the TMA-store epilogue: [rows][cols] of BF16 (esize 2)
-// or E4M3 (esize 1), box 32 rows x 16 columns, no swizzle.
-inline int make_tmap_out(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld, int esize) {
+// or E4M3 (esize 1), box 32 rows x box_cols columns, no swizzle.
+inline int make_tmap_out(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld, int esize,
+                         int box_cols) {
     if (!aligned16(ptr) || (ld * esize) % 16 != 0)
         return set_error(CHEM_EINVAL, "GEMM output: base must be 16-byte aligned and rows a multiple of 16 bytes");
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)(ld * esize)};
-    cuuint32_t box[2] = {16, 32};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, 32};
     cuuint32_t estr[2] = {1, 1};
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled_fn();
     if (!enc) return set_error(CHEM_EUNSUPPORTED, "cuTensorMapEncodeTiled is not available from the driver");
@@ -133,16 +134,16 @@ inline int make_tmap_out(CUtensorMap *map, const void *ptr, int64_t rows, int64_
     return CHEM_OK;
 }
 
-// Output map of a grouped TMA-store epilogue: box 32 rows x 16 columns of one group.
+// Output map of a grouped TMA-store epilogue: box 32 rows x box_cols columns of one group.
 inline int make_tmap_out_grouped(CUtensorMap *map, const void *ptr, int kind, int64_t rows, int64_t cols, int G,
-                                 int64_t ld, int64_t gstride, int esize) {
-    if (kind == kMap2D) return make_tmap_out(map, ptr, rows, cols, ld, esize);
+                                 int64_t ld, int64_t gstride, int esize, int box_cols) {
+    if (kind == kMap2D) return make_tmap_out(map, ptr, rows, cols, ld, esize, box_cols);
     if (!aligned16(ptr) || (ld * esize) % 16 != 0 || (gstride * esize) % 16 != 0 || gstride <= 0)
         return set_error(CHEM_EINVAL, "grouped GEMM output: base, row and group strides must be 16-byte multiples");
     const bool rowg = kind == kMapRowGrp;
     cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)(rowg ? rows : G), (cuuint64_t)(rowg ? G : rows)};
     cuuint64_t strides[2] = {(cuuint64_t)((rowg ? ld : gstride) * esize), (cuuint64_t)((rowg ? gstride : ld) * esize)};
-    cuuint32_t box[3] = {16, (cuuint32_t)(rowg ? 32 : 1), (cuuint32_t)(rowg ? 1 : 32)};
+    cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)(rowg ? 32 : 1), (cuuint32_t)(rowg ? 1 : 32)};
     cuuint32_t estr[3] = {1, 1, 1};
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled_fn();
     if (!enc) return set_error(CHEM_EUNSUPPORTED, "cuTensorMapEncodeTiled is not available from the driver");
@@ -170,15 +171,18 @@ int launch_gemm_grouped_bn(const GemmOperand &A, const GemmOperand &B, int G, in
         configured = true;
     }
     const int esize = Epi::kF8 ? 1 : 2;
-    CUtensorMap ta, tb, tc;
+    CUtensorMap ta, tb, tc, tc1;
     int rc = make_operand_map(&ta, A, M, K, G, kBM, esize);
     if (rc) return rc;
     // N-major B: [K][N], boxes of 64 columns x 64 rows
     rc = Epi::kBNMajor ? make_operand_map(&tb, B, K, N, G, kBK, esize) : make_operand_map(&tb, B, N, K, G, BN, esize);
     if (rc) return rc;
     std::memset(&tc, 0, sizeof(tc));
-    if (const void *op = epi.tma_ptr()) {
-        rc = make_tmap_out_grouped(&tc, op, out_kind, M, N, G, epi.ldo, out_gstride, Epi::kOutBytes / 16);
+    std::memset(&tc1, 0, sizeof(tc1));
+    if (const void *op = epi.tma_ptr()) {                    // 32-byte row pieces; one E4M3 chunk by itself
+        const int os = Epi::kOutBytes / 16;
+        rc = make_tmap_out_grouped(&tc, op, out_kind, M, N, G, epi.ldo, out_gstride, os, 32 / os);
+        if (!rc && os == 1) rc = make_tmap_out_grouped(&tc1, op, out_kind, M, N, G, epi.ldo, out_gstride, os, 16);
         if (rc) return rc;
     }
     const int64_t tiles64 = (int64_t)((M + kBM - 1) / kBM) * ((N + BN - 1) / BN) * G;
@@ -189,7 +193,7 @@ int launch_gemm_grouped_bn(const GemmOperand &A, const GemmOperand &B, int G, in
     if (tiles < grid) grid = tiles;
     const GemmGroups grp{G, A.kind, B.kind, out_kind, gemm_wait_limit()};
     void *pb = prof_begin(st);
-    gemm_tn_kernel<BN, STAGES, Epi><<<grid, kGemmThreads, L::kTotal, st>>>(ta, tb, tc, M, N, K, grp, epi, err);
+    gemm_tn_kernel<BN, STAGES, Epi><<<grid, kGemmThreads, L::kTotal, st>>>(ta, tb, tc, tc1, M, N, K, grp, epi, err);
     if (pb)
         prof_end(pb, st, "gemm_tn_kernel<" + std::to_string(BN) + (Epi::kF8 ? ",e4m3> " : "> ") +
                              (G > 1 ? std::to_string(G) + "x" : std::string()) + std::to_string(N) + "x" +
