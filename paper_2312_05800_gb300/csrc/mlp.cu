@@ -2146,10 +2146,8 @@ extern "C" int chem_mlp_autotune(chem_mlp *m, int64_t rows, int32_t *tiles_out, 
         float best = 3.4e38f;
         int best_bn = L.tile;
         best_ms[l] = 0.0f;
-        // the two-CTA variant is not a candidate: measured on GB300 it runs at half the single-CTA rate
-        const std::vector<int> codes(std::begin(kTileWidths), std::end(kTileWidths));
-        for (int bn : codes) {
-            const int w = bn & 0xFFFF;
+        for (int bn : kTileWidths) {
+            const int w = bn;
             if (w < 64 && width > 64) continue;
             if (w > 2 * ((width + 15) / 16) * 16 && w > 64) continue;   // tiles far wider than the layer
             float ms_sum = 0.0f;
