@@ -30,7 +30,7 @@ int launch_fused34_nb(const void *X, int64_t ldx, int K3, const void *W3, int64_
     if (m_tiles < grid) grid = m_tiles;
     const F34Args a{M, K3, NA + NB, N4, b3, b4, u, ldu, gemm_wait_limit()};
     void *pb = prof_begin(st);
-    gemm_fused34_kernel<NA, NB><<<grid, kF34Threads, L::kTotal, st>>>(tx, t3a, t3b, t4, a, err);
+    launch_dependent(gemm_fused34_kernel<NA, NB>, m_tiles, grid, kF34Threads, L::kTotal, st, tx, t3a, t3b, t4, a, err);
     if (pb)
         prof_end(pb, st, "gemm_fused34_kernel " + std::to_string(NA + NB) + "x" + std::to_string(K3) + "+" +
                              std::to_string(N4) + "x" + std::to_string(NA + NB),

@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(kF34Threads, 1)
         tc::tmem_alloc(tmem_slot, kTmemCols);
         tc::tmem_relinquish();
     }
+    tc::grid_trigger();
+    tc::grid_wait();
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) gemm_wgrad_kernel(const __grid_
         tc::tmem_alloc(tmem_slot, 256);
         tc::tmem_relinquish();
     }
+    tc::grid_wait();
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -192,7 +193,7 @@ int gemm_wgrad(const WgradLayer *layers, int count, int B, int *err, cudaStream_
         tiles += (L.out + 127) / 128 * p.n_tiles;
     }
     void *pb = prof_begin(st);
-    gemm_wgrad_kernel<<<tiles, kWgThreads, kWgSmem, st>>>(a, err);
+    launch_dependent(gemm_wgrad_kernel, tiles, tiles, kWgThreads, kWgSmem, st, a, err);
     if (pb) {
         double fl = 0.0, by = 0.0;
         for (int l = 0; l < count; ++l) {

@@ -151,6 +151,7 @@ __global__ void prologue_kernel(int64_t n, int64_t ld, const double *__restrict_
                                 const float *__restrict__ mu, const float *__restrict__ isd,
                                 __nv_bfloat16 *__restrict__ out) {
     extern __shared__ __align__(16) uint4 pro_smem[];        // [32][3 n_in_pad / 8 + 1]
+    tc::grid_trigger();
     const int lane = threadIdx.x & 31, j0 = (threadIdx.x >> 5) * 8, nc = n_in_pad / 8;
     const int pitch = kXTerms * nc + 1;
     const int64_t i0 = (int64_t)blockIdx.x * 32, i = i0 + lane;
@@ -514,6 +515,7 @@ __global__ void __launch_bounds__(128) l1_loss_kernel(int64_t B, const float *__
                                float *__restrict__ part, const double *__restrict__ Tc, PhysLoss ph) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    tc::grid_trigger();
     if (i >= B) return;                              // warp-uniform
     const int64_t c = idx ? (int64_t)idx[i] : i;
     const float invB = 1.0f / (float)B;
@@ -625,6 +627,7 @@ __global__ void phys_scales_reduce_kernel(int nblocks, int64_t n, const double *
 // Deterministic sum of the per-sample partials (one block, fixed order), then / B.
 __global__ void loss_reduce_kernel(int64_t B, const float *__restrict__ part, float *__restrict__ loss) {
     __shared__ float sh[256];
+    tc::grid_trigger();
     float a = 0.0f;
     for (int64_t i = threadIdx.x; i < B; i += blockDim.x) a += part[i];
     sh[threadIdx.x] = a;

@@ -11,6 +11,12 @@
 namespace chemgb {
 namespace tc {
 
+// Programmatic dependent launch. grid_wait: until the kernels before this one in the stream have ended and their
+// writes are visible (nothing to wait for unless launched by launch_dependent). grid_trigger: the next
+// kernel's blocks may take their places once every block of this kernel has started.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // try_wait iterations before a wait is declared failed (each try may suspend
 // the thread for a short hardware-defined time; this is seconds in total)
 constexpr uint32_t kSpinLimit = 1u << 22;
