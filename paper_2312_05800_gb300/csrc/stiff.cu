@@ -292,7 +292,7 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
     const double Wbar = 1.0 / S;
     const double rho = p * invT * Wbar * (1.0 / kR);
     // FP64 mode: 1 / rho without another division. The mixed mode keeps every FP64 rounding as it is
-    // (see the error norm below)
+    // (see stage_add)
     const double invrho = MX ? 1.0 / rho : Rinvp * (T * S);
     info.rho = rho;
     info.cp = cp;
@@ -916,6 +916,17 @@ struct Factors {
     }
 };
 
+// v + c k, a term of the right-hand sides of stages 3 and 4. In the mixed mode the product is rounded before it
+// is added (the FP64 mode fuses it): the mode's exponentials cut their FP64 arguments to FP32, so where a
+// last-bit change moves an argument across a cut, a rate jumps by 2e-6 and T by up to 6e-8. Fused here, one
+// step of h0 = 1e-9 differs by 1e-16 of T, but 20,000 integrations at rtol 1e-2 by up to 2e-7 of T and 4e-7 of a
+// species' maximum. Every rounding of that mode is therefore written out.
+template <bool MX>
+__device__ __forceinline__ double stage_add(double v, double c, double k) {
+    if constexpr (MX) return __dadd_rn(v, __dmul_rn(c, k));
+    else return v + c * k;
+}
+
 // Integrates cells popped from the work queue until it is exhausted; W warps per cell. MX: the
 // mixed mode (FP32 rate exponentials and fall-off blending; FP32 LU with one FP64 refinement).
 template <int W, int NC, bool MX>
@@ -991,17 +1002,17 @@ __device__ __forceinline__ void integrate_cells(const DevMech &m, char *smem, in
                     for (int s = 0; s < NS; ++s) ys[s] = y[s] + 2.0 * K1[s] + K3[s];
                     eval_rhs<W, NS, MX, false>(m, sh, tm, lane, p, Rinvp, ys, v);
                 }
-                if (st >= 1) {
-                    const double c1 = (st == 1 ? kC21 : (st == 2 ? kC31 : kC41)) * ih;
+                if (st == 1) {
 #pragma unroll
-                    for (int s = 0; s < NS; ++s) v[s] += c1 * K1[s];
+                    for (int s = 0; s < NS; ++s) v[s] = fma(kC21 * ih, K1[s], v[s]);
                 }
                 if (st >= 2) {
-                    const double c2 = (st == 2 ? kC32 : kC42) * ih, c3 = (st == 3 ? kC43 : 0.0) * ih;
+                    const double c1 = (st == 2 ? kC31 : kC41) * ih, c2 = (st == 2 ? kC32 : kC42) * ih;
+                    const double c3 = (st == 3 ? kC43 : 0.0) * ih;
 #pragma unroll
                     for (int s = 0; s < NS; ++s) {
-                        v[s] += c2 * K2[s];
-                        v[s] += c3 * K3[s];
+                        v[s] = stage_add<MX>(stage_add<MX>(v[s], c1, K1[s]), c2, K2[s]);
+                        v[s] = fma(c3, K3[s], v[s]);
                     }
                 }
                 A.solve(sh, xs, lane, n, v);
@@ -1036,9 +1047,7 @@ __device__ __forceinline__ void integrate_cells(const DevMech &m, char *smem, in
             }
             acc = warp_sum<32>(acc);
             nonfinite = __any_sync(kFull, nonfinite);
-            // The mixed mode's exponentials cut their FP64 arguments to FP32: where a last-bit change of T
-            // or of the step moves an argument across a cut, a rate jumps by 2e-6 and T by up to 6e-8. So
-            // that mode's FP64 operations are never reformulated, only the FP64 mode's.
+            // reformulated in the FP64 mode only (see stage_add)
             double err = sqrt(MX ? acc / (double)n : acc * rn);
             double fac;
             if (nonfinite || !isfinite(err)) {
@@ -1145,10 +1154,11 @@ __device__ __forceinline__ void integrate_halves(const DevMech &m, char *smem, i
                     const double ys[1] = {y[0] + 2.0 * K1 + K3};
                     eval_rhs<1, 1, MX, false, 16>(m, sh, tm, lane, p, Rinvp, ys, v);
                 }
-                if (st >= 1) v[0] += ((st == 1 ? kC21 : (st == 2 ? kC31 : kC41)) * ih) * K1;
+                if (st == 1) v[0] = fma(kC21 * ih, K1, v[0]);
                 if (st >= 2) {
-                    v[0] += ((st == 2 ? kC32 : kC42) * ih) * K2;
-                    v[0] += ((st == 3 ? kC43 : 0.0) * ih) * K3;
+                    const double c1 = (st == 2 ? kC31 : kC41) * ih, c2 = (st == 2 ? kC32 : kC42) * ih;
+                    v[0] = stage_add<MX>(stage_add<MX>(v[0], c1, K1), c2, K2);
+                    v[0] = fma((st == 3 ? kC43 : 0.0) * ih, K3, v[0]);
                 }
                 A.solve(sh, sh.xs, lane, n, v);
                 if (st == 0) K1 = v[0];
