@@ -48,6 +48,7 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "stiff_lu.cuh"
 
 namespace chemgb {
 namespace {
@@ -98,6 +99,7 @@ __device__ __forceinline__ void warp_sum3(double &a, double &b, double &c, int l
 // The warps integrating one cell: W = 1 (a lone warp) or W = kWarps (the block).
 template <int W>
 struct Team {
+    static constexpr int kWarps = W;
     int wt;                    // rank of this warp in the team
     __device__ __forceinline__ void sync() const {
         if (W == 1) __syncwarp();
@@ -741,64 +743,6 @@ struct RowLU {
     }
 };
 
-// In-place LU with partial pivoting in shared memory (n > 32), the reciprocal pivots in invd and the
-// pivot rows in sh.piv; false for a zero or non-finite pivot column. In a team every warp searches the
-// pivot (same data, same choice), the first warp swaps and scales, and the trailing update splits
-// the rows over the warps.
-template <int W, typename real>
-__device__ bool lu_factor(int *piv, real *G, real *invd, Team<W> tm, int lane, int n) {
-    for (int k = 0; k < n; ++k) {
-        real best = -1;
-        int bi = n;
-        for (int s = 0; s < 2; ++s) {
-            const int i = lane + 32 * s;
-            if (i >= k && i < n) {
-                const real v = fabs(G[i * n + k]);
-                if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const real ob = __shfl_xor_sync(kFull, best, o);
-            const int oi = __shfl_xor_sync(kFull, bi, o);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (!(best > 0) || !(best < (real)INFINITY) || bi >= n) return false;
-        if (tm.lead()) {
-            if (lane == 0) piv[k] = bi;
-            if (bi != k) {
-                for (int s = 0; s < 2; ++s) {
-                    const int c = lane + 32 * s;
-                    if (c < n) {
-                        const real t = G[k * n + c];
-                        G[k * n + c] = G[bi * n + c];
-                        G[bi * n + c] = t;
-                    }
-                }
-            }
-        }
-        tm.sync();
-        const real rp = (real)1 / G[k * n + k];
-        if (tm.lead()) {
-            if (lane == 0) invd[k] = rp;
-            for (int s = 0; s < 2; ++s) {
-                const int i = lane + 32 * s;
-                if (i > k && i < n) G[i * n + k] *= rp;
-            }
-        }
-        tm.sync();
-        for (int s = 0; s < 2; ++s) {
-            const int c = lane + 32 * s;
-            if (c > k && c < n) {
-                const real akc = G[k * n + c];
-                for (int i = k + 1 + tm.wt; i < n; i += W) G[i * n + c] -= G[i * n + k] * akc;
-            }
-        }
-        tm.sync();
-    }
-    return true;
-}
-
 // b <- G^-1 b with the factors G, invd in shared memory (n > 32); b is lane-distributed, bsw this
 // warp's own buffer.
 template <typename real>
@@ -854,7 +798,7 @@ struct Factors {
                     for (int c = lane; c < n; c += 32) sh.F[r * n + c] = sh.G[r * n + c];
                 tm.sync();
             }
-            return lu_factor<W, real>(sh.piv, sh.F, sh.invd, tm, lane, n);
+            return lu_factor<Team<W>, real>(sh.piv, sh.F, sh.invd, tm, lane, n);
         } else {
             return lu.factor(sh.G, lane, n);
         }
