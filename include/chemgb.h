@@ -99,6 +99,10 @@ int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech **out);
 int chem_mech_free(chem_mech *mech);
 /* Number of species / reactions of a loaded mechanism (-1 on a null handle). */
 int chem_mech_nspecies(const chem_mech *mech);
+/* Tries of each bounded wait of props_eval's float passes for this mechanism, also
+ * inside chem_step_ann_props (0 = the default, 2^22, seconds in total; a failure-detection
+ * aid as chem_mlp_set_wait_limit). */
+int chem_mech_set_wait_limit(chem_mech *mech, uint32_t tries);
 int chem_mech_nreactions(const chem_mech *mech);
 
 /* ---------------------------------------------------------------------------
@@ -118,9 +122,10 @@ int chem_mech_nreactions(const chem_mech *mech);
  * lambda and Dk together select the transport part). ncells == 0 is a no-op.
  * Every array is 16-byte aligned and ld a multiple of 4 (else CHEM_EINVAL):
  * without transport outputs, in float arithmetic, the state is streamed by
- * 16-byte bulk copies that may read up to 3 cells past ncells (inside ld). If
- * one of those copies never lands (a bounded wait runs out), the affected
- * cells' cp and h are NaN.
+ * 16-byte bulk copies that may read up to 3 cells past ncells (inside ld). The
+ * float passes wait for copies and tensor-core products with a limit. Where
+ * such a wait runs out, the requested outputs of the cells that were not
+ * finished are NaN: no output keeps its old contents.
  */
 int props_eval(const chem_mech *mech, int64_t ncells, int64_t ld, int dtype,
                const void *T, const void *p, const void *Y,

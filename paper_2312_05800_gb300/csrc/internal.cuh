@@ -88,7 +88,7 @@ struct DevMech {
 };
 
 constexpr int kNumCounters = 8;
-constexpr int kPropsErrCounter = 7;       // props_eval's staged thermo pass: a copy wait ran out
+constexpr int kPropsErrCounter = 7;       // props_eval: a pipeline wait ran out (its cells' outputs are NaN)
 
 }  // namespace chemgb
 
@@ -99,6 +99,7 @@ struct chem_mech {
     void *blob;            // single device allocation holding every table
     size_t blob_bytes;
     int device;
+    uint32_t wait_limit;   // tries of each pipeline wait of props_eval (chem_mech_set_wait_limit)
 };
 
 namespace chemgb {

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "tc.cuh"
 
 namespace chemgb {
 
@@ -437,6 +438,7 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     m->blob = blob;
     m->blob_bytes = bb.bytes.size();
     cudaGetDevice(&m->device);
+    m->wait_limit = tc::kSpinLimit;
     uint8_t *base = static_cast<uint8_t *>(blob);
     DevMech &d = m->dev;
     d.N = N; d.R = R; d.Np = Np; d.n_tb = n_tb; d.P_std = th[0]; d.T_mid = th[2];
@@ -504,6 +506,12 @@ extern "C" int chem_mech_free(chem_mech *m) {
 
 extern "C" int chem_mech_nspecies(const chem_mech *m) { return m ? m->N : -1; }
 extern "C" int chem_mech_nreactions(const chem_mech *m) { return m ? m->R : -1; }
+
+extern "C" int chem_mech_set_wait_limit(chem_mech *m, uint32_t tries) {
+    if (!m) return set_error(CHEM_EINVAL, "chem_mech_set_wait_limit: null handle");
+    m->wait_limit = tries == 0 ? tc::kSpinLimit : tries;
+    return CHEM_OK;
+}
 
 extern "C" void chem_ode_opts_default(chem_ode_opts *o) {
     if (!o) return;

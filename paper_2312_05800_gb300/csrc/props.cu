@@ -422,8 +422,8 @@ int launch_props_split(const chem_mech *m, int64_t ncells, int64_t ld, const voi
 // float4 per species and range). The arithmetic and the species order per cell
 // are those of props_kernel's first pass, so cp and h are bitwise the full
 // pass's. A copy wait that runs out (bounded, spin tries) records
-// kPropsErrCounter, writes NaN to the tile's cp and h and stops the CTA after
-// its issued copies have landed.
+// kPropsErrCounter and writes NaN to cp and h of the tile and of every tile the CTA had
+// still to do; the CTA ends after its issued copies have landed.
 constexpr int kThTile = 512;                  // cells per tile = consumer threads
 constexpr int kThRows = 8;                    // state rows per stage
 constexpr int kThThreads = kThTile + 32;      // + the producer warp
@@ -550,9 +550,9 @@ __global__ void __launch_bounds__(kThThreads, 1)
         }
         if (!ok) {
             if (lane == 0) atomicExch(err, 1u);
-            if (i < ncells) {
-                if (cpg) cpg[i] = __int_as_float(0x7fc00000);
-                if (hg) hg[i] = __int_as_float(0x7fc00000);
+            for (int64_t q = i; q < ncells; q += (int64_t)gridDim.x * kThTile) {
+                if (cpg) cpg[q] = __int_as_float(0x7fc00000);
+                if (hg) hg[q] = __int_as_float(0x7fc00000);
             }
             break;
         }
@@ -587,7 +587,7 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
     thermo_kernel<in_t><<<blocks, kThThreads, smem, st>>>(m->N, float(m->T_mid), m->dev.f32, ncells, ld,
                                                           static_cast<const in_t *>(T), static_cast<const in_t *>(Y),
                                                           static_cast<float *>(cp), static_cast<float *>(h),
-                                                          m->dev.counters + kPropsErrCounter, tc::kSpinLimit);
+                                                          m->dev.counters + kPropsErrCounter, m->wait_limit);
     prof_end(pb, st, "thermo_kernel", (double)ncells * 24.0 * m->N,
              (double)ncells * ((m->N + 1) * sizeof(in_t) + 2 * sizeof(float)));
     return check_cuda(cudaGetLastError(), "props_eval (thermo) launch");
@@ -1046,10 +1046,20 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
             if (valid && g.lam) g.lam[i] = lam;
         }
         if (!all_ok) {
-            // a wait ran out: NaN for the tile, and the CTA ends once what it issued has finished
-            if (g.Dk && valid)
-                for (int k = grp; k < N; k += TPR) g.Dk[(int64_t)k * g.ld + i] = __int_as_float(0x7fc00000);
+            // a wait ran out: NaN for the tile's transport and for every output of the tiles the CTA had
+            // still to do, and the CTA ends once what it issued has finished
+            const float nan = __int_as_float(0x7fc00000);
             if (threadIdx.x == 0) atomicExch(g.err, 1u);
+            for (int64_t c = cell; c < g.ncells; c += (int64_t)gridDim.x * 128) {
+                if (g.Dk)
+                    for (int k = grp; k < N; k += TPR) g.Dk[(int64_t)k * g.ld + c] = nan;
+                if (grp == 0 && c != cell) {
+                    if (g.cp) g.cp[c] = nan;
+                    if (g.h) g.h[c] = nan;
+                    if (g.mu) g.mu[c] = nan;
+                    if (g.lam) g.lam[c] = nan;
+                }
+            }
             break;
         }
         if (RED2 == 0) __syncthreads();                                // the sums' rows are written again
@@ -1092,7 +1102,7 @@ int launch_props_tc(const chem_mech *m, int64_t ncells, int64_t ld, const void *
     const int64_t most = (int64_t)sms * L::kCtas;                      // the resident CTAs
     const TcArgs a{m->N, float(m->T_mid), m->dev.f32, m->dev.tc, ncells, ld, static_cast<float *>(cp),
                    static_cast<float *>(h), static_cast<float *>(mu), static_cast<float *>(lam),
-                   static_cast<float *>(Dk), m->dev.counters + kPropsErrCounter, tc::kSpinLimit};
+                   static_cast<float *>(Dk), m->dev.counters + kPropsErrCounter, m->wait_limit};
     void *pb = prof_begin(st);
     props_tc_kernel<in_t, NMAX><<<(unsigned)(ntiles < most ? ntiles : most), L::kThreads, smem, st>>>(
         a, static_cast<const in_t *>(T), static_cast<const in_t *>(p), static_cast<const in_t *>(Y));
