@@ -11,16 +11,11 @@ int launch_fused34_nb(const void *X, int64_t ldx, int K3, const void *W3, int64_
                       int M, int N4, const float *b3, const float *b4, float *u, int64_t ldu, int *err,
                       cudaStream_t st) {
     using L = F34Smem<NA, NB>;
-    static bool configured = false;
-    if (!configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(gemm_fused34_kernel<NA, NB>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::kTotal),
-                            "fused output GEMM smem attribute");
-        if (rc) return rc;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    int rc = dynamic_smem_limit(configured, gemm_fused34_kernel<NA, NB>, L::kTotal, "fused output GEMM smem attribute");
+    if (rc) return rc;
     CUtensorMap tx, t3a, t3b, t4;
-    int rc = make_tmap_operand(&tx, X, M, K3, ldx, kBM, 2);
+    rc = make_tmap_operand(&tx, X, M, K3, ldx, kBM, 2);
     if (!rc) rc = make_tmap_operand(&t3a, W3, NA + NB, K3, ldw3, NA, 2);
     if (!rc) rc = make_tmap_operand(&t3b, W3, NA + NB, K3, ldw3, NB, 2);
     if (!rc) rc = make_tmap_operand(&t4, W4, N4, NA + NB, ldw4, 32, 2);

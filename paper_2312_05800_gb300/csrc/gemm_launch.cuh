@@ -106,13 +106,14 @@ struct WaitLimitScope {
 };
 
 inline int num_sms() {
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    return sms;
+    static DeviceInt sms;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return sms.value(dev, [dev] {
+        int v = 0;
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v;
+    });
 }
 
 // Output tensor map for the TMA-store epilogue: [rows][cols] of BF16 (esize 2)
@@ -184,17 +185,12 @@ template <int BN, int STAGES, class Epi>
 int launch_gemm_grouped_bn(const GemmOperand &A, const GemmOperand &B, int G, int out_kind, int64_t out_gstride, int M,
                            int N, int K, const Epi &epi, int *err, cudaStream_t st, int max_ctas) {
     using L = GemmSmem<BN, STAGES>;
-    static bool configured = false;
-    if (!configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(gemm_tn_kernel<BN, STAGES, Epi>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::kTotal),
-                            "GEMM smem attribute");
-        if (rc) return rc;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    int rc = dynamic_smem_limit(configured, gemm_tn_kernel<BN, STAGES, Epi>, L::kTotal, "GEMM smem attribute");
+    if (rc) return rc;
     const int esize = Epi::kF8 ? 1 : 2;
     CUtensorMap ta, tb, tc, tc1;
-    int rc = make_operand_map(&ta, A, M, K, G, kBM, esize);
+    rc = make_operand_map(&ta, A, M, K, G, kBM, esize);
     if (rc) return rc;
     // N-major B: [K][N], boxes of 64 columns x 64 rows
     rc = Epi::kBNMajor ? make_operand_map(&tb, B, K, N, G, kBK, esize) : make_operand_map(&tb, B, N, K, G, BN, esize);

@@ -162,13 +162,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) gemm_wgrad_kernel(const __grid_
 
 int gemm_wgrad(const WgradLayer *layers, int count, int B, int *err, cudaStream_t st) {
     if (count < 1 || count > kWgMaxLayers || B < 1) return set_error(CHEM_EINVAL, "weight gradients: bad sizes");
-    static bool configured = false;
-    if (!configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(gemm_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)kWgSmem), "weight gradient smem attribute");
-        if (rc) return rc;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    if (int rc = dynamic_smem_limit(configured, gemm_wgrad_kernel, kWgSmem, "weight gradient smem attribute")) return rc;
     WgradArgs a;
     std::memset(&a, 0, sizeof(a));
     a.count = count;

@@ -8,6 +8,7 @@
 #include <string>
 
 #include "chemgb.h"
+#include "device_once.h"
 
 #define CHEMGB_STR2(x) #x
 #define CHEMGB_STR(x) CHEMGB_STR2(x)
@@ -104,11 +105,20 @@ struct chem_mech {
 
 namespace chemgb {
 int set_error(int code, const std::string &msg);
+int check_cuda(cudaError_t e, const char *what);
+// Opts a kernel into `bytes` of dynamic shared memory on the current device, once per device.
+template <class Kernel>
+inline int dynamic_smem_limit(DeviceOnce &once, Kernel *kernel, size_t bytes, const char *what) {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    return once.run(dev, [&] {
+        return check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
+    });
+}
 // opt-in per-kernel timing (chem_prof_enable): events around tagged launches
 bool prof_on();
 void *prof_begin(cudaStream_t st);
 void prof_end(void *begin, cudaStream_t st, const std::string &tag, double flops, double bytes);
-int check_cuda(cudaError_t e, const char *what);
 bool device_ok(std::string *why);
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

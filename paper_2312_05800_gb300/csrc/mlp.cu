@@ -1555,9 +1555,9 @@ int step_ann_impl(const chem_mech *mech, const chem_mlp *m, int64_t ncells, int6
             queued += n;
         }
         void *pb = prof_begin(st);
-        auto epi = [&](auto kernel, size_t smem, int threads) -> int {
-            int r = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                               "chem_step_ann epilogue");
+        static DeviceOnce configured[6];
+        auto epi = [&](int which, auto kernel, size_t most, size_t smem, int threads) -> int {
+            int r = dynamic_smem_limit(configured[which], kernel, most, "chem_step_ann epilogue");
             if (r) return r;
             kernel<<<(unsigned)((n + threads - 1) / threads), threads, smem, st>>>(
                 n, ld, m->out, m->n_out_pad, m->N, m->bath, m->mu_u, m->sd_u, mech->dev.f32, (float)mech->T_mid, T + c0,
@@ -1567,14 +1567,14 @@ int step_ann_impl(const chem_mech *mech, const chem_mlp *m, int64_t ncells, int6
         // blocks of 32 cells while blocks of 128 would leave SMs without one
         const bool few = n < (int64_t)128 * num_sms();
         if (m->N <= 16)
-            rc = few ? epi(epilogue_kernel<16, 32>, EpiLayout<16, 32>::bytes(m->N), 32)
-                     : epi(epilogue_kernel<16, 128>, EpiLayout<16, 128>::bytes(m->N), 128);
+            rc = few ? epi(0, epilogue_kernel<16, 32>, EpiLayout<16, 32>::bytes(16), EpiLayout<16, 32>::bytes(m->N), 32)
+                     : epi(1, epilogue_kernel<16, 128>, EpiLayout<16, 128>::bytes(16), EpiLayout<16, 128>::bytes(m->N), 128);
         else if (m->N <= 32)
-            rc = few ? epi(epilogue_kernel<32, 32>, EpiLayout<32, 32>::bytes(m->N), 32)
-                     : epi(epilogue_kernel<32, 128>, EpiLayout<32, 128>::bytes(m->N), 128);
+            rc = few ? epi(2, epilogue_kernel<32, 32>, EpiLayout<32, 32>::bytes(32), EpiLayout<32, 32>::bytes(m->N), 32)
+                     : epi(3, epilogue_kernel<32, 128>, EpiLayout<32, 128>::bytes(32), EpiLayout<32, 128>::bytes(m->N), 128);
         else
-            rc = few ? epi(epilogue_kernel<64, 32>, EpiLayout<64, 32>::bytes(m->N), 32)
-                     : epi(epilogue_kernel<64, 128>, EpiLayout<64, 128>::bytes(m->N), 128);
+            rc = few ? epi(4, epilogue_kernel<64, 32>, EpiLayout<64, 32>::bytes(64), EpiLayout<64, 32>::bytes(m->N), 32)
+                     : epi(5, epilogue_kernel<64, 128>, EpiLayout<64, 128>::bytes(64), EpiLayout<64, 128>::bytes(m->N), 128);
         prof_end(pb, st, "epilogue_kernel", 0.0, (double)n * (m->N * 16 + 16 + m->n_out_pad * 4));
         if (rc) return rc;
     }

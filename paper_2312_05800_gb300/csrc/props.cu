@@ -570,14 +570,10 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
     if (!aligned16(T) || !aligned16(Y) || (ld & 3) != 0)
         return set_error(CHEM_EINVAL, "props_eval: the state arrays must be 16-byte aligned and ld a multiple of 4");
     const size_t smem = L::bytes(m->N);
-    static bool configured = false;
-    if (!configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(thermo_kernel<in_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)L::bytes(kMaxSpecies)),
-                            "props_eval (thermo) smem attribute");
-        if (rc) return rc;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    if (int rc = dynamic_smem_limit(configured, thermo_kernel<in_t>, L::bytes(kMaxSpecies),
+                                    "props_eval (thermo) smem attribute"))
+        return rc;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1086,15 +1082,10 @@ int launch_props_tc(const chem_mech *m, int64_t ncells, int64_t ld, const void *
                     void *cp, void *h, void *mu, void *lam, void *Dk, cudaStream_t st) {
     using L = TcLayout<NMAX>;
     const size_t smem = L::bytes(m->dev.tc.rows);
-    static bool configured = false;
-    if (!configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(props_tc_kernel<in_t, NMAX>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 NMAX <= 32 ? 113 * 1024 : 227 * 1024),
-                            "props_eval smem attribute");
-        if (rc) return rc;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    if (int rc = dynamic_smem_limit(configured, props_tc_kernel<in_t, NMAX>, NMAX <= 32 ? 113 * 1024 : 227 * 1024,
+                                    "props_eval smem attribute"))
+        return rc;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1118,14 +1109,11 @@ int launch_props(const chem_mech *m, int64_t ncells, int64_t ld, const void *T, 
     const size_t smem = tables_in_smem<real>() ? ((transport ? (size_t)8 * m->N * m->dev.Np : 0) +
                                                   (size_t)kSpeciesFloats * m->N) * sizeof(real)
                                                : 0;
-    static size_t configured = 0;
-    if (smem > configured) {
-        int rc = check_cuda(cudaFuncSetAttribute(props_kernel<real, in_t, NMAX>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPropsSmemMax),
-                            "props_eval smem attribute");
-        if (rc) return rc;
-        configured = kPropsSmemMax;
-    }
+    static DeviceOnce configured;
+    if (smem > 0)
+        if (int rc = dynamic_smem_limit(configured, props_kernel<real, in_t, NMAX>, kPropsSmemMax,
+                                        "props_eval smem attribute"))
+            return rc;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -1235,7 +1235,9 @@ int launch_stiff_nc(const chem_mech *m, int64_t capacity, int64_t ld, double dt,
     if (smem > kSmemMax)
         return set_error(CHEM_EUNSUPPORTED, std::string(who) + ": mechanism too large for shared memory");
     auto kernel = stiff_kernel<NC, MX>;
-    int rc = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), who);
+    // the largest size, once: launches of other mechanisms from other threads find it large enough
+    static DeviceOnce configured;
+    int rc = dynamic_smem_limit(configured, kernel, kSmemMax, who);
     if (rc) return rc;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -1370,8 +1372,8 @@ extern "C" int chem_pasr(const chem_mech *m, int64_t ncells, int64_t ld, double 
     const size_t smem = pasr_slice_bytes(m->N, m->R) * kWarps;
     if (smem > 227 * 1024) return set_error(CHEM_EUNSUPPORTED, "chem_pasr: mechanism too large for shared memory");
     auto kernel = m->N <= 31 ? pasr_kernel<1> : pasr_kernel<2>;
-    int rc = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                        "chem_pasr: smem attribute");
+    static DeviceOnce configured[2];
+    int rc = dynamic_smem_limit(configured[m->N > 31], kernel, 227 * 1024, "chem_pasr: smem attribute");
     if (rc) return rc;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
