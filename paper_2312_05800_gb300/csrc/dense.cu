@@ -26,7 +26,7 @@ extern "C" int chem_dense_bf16(int64_t M, int N, int K, const void *x, int64_t l
         int rc = check_cuda(cudaGetSymbolAddress(reinterpret_cast<void **>(&e), g_dense_err), "chem_dense_bf16");
         if (rc) return rc;
     }
-    int bn = tile_n > 0 ? tile_n : default_tile_width(N);
+    int bn = tile_n > 0 ? tile_n : product_tile_width(M, N, K, act == 1, num_sms());
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (act == 1) return gemm_gelu(bn, x, ldx, W, ldw, (int)M, N, K, b, y, ldy, nullptr, 0, e, st);
     return gemm_linear(bn, x, ldx, W, ldw, (int)M, N, K, b, static_cast<float *>(y), ldy, e, st);

@@ -12,6 +12,7 @@
 
 #include "gemm.cuh"
 #include "internal.cuh"
+#include "tile_width.h"
 
 namespace chemgb {
 
@@ -221,9 +222,6 @@ int launch_gemm_grouped_bn(const GemmOperand &A, const GemmOperand &B, int G, in
     return check_cuda(cudaGetLastError(), "GEMM launch");
 }
 
-// Tile widths the library is built with (the autotuner picks among them).
-constexpr int kTileWidths[] = {32, 64, 128, 160, 208, 256};
-
 // G products in one launch (single-CTA tiles only).
 template <class Epi>
 int launch_gemm_grouped(int bn, const GemmOperand &A, const GemmOperand &B, int G, int out_kind, int64_t out_gstride,
@@ -250,21 +248,6 @@ int launch_gemm(int bn, const void *X, int64_t ldx, const void *W, int64_t ldw, 
     if (M <= 0 || N <= 0 || K <= 0) return CHEM_OK;
     return launch_gemm_grouped(bn, GemmOperand{X, ldx, kMap2D, 0}, GemmOperand{W, ldw, kMap2D, 0}, 1, kMap2D, 0, M, N,
                                K, epi, err, st, max_ctas);
-}
-
-// Default tile width for an output width N: a tile's time is about that of its columns plus 290 (the
-// operands' k-blocks and the tile's own start and end), so the width with the smallest sum over the
-// N tiles. Measured on 262,144 rows (us at 160 / 208 / 256): 800 x 1600 553 / 488 / 502, 1600 x 96 330 / 348 /
-// 310, 400 x 800 201 / 159 / 205, 1024 x 2048 954 / 766 / 671; the fewest padded columns, the rule before, took 160
-// for the first two.
-inline int default_tile_width(int N) {
-    int best = 256;
-    long best_cost = -1;
-    for (int bn : kTileWidths) {
-        const long cost = (long)((N + bn - 1) / bn) * (bn + 290);
-        if (best_cost < 0 || cost < best_cost) { best = bn; best_cost = cost; }
-    }
-    return best;
 }
 
 // Forward declarations of the per-epilogue launchers (one translation unit each).
