@@ -4,7 +4,9 @@
 //
 // Three kernels: thermo_kernel (cp and h alone), props_tc_kernel (the full pass
 // in FP32, species-pair sums on the tensor cores), and the pair loop below for
-// FP64 and for what the tensor-core pass does not take (more than 56 species).
+// FP64 and for what the tensor-core pass does not take (more than 56 species, or tables
+// that FP16 pairs do not hold: 524,288 cells of 9 / 30 species 69 / 389 us in FP32 with the
+// instances for 16 and 32 species, 188 / 664 us with the one for 64).
 //
 // The pair loop: one thread per cell, persistent grid-stride loop. Cell data are SoA, so a
 // warp's loads of T, p and each Y_k row are 128-byte coalesced. The per-pair
@@ -98,7 +100,7 @@ __device__ __forceinline__ bool pure_species(real Xk, real y, real ds, real gs, 
 }
 
 template <typename real, typename in_t, int NMAX>
-__global__ void __launch_bounds__(128) props_kernel(int N, int Np, real T_mid, PropTables<real> tb, int64_t ncells,
+__global__ void __launch_bounds__(128, sizeof(real) == 4 && NMAX <= 32 ? 4 : 1) props_kernel(int N, int Np, real T_mid, PropTables<real> tb, int64_t ncells,
                                                     int64_t ld, const in_t *__restrict__ Tg,
                                                     const in_t *__restrict__ pg, const in_t *__restrict__ Yg,
                                                     real *__restrict__ cpg, real *__restrict__ hg,
@@ -1161,9 +1163,9 @@ int dispatch_props(const chem_mech *m, int64_t ncells, int64_t ld, const void *T
                 return launch_props_split<16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
             return launch_props_split<32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
         }
-        if (m->N <= 16) return launch_props<real, in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
-        if (m->N <= 32) return launch_props<real, in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
     }
+    if (m->N <= 16) return launch_props<real, in_t, 16>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
+    if (m->N <= 32) return launch_props<real, in_t, 32>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
     return launch_props<real, in_t, 64>(m, ncells, ld, T, p, Y, cp, h, mu, lam, Dk, st);
 }
 
