@@ -606,7 +606,8 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
 // vector entry is then at most 1 in magnitude and scaled by 2^14, and the tables' rows by powers of
 // two (PropTcTables). What is left of absolute error, 2^-39 of a mole fraction, only shows in D_k of
 // a species that is nearly alone (its sum runs over traces): for X_k > 0.999 that sum is taken in FP32
-// from the FP32 tables (near_pure_D). The tensor core cuts its accumulator instead of rounding it,
+// from the FP32 tables (near_pure_D), and a cell with |X_k| >= 4 (mass fractions of both signs), past FP16's
+// range, is redone in FP32 as a whole (wide_cell). The tensor core cuts its accumulator instead of rounding it,
 // which takes a mean share of a sum that grows with the instructions of full size (K / 16): measured
 // 0.5e-7, 2.8e-7 and 5.7e-7 for 1, 2 and 4, and given back (`cut`). r_k = 2^(polynomial) is formed with
 // the whole part of its exponent taken out at load time. Relative errors against 64 bits (2-norm, 100,003
@@ -693,6 +694,61 @@ __device__ __noinline__ float near_pure_D(const PropTables<float> &tb, int N, in
     return (1.0f - y) * T15 / (p * ds);
 }
 
+// Transport of cell i where the tensor-core sums are not finite although the state is: mole fractions that FP16 does
+// not hold (|X_k| >= 4, from mass fractions of both signs). The pair loop's sums in FP32, by one thread.
+template <typename in_t>
+__device__ __forceinline__ void wide_cell(const TcArgs &g, const in_t *__restrict__ Tg, const in_t *__restrict__ pg,
+                                       const in_t *__restrict__ Yg, int64_t i) {
+    const PropTables<float> &tb = g.tb;
+    const int N = g.N, Np = (N + 3) & ~3;
+    const int64_t ld = g.ld;
+    const float out = g.mu ? g.mu[i] : (g.lam ? g.lam[i] : g.Dk[i]);
+    if (fabsf(out) < INFINITY) return;
+    const float T = to_real<float>(Tg[i]), p = to_real<float>(pg[i]), x = logf(T * 1e-3f);
+    float S = 0.0f;
+    for (int k = 0; k < N; ++k) S = fmaf(to_real<float>(Yg[(int64_t)k * ld + i]), __ldg(tb.invW + k), S);
+    if (!(fabsf(S) < INFINITY && fabsf(x) < INFINITY)) return;
+    const float Wbar = 1.0f / S;
+    const int rng = (T >= g.T_mid) ? 1 : 0;
+    float *mug = g.mu, *lamg = g.lam, *Dkg = g.Dk;
+    const float T15 = T * sqrtf(T), R = float(kR);
+    auto log_mu = [&](int k) {
+        const float *c = tb.visc + k * 5;
+        return fmaf(fmaf(fmaf(fmaf(__ldg(c + 4), x, __ldg(c + 3)), x, __ldg(c + 2)), x, __ldg(c + 1)), x, __ldg(c));
+    };
+    float mu = 0.0f, lam = 0.0f;
+    for (int k = 0; k < N; ++k) {
+        const float y = to_real<float>(Yg[(int64_t)k * ld + i]), iw = __ldg(tb.invW + k), Xk = y * iw * Wbar;
+        const float muk = expf(log_mu(k)), rk = sqrtf(muk);
+        const float *a = tb.nasa_cp + (rng * N + k) * 5;
+        const float cpR = fmaf(fmaf(fmaf(fmaf(__ldg(a + 4), T, __ldg(a + 3)), T, __ldg(a + 2)), T, __ldg(a + 1)), T, __ldg(a));
+        float den = 0.0f, ds = 0.0f, gs = 0.0f;
+        for (int j = 0; j < N; ++j) {
+            const float Xj = to_real<float>(Yg[(int64_t)j * ld + i]) * __ldg(tb.invW + j) * Wbar;
+            const float t = expf(-0.5f * log_mu(j)) * rk;
+            const float *w = tb.wilke + (size_t)k * Np + j, *d = tb.diff + (size_t)k * Np + j;
+            const size_t st = (size_t)N * Np;
+            den = fmaf(fmaf(t, fmaf(t, __ldg(w + 2 * st), __ldg(w + st)), __ldg(w)), Xj, den);
+            float g = 0.0f;
+            for (int n = 4; n >= 0; --n) g = fmaf(g, x, __ldg(d + n * st));
+            ds = fmaf(g, Xj, ds);
+            gs += g;
+        }
+        mu = fmaf(Xk, muk / den, mu);
+        lam = fmaf(Xk, muk * (cpR + 1.25f) * R * iw / den, lam);      // Eucken
+        if (Dkg)
+            Dkg[(int64_t)k * ld + i] = pure_species(Xk, y, ds, gs, N) ? T15 / (p * gs / float(N - 1)) : (1.0f - y) * T15 / (p * ds);
+    }
+    if (mug) mug[i] = mu;
+    if (lamg) lamg[i] = lam;
+}
+template <typename in_t>
+__device__ __noinline__ void wide_cells(const TcArgs *g, const in_t *Tg, const in_t *pg, const in_t *Yg) {
+    if (threadIdx.x >= 128) return;
+    for (int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x; i < g->ncells; i += (int64_t)gridDim.x * 128)
+        wide_cell(*g, Tg, pg, Yg, i);
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -728,7 +784,7 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_plain(uint32_t saddr, uint32_t 
 
 template <typename in_t, int NMAX>
 __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCtas)
-    props_tc_kernel(TcArgs g, const in_t *__restrict__ Tg, const in_t *__restrict__ pg, const in_t *__restrict__ Yg) {
+    props_tc_kernel(const __grid_constant__ TcArgs g, const in_t *__restrict__ Tg, const in_t *__restrict__ pg, const in_t *__restrict__ Yg) {
     using L = TcLayout<NMAX>;
     constexpr int TPR = L::kTPR, SH = L::kShares;
     extern __shared__ __align__(128) uint8_t tc_smem[];
@@ -749,6 +805,7 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
     uint64_t *bars = reinterpret_cast<uint64_t *>(red + L::kRedRows * SH * 128);
     uint64_t *bar_b = bars, *bar_m = bars + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2);
+    volatile uint32_t *wide = tmem_slot + 1;                           // 1: some cell's sums are not finite; 2: a wait ran out
     const int warp = threadIdx.x >> 5;
     const int grp = warp >> 2;                                         // which share of the species
     const int row = threadIdx.x & 127;                                 // cell of the tile = TMEM lane
@@ -758,6 +815,7 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
         tc::mbar_init(bar_b, 1);
         tc::mbar_init(bar_m, 1);
         tc::fence_barrier_init();
+        *wide = 0;
         tc::mbar_arrive_expect_tx(bar_b, 2 * b_term);
         for (uint32_t o = 0; o < 2 * b_term; o += 16384) {
             const uint32_t n = 2 * b_term - o < 16384 ? 2 * b_term - o : 16384;
@@ -1030,7 +1088,9 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
             red[(RED2 + SH + grp) * 128 + row] = lam * unit;
         }
         tc::tc_fence_before();                                         // TMEM reads before the next tile's products
-        const bool all_ok = __syncthreads_and(ok);
+        const bool fin = __syncthreads_and(ok && fabsf(mu) < INFINITY);
+        const bool all_ok = fin || __syncthreads_and(ok);
+        if (!fin && threadIdx.x == 0) *wide = 1;
         if (grp == 0) {
             mu = 0.0f;
             lam = 0.0f;
@@ -1047,7 +1107,10 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
             // a wait ran out: NaN for the tile's transport and for every output of the tiles the CTA had
             // still to do, and the CTA ends once what it issued has finished
             const float nan = __int_as_float(0x7fc00000);
-            if (threadIdx.x == 0) atomicExch(g.err, 1u);
+            if (threadIdx.x == 0) {
+                atomicExch(g.err, 1u);
+                *wide = 2;
+            }
             for (int64_t c = cell; c < g.ncells; c += (int64_t)gridDim.x * 128) {
                 if (g.Dk)
                     for (int k = grp; k < N; k += TPR) g.Dk[(int64_t)k * g.ld + c] = nan;
@@ -1062,6 +1125,11 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
         }
         if (RED2 == 0) __syncthreads();                                // the sums' rows are written again
     }
+    // An entry past FP16's range (|X_k| >= 4) has made every sum of its cell NaN: such cells, found by their own
+    // output, are redone here, out of the loop above, whose registers a call would spill. (A state that is itself
+    // not finite stays as it is.)
+    __syncthreads();
+    if (*wide == 1) wide_cells(&g, Tg, pg, Yg);
     if (threadIdx.x == 0) {
         // nothing in flight when the CTA ends (full limit): the table copy, then the products
         if (!b_ready && !tc::mbar_wait(bar_b, 0)) atomicExch(g.err, 1u);
