@@ -101,8 +101,9 @@ int chem_mech_free(chem_mech *mech);
 int chem_mech_nspecies(const chem_mech *mech);
 /* Tries of each bounded wait of props_eval's float passes for this mechanism, also
  * inside chem_step_ann_props (0 = the default, 2^22, seconds in total; a failure-detection
- * aid as chem_mlp_set_wait_limit). */
-int chem_mech_set_wait_limit(chem_mech *mech, uint32_t tries);
+ * aid as chem_mlp_set_wait_limit). Negative: no try at all, every such wait counts as run out
+ * (a single try may suspend the thread until its phase ends). */
+int chem_mech_set_wait_limit(chem_mech *mech, int32_t tries);
 int chem_mech_nreactions(const chem_mech *mech);
 
 /* ---------------------------------------------------------------------------

@@ -70,7 +70,7 @@ def lib() -> ctypes.CDLL:
     L.chem_mech_load_bytes.argtypes = [vp, ctypes.c_size_t, ctypes.POINTER(vp)]
     L.chem_mech_free.argtypes = [vp]
     L.chem_mech_nspecies.argtypes = [vp]
-    L.chem_mech_set_wait_limit.argtypes = [vp, ctypes.c_uint32]
+    L.chem_mech_set_wait_limit.argtypes = [vp, ctypes.c_int32]
     L.chem_mech_nreactions.argtypes = [vp]
     L.props_eval.argtypes = [vp, i64, i64, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp]
     L.chem_ode_opts_default.argtypes = [ctypes.POINTER(chem_ode_opts)]

@@ -507,9 +507,9 @@ extern "C" int chem_mech_free(chem_mech *m) {
 extern "C" int chem_mech_nspecies(const chem_mech *m) { return m ? m->N : -1; }
 extern "C" int chem_mech_nreactions(const chem_mech *m) { return m ? m->R : -1; }
 
-extern "C" int chem_mech_set_wait_limit(chem_mech *m, uint32_t tries) {
+extern "C" int chem_mech_set_wait_limit(chem_mech *m, int32_t tries) {
     if (!m) return set_error(CHEM_EINVAL, "chem_mech_set_wait_limit: null handle");
-    m->wait_limit = tries == 0 ? tc::kSpinLimit : tries;
+    m->wait_limit = tries == 0 ? tc::kSpinLimit : (tries < 0 ? 0u : (uint32_t)tries);
     return CHEM_OK;
 }
 
