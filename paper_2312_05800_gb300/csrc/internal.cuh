@@ -75,7 +75,7 @@ struct DevMech {
     int nslot;              // distinct species of a reaction, at most (row length of d q / d C)
     int three;              // some reaction has a third reactant or product
     int gath_len;           // longest species incidence list, rounded up to 4
-    const unsigned *gath;   // [gath_len][64] code: nu (FP64), reaction; 0 pads
+    const unsigned *gath;   // [gath_len][64] code: nu (FP64), reaction; pads: 0, R
     int ell_groups;         // groups of 32 entries of the sparse part of d wdot / d C, longest first
     const int *ell_off, *ell_len, *ell_pos;   // [groups] first word, iterations; [groups][32] matrix offset or -1
     const unsigned *ell_f, *ell_d;            // code: nu (FP32 / FP64), index in d q / d C [R][nslot]; 0 pads

@@ -363,7 +363,7 @@ extern "C" int chem_mech_load_bytes(const void *data, size_t nbytes, chem_mech *
     tbrow_ptr[N] = (int)tbrow_f.size();
     if (tbrow_f.empty()) { tbrow_f.push_back(0u); tbrow_d.push_back(0u); }
     const int gath_len = (int)((longest + 3) & ~size_t(3));
-    std::vector<unsigned> gath((size_t)gath_len * 64, 0u);
+    std::vector<unsigned> gath((size_t)gath_len * 64, (unsigned)R);      // pads: the absent reaction, rate 0
     for (int k = 0; k < N; ++k)
         for (size_t t = 0; t < inc[k].size(); ++t) gath[t * 64 + k] = inc[k][t];
     // entries (row, column) of the sparse part of d wdot / d C: their reactions ascending, entries

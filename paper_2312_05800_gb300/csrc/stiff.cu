@@ -110,12 +110,13 @@ struct Team {
 
 // One warp's shared-memory slice. mreal is the type of the matrix and of what only the matrix reads:
 // FP32 in the mixed mode (values cut from FP64 once, when they are stored). BIG (n > 32): the LU
-// factors live in shared memory too. Absent species have index N: C = 1, g = H = 0.
+// factors live in shared memory too. Absent species have index N: C = 1, g = H = 0; the absent reaction
+// has index R: rq = rdqT = 0.
 template <bool MX>
 struct Slice {
     using mreal = typename std::conditional<MX, float, double>::type;
     double *C, *g, *H;             // [N+1] concentration, S/R - H/RT, H/RT
-    double *rq, *rdqT;             // [R] rate of progress, its derivative to T
+    double *rq, *rdqT;             // [R+1] rate of progress, its derivative to T
     double *xs;                    // [n] this warp's own vector buffer
     mreal *G;                      // [n][n] I/(h g) - J
     mreal *F, *invd;               // [n][n], [n] LU factors, reciprocal pivots (BIG)
@@ -143,12 +144,12 @@ __host__ __device__ inline size_t make_slice(char *base, int N, int R, int n_tb,
     t.g = reinterpret_cast<double *>(take((size_t)(N + 1) * 8));
     t.H = reinterpret_cast<double *>(take((size_t)(N + 1) * 8));
     t.xs = reinterpret_cast<double *>(take((size_t)n * 8));
-    const size_t g_bytes = (size_t)n * n * sizeof(mreal), q_bytes = (size_t)R * 8;
+    const size_t g_bytes = (size_t)n * n * sizeof(mreal), q_bytes = (size_t)(R + 1) * 8;
     if (!MX && !BIG) {
         char *p = take(g_bytes > 2 * q_bytes ? g_bytes : 2 * q_bytes);
         t.G = reinterpret_cast<mreal *>(p);
         t.rq = reinterpret_cast<double *>(p);
-        t.rdqT = t.rq + R;
+        t.rdqT = t.rq + R + 1;
     } else {
         t.rq = reinterpret_cast<double *>(take(q_bytes));
         t.rdqT = reinterpret_cast<double *>(take(q_bytes));
@@ -310,10 +311,12 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
                 if (MX) sh.Cf[c - 1] = f64_to_f32_trunc(C);
             }
         }
-        if (lane == 0) {                             // the absent species
+        if (lane == 0) {                             // the absent species, the absent reaction
             sh.C[N] = 1.0;
             sh.g[N] = 0.0;
             sh.H[N] = 0.0;
+            sh.rq[R] = 0.0;
+            if (JAC) sh.rdqT[R] = 0.0;
         }
     }
     tm.sync();
@@ -437,7 +440,8 @@ __device__ __forceinline__ EvalInfo eval_rhs(const DevMech &m, const Slice<MX> &
         }
     }
     tm.sync();
-    // species gather: wdot_k = sum_j nu_kj q_j (reactions ascending)
+    // species gather: wdot_k = sum_j nu_kj q_j (reactions ascending). Lists are padded with the absent reaction: a rate
+    // that is not finite reaches its own species only
     double w[NS], wt[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
@@ -1290,7 +1294,7 @@ int launch_stiff(const chem_mech *m, int64_t capacity, int64_t ld, double dt, co
 // (the slowest formation rate), +inf when none qualifies; tau_mix = sqrt(tau_T tau_K);
 // kappa = tau_c / (tau_c + tau_mix), 1 for an infinite tau_c. With T, Y given (the chemistry
 // step's result), they become T0 + kappa (T - T0), Y0 + kappa (Y - Y0).
-__host__ __device__ inline size_t pasr_slice_bytes(int N, int R) { return (size_t)(3 * (N + 1) + R) * 8; }
+__host__ __device__ inline size_t pasr_slice_bytes(int N, int R) { return (size_t)(3 * (N + 1) + R + 1) * 8; }
 template <int NS>
 __global__ void __launch_bounds__(kWarps * 32) pasr_kernel(const __grid_constant__ DevMech m, int64_t ncells,
                                                             int64_t ld, double y_min, const double *__restrict__ T0,
