@@ -607,9 +607,18 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
 // two (PropTcTables). What is left of absolute error, 2^-39 of a mole fraction, only shows in D_k of
 // a species that is nearly alone (its sum runs over traces): for X_k > 0.999 that sum is taken in FP32
 // from the FP32 tables (near_pure_D), and a cell with |X_k| >= 4 (mass fractions of both signs), past FP16's
-// range, is redone in FP32 as a whole (wide_cell). The tensor core cuts its accumulator instead of rounding it,
-// which takes a mean share of a sum that grows with the instructions of full size (K / 16): measured
-// 0.5e-7, 2.8e-7 and 5.7e-7 for 1, 2 and 4, and given back (`cut`). r_k = 2^(polynomial) is formed with
+// range, is redone in FP32 as a whole (wide_cell). The tensor core cuts its accumulator instead of rounding it:
+// a sum loses 0.4e-7 of itself (0.6e-7 as mu and lambda show it) in the instruction that takes a species in and
+// 1.8 to 2.4e-7 in each K step after that, so how much depends on where in the species' order a cell has its
+// moles. The mean is given back per cell (`cut`), with the mole fraction of each K step as its share of every sum.
+// Mean signed errors of mu / D without it, with one constant per step count, and so (60,000 cells, FP32 state):
+//   30 species, premixed profiles              2.8e-7 / 2.7e-7    0.1e-7 /  0.0e-7    0.1e-7 /  0.0e-7
+//   53 species, premixed profiles              5.8e-7 / 5.6e-7    0.4e-7 /  0.0e-7    0.0e-7 /  0.0e-7
+//   53 species, X spread by a Dirichlet law    2.8e-7 / 2.5e-7   -2.6e-7 / -3.1e-7   -1.7e-7 / -1.7e-7
+//   53 species, three quarters of Y the last   1.3e-7 / 1.1e-7   -4.0e-7 / -4.5e-7   -0.6e-7 / -0.6e-7
+//   40 species (3 steps), same of the first    3.7e-7 / 3.3e-7   -0.5e-7 / -0.9e-7   -0.5e-7 / -0.7e-7
+//   9 species, Dirichlet law                   0.8e-7 / 0.5e-7   -0.1e-7 /  0.1e-7   -0.1e-7 /  0.1e-7
+// (The resistance polynomials' sums have both signs, and lose the same within 0.5e-7.) r_k = 2^(polynomial) is formed with
 // the whole part of its exponent taken out at load time. Relative errors against 64 bits (2-norm, 100,003
 // cells, FP32 state; the former pair loop -> this kernel): 30 species mu 3.6e-7 -> 1.2e-7, lambda 3.2e-7 ->
 // 1.1e-7, D 2.0e-7 -> 1.6e-7; 53 species 3.2e-7 -> 1.4e-7, 3.1e-7 -> 1.3e-7, 2.4e-7 -> 1.8e-7; 9 species
@@ -827,9 +836,10 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
         tc::tmem_relinquish();
     }
     const float R = float(kR);
-    // the mean share that the cuts of the hi hi instructions take off a sum (measured, below)
-    const int ks16 = (N + 15) / 16;
-    const float cut = ks16 == 1 ? 4e-8f : (ks16 == 2 ? 2.7e-7f : (ks16 == 3 ? 4.2e-7f : 5.6e-7f));
+    const int ks16 = (N + 15) / 16;                                    // K steps: 16 species each
+    // the accumulator's cuts (above): of a K step after a species', for 2, 3 and 4 steps; `later` counts up to NMAX / 16
+    const float per_step = NMAX <= 32 ? 2.37e-7f : (ks16 == 3 ? 2.0e-7f : 1.76e-7f);
+    const float first = NMAX <= 32 ? 4e-8f : (ks16 == 3 ? 4e-8f - 2.0e-7f : 4e-8f);
     for (int e = threadIdx.x; e < 2 * PAD; e += blockDim.x) {
         const int rg = e / PAD, k = e % PAD;
         float a[5] = {0, 0, 0, 0, 0}, b[6] = {0, 0, 0, 0, 0, 0}, iw = 0.0f;
@@ -910,12 +920,16 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
         __syncthreads();
         S = 0.0f;
         rmin = 3.0e38f;
+        float later = 0.0f;                                            // shares of S times the K steps that may follow theirs
 #pragma unroll
         for (int q = 0; q < SH; ++q) {
-            S += red[q * 128 + row];
+            const float Sq = red[q * 128 + row];
+            S += Sq;
+            if (NMAX / 16 - 1 - q / 2 > 0) later = fmaf(Sq, (float)(NMAX / 16 - 1 - q / 2), later);
             rmin = fminf(rmin, red[(SH + q) * 128 + row]);
         }
         const float Wbar = 1.0f / S;
+        const float cut = NMAX <= 16 ? 4e-8f : fmaf(per_step * later, Wbar, first);
         // r is scaled by a power of two that brings the smallest one to 1 .. 2, and 1/r by its reciprocal
         int e = 127 - (int)(__float_as_uint(rmin) >> 23);
         e = e < -100 ? -100 : (e > 100 ? 100 : e);
@@ -1082,7 +1096,7 @@ __global__ void __launch_bounds__(TcLayout<NMAX>::kThreads, TcLayout<NMAX>::kCta
                                                               yw * Wbar, T15, p);
             }
         }
-        const float unit = Wbar * (kTcXScale * kTcWilkeScale) * (1.0f - cut);
+        const float unit = Wbar * (kTcXScale * kTcWilkeScale) * (1.0f - (cut + 2e-8f));
         if (SH == TPR || grp < SH) {
             red[(RED2 + grp) * 128 + row] = mu * unit;
             red[(RED2 + SH + grp) * 128 + row] = lam * unit;
