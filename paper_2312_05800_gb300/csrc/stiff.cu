@@ -120,7 +120,7 @@ struct Slice {
     double *xs;                    // [n] this warp's own vector buffer
     mreal *G;                      // [n][n] I/(h g) - J
     mreal *F, *invd;               // [n][n], [n] LU factors, reciprocal pivots (BIG)
-    mreal *cpR, *wdot, *wT, *JCC, *U, *V, *HR;   // [N]
+    mreal *cpR, *wdot, *wT, *JCC, *U, *V, *HR;   // [N] (wT [n])
     mreal *rc3, *rdq;              // [n_tb] third-body coefficient, [R][nslot] d q / d C of its species
     float *Cf;                     // [N] concentrations in FP32 (mixed mode)
     int *piv;                      // [n] (BIG)
@@ -128,7 +128,9 @@ struct Slice {
 
 // Lays the slice out from `base` (null: only counts) and returns its bytes. Overlaps: in FP64 up to n = 32
 // the matrix (dead once its rows are in registers) shares its space with rq and rdqT (dead when it
-// is built); BIG mixed factors share theirs with rdq (dead when the matrix is built).
+// is built); BIG mixed factors share theirs with rdq (dead when the matrix is built), and BIG pivots and
+// reciprocal pivots with wT and rc3 (likewise), without which a mechanism of third-body reactions with six species
+// each took more than the layout before.
 template <bool MX, bool BIG>
 __host__ __device__ inline size_t make_slice(char *base, int N, int R, int n_tb, int nslot, Slice<MX> *s) {
     using mreal = typename Slice<MX>::mreal;
@@ -163,12 +165,12 @@ __host__ __device__ inline size_t make_slice(char *base, int N, int R, int n_tb,
         t.rdq = reinterpret_cast<mreal *>(take(d_bytes));
         t.F = t.G;
     }
-    t.invd = BIG ? reinterpret_cast<mreal *>(take((size_t)n * sizeof(mreal))) : nullptr;
     mreal **small[] = {&t.cpR, &t.wdot, &t.wT, &t.JCC, &t.U, &t.V, &t.HR};
-    for (mreal **q : small) *q = reinterpret_cast<mreal *>(take((size_t)N * sizeof(mreal)));
-    t.rc3 = reinterpret_cast<mreal *>(take((size_t)n_tb * sizeof(mreal)));
+    for (mreal **q : small) *q = reinterpret_cast<mreal *>(take((size_t)(q == &t.wT ? n : N) * sizeof(mreal)));
+    t.rc3 = reinterpret_cast<mreal *>(take((size_t)(BIG && n > n_tb ? n : n_tb) * sizeof(mreal)));
+    t.invd = BIG ? t.rc3 : nullptr;
     t.Cf = MX ? reinterpret_cast<float *>(take((size_t)N * 4)) : nullptr;
-    t.piv = BIG ? reinterpret_cast<int *>(take((size_t)n * 4)) : nullptr;
+    t.piv = BIG ? reinterpret_cast<int *>(t.wT) : nullptr;
     if (s) *s = t;
     return (o + 15) & ~size_t(15);
 }
