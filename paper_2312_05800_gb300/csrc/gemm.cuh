@@ -84,12 +84,6 @@ struct GemmSmem {
     static_assert(kBBytes % 1024 == 0, "B tile must keep 1024-byte alignment");
 };
 
-__device__ __forceinline__ float ex2_approx(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // ---- GELU (Sec. 3.2) ---------------------------------------------------------
 // GELU(z) = z Phi(z) = h + |h| erf(sqrt(2) |h|) with h = z / 2. For a >= 0,
 // erf(a) = 1 - erfcx(a) exp(-a^2), erfcx(a) = exp(a^2) erfc(a) (smooth, from 1 at 0

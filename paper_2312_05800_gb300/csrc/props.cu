@@ -758,11 +758,6 @@ __device__ __noinline__ void wide_cells(const TcArgs *g, const in_t *Tg, const i
         wide_cell(*g, Tg, pg, Yg, i);
 }
 
-__device__ __forceinline__ float ex2_approx(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

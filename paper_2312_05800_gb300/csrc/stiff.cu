@@ -40,7 +40,8 @@
 //    method of order 3(2), in the transformed form
 //      (I/(h g) - J) K_i = f(y + sum_j a_ij K_j) + sum_j (c_ij / h) K_j,
 //    y_new = y + sum_i m_i K_i, error estimate sum_i e_i K_i, with the
-//    step-size controller of chem_ode_opts. Everything is FP64.
+//    step-size controller of chem_ode_opts. The FP64 mode is FP64 throughout; the mixed mode takes
+//    the rate constants' exponentials, the fall-off blending and the linear algebra in FP32.
 #include <math_constants.h>
 
 #include <cmath>
