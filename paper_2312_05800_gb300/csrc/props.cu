@@ -613,7 +613,7 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
 // moles. The mean is given back per cell (`cut`), with the mole fraction of each K step as its share of every sum.
 // Mean signed errors of mu / D without it, with one constant per step count, and so (60,000 cells, FP32 state):
 //   30 species, premixed profiles              2.8e-7 / 2.7e-7    0.1e-7 /  0.0e-7    0.1e-7 /  0.0e-7
-//   53 species, premixed profiles              5.8e-7 / 5.6e-7    0.4e-7 /  0.0e-7    0.0e-7 /  0.0e-7
+//   53 species, premixed profiles              5.8e-7 / 5.6e-7    0.4e-7 /  0.0e-7   -0.2e-7 /  0.0e-7
 //   53 species, X spread by a Dirichlet law    2.8e-7 / 2.5e-7   -2.6e-7 / -3.1e-7   -1.7e-7 / -1.7e-7
 //   53 species, three quarters of Y the last   1.3e-7 / 1.1e-7   -4.0e-7 / -4.5e-7   -0.6e-7 / -0.6e-7
 //   40 species (3 steps), same of the first    3.7e-7 / 3.3e-7   -0.5e-7 / -0.9e-7   -0.5e-7 / -0.7e-7
@@ -621,13 +621,13 @@ int launch_thermo(const chem_mech *m, int64_t ncells, int64_t ld, const void *T,
 // (The resistance polynomials' sums have both signs, and lose the same within 0.5e-7.) r_k = 2^(polynomial) is formed with
 // the whole part of its exponent taken out at load time. Relative errors against 64 bits (2-norm, 100,003
 // cells, FP32 state; the former pair loop -> this kernel): 30 species mu 3.6e-7 -> 1.2e-7, lambda 3.2e-7 ->
-// 1.1e-7, D 2.0e-7 -> 1.6e-7; 53 species 3.2e-7 -> 1.4e-7, 3.1e-7 -> 1.3e-7, 2.4e-7 -> 1.8e-7; 9 species
+// 1.1e-7, D 2.0e-7 -> 1.6e-7; 53 species 3.2e-7 -> 1.3e-7, 3.1e-7 -> 1.2e-7, 2.4e-7 -> 1.8e-7; 9 species
 // 2.4e-7 -> 0.9e-7, 2.7e-7 -> 1.0e-7, 1.1e-7 -> 1.1e-7.
 //
 // What bounds it: instruction issue (51 % of the slots) and its latencies for the per-species FP32
 // work that is left; the tensor cores are busy a few per cent of the time, HBM 10 %. The pair loop (10
 // instructions a pair, tables from shared memory) took 1,580 us on 2,097,152 cells of 30 species from
-// FP64 state and 799 us on 300,001 of 53 from FP32; this kernel takes 625 and 192 us.
+// FP64 state and 799 us on 300,001 of 53 from FP32; this kernel takes 629 and 188 us.
 //
 // Layout: a thread per cell and chunk of eight species (2, 4 or 8 threads a cell for up to 16, 32 or
 // 56 species: 256 to 1,024 threads, 64 registers; two threads a cell with twice the species each
